@@ -168,8 +168,9 @@ enum {
     CHHS_K_RESTRICT = 1,    /* residual + restriction to the next level; units: fine cells */
     CHHS_K_COARSE_RHS = 2,  /* FAS coarse right-hand side; units: coarse cells */
     CHHS_K_PROLONG = 3,     /* prolongation + correction; units: fine cells */
-    CHHS_K_COARSEST = 4,    /* the one-block tail: the bottom levels of a V-cycle and the
-                               coarsest-grid solve; units: 1 per launch */
+    CHHS_K_COARSEST = 4,    /* the one-launch coarse levels: the one-block tail (the bottom levels
+                               of a V-cycle and the coarsest-grid solve) or the block cluster that
+                               holds the levels above it as well; units: 1 per launch */
     CHHS_K_NORM = 5,        /* stopping norm on the finest grid; units: cells */
     CHHS_K_FRAME = 6,       /* setup, coefficient restriction, mean of p, accept, and the
                                mixed form's double-precision update; units: launches */
@@ -231,7 +232,8 @@ chhs_status chhs_probe_l2(size_t bytes, int passes, double* gbs_out);
 typedef struct {
   int tail_cells;     /* levels with at most this many cells run in the one-block tail */
   int split_threads;  /* double-precision levels with at most this many cells per colour
-                         use the three-warp split update (0: never) */
+                         use the three-warp split update (0: never); unless 0, 2D levels of at
+                         most 4096 cells run in one launch of a block cluster */
   int tile_threads;   /* threads per tile on the 2D mixed form's levels of at least 512 x 256 cells */
   int coarse_nu1;     /* pre- and post-smoothing sweeps on the levels below the finest (the finest */
   int coarse_nu2;     /* keeps opts->nu1, nu2) */

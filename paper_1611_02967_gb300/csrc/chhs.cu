@@ -26,6 +26,7 @@
 
 #include "../../include/chhs.h"
 #include "chhs_kernels.cuh"
+#include "chhs_cluster.cuh"
 #include "chhs_tile.cuh"
 #include "chhs_corr3.cuh"
 #include "chhs_norm_df.cuh"
@@ -198,6 +199,9 @@ struct chhs {
   std::vector<Level<double>> lev;   // double precision: all levels, or the finest only when mixed
   std::vector<Level<float>> lev32;  // single-precision correction hierarchy (mixed precision)
   int tail_start = 0;               // first level run by the one-block tail kernel
+  int cluster_start = -1;           // double precision: first level run by k_cluster with the tail, -1 without it
+  Tail<double> cluster{};           // its levels, cluster_start to the coarsest
+  ClusterPlan cplan{};
   // launch shapes (defaults above; chhs_autotune may change them): levels of at
   // most tail_cells cells go to the tail, double-precision levels of at most
   // split_threads threads per colour pass use the split update, tiles run
@@ -297,6 +301,26 @@ void pdl_grid(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaS
   cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// One cluster of `blocks` blocks.
+template <typename... KArgs, typename... Args>
+cudaError_t pdl_cluster(void (*kernel)(KArgs...), int blocks, int block, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)blocks;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <typename... KArgs, typename... Args>
 void pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
   pdl_smem(kernel, grid, block, 0, s, args...);
@@ -354,6 +378,15 @@ struct Enqueue {
                      int l) {
     const Coefs<T> K = coefs<T>(run);
     const Level<T>& L = lev[l];
+    if constexpr (std::is_same<T, double>::value && !CORR) {
+      if (l == run->cluster_start) {
+        launch(run, s, CHHS_K_COARSEST, 1.0, [&] {
+          pdl_cluster(k_cluster<DIM>, run->cplan.blocks, kTailThreads, cluster_smem_bytes<DIM>(run->cluster, run->cplan),
+                      s, run->cluster, run->cplan, K, nu_pre(run, l), nu_post(run, l));
+        });
+        return;
+      }
+    }
     if (l == run->tail_start) {
       const size_t smem = tail_bytes<T, CORR>(tail);
       launch(run, s, CHHS_K_COARSEST, 1.0, [&] {
@@ -874,6 +907,68 @@ void fill_tail(Tail<T>& tail, const std::vector<Level<T>>& lev, int start, const
   tail.coarsest_f64 = (sizeof(T) == 4 && o.coarsest_f64) ? 1 : 0;
 }
 
+// The levels of k_cluster: above the one-block tail, those of at most
+// kClusterCells cells, as many as the shared memory takes (2D double
+// precision).  In 3D a 16^3 level would leave a block 512 cells and 24 arrays
+// of them (196 KB), for passes that the FP64 pipes of 16 SMs bound anyway.
+// With split_threads 0 the handle asks for the grid-wide passes.
+template <int DIM>
+void place_cluster(chhs_t* run) {
+  if (run->opts.precision != 0 || run->split_threads <= 0) return;
+  const Layout& Lo = run->layout;
+  const int nl = (int)Lo.shapes.size();
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa;
+  const void* fn = reinterpret_cast<const void*>(k_cluster<DIM>);
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  for (int start = 0; start < run->tail_start; ++start) {
+    if (run->lev[start].ncell > kClusterCells || nl - start > kTailMaxLevels) continue;
+    Tail<double> tl{};
+    fill_tail(tl, run->lev, start, run->opts, run->nu1c, run->nu2c);
+    tl.nu1 = run->nu1c;
+    tl.nu2 = run->nu2c;
+    ClusterPlan P{};
+    auto nrows = [&](int l) { return DIM == 3 ? tl.lev[l].nz : tl.lev[l].ny; };
+    P.blocks = 2;
+    while (P.blocks < kClusterMax && 2 * P.blocks < nrows(0)) P.blocks *= 2;
+    P.tail = run->tail_start - start;
+    for (int l = 0; l < tl.n; ++l) P.rows[l] = l < P.tail ? cluster_rows(nrows(l), P.blocks) : nrows(l);
+    const size_t smem = cluster_smem_bytes<DIM>(tl, P);
+    if (smem + fa.sharedSizeBytes > (size_t)optin) continue;
+    if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    // room for one whole cluster on this device (a partition of one may have less)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)P.blocks);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)P.blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, k_cluster<DIM>, &cfg) != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    run->cluster_start = start;
+    run->cluster = tl;
+    run->cplan = P;
+    return;
+  }
+}
+
 // The first level of the one-block tail: the coarsest, and every level above
 // it with at most tail_cells cells (up to kTailMaxLevels levels).
 void place_tail(chhs_t* run) {
@@ -886,6 +981,8 @@ void place_tail(chhs_t* run) {
     --run->tail_start;
   fill_tail(run->tail, run->lev, run->tail_start, run->opts, run->nu1c, run->nu2c);
   fill_tail(run->tail32, run->lev32, run->tail_start, run->opts, run->nu1c, run->nu2c);
+  run->cluster_start = -1;
+  if (run->dim == 2) place_cluster<2>(run);
 }
 
 chhs_status setup_handle(chhs_t* run) {
