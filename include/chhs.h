@@ -238,9 +238,10 @@ typedef struct {
   int coarse_nu1;     /* pre- and post-smoothing sweeps on the levels below the finest (the finest */
   int coarse_nu2;     /* keeps opts->nu1, nu2) */
   int tile_w, tile_h; /* interior of a tile on those levels (even; default 32 x 32 on 512 threads) */
-  int norm_f64_per8;  /* mixed form, double-single residual: of every 8 tiles of the residual
-                         kernel, how many use double-precision instructions (0..8; default 3), so
-                         that the FP64 pipe works beside the single-precision ones */
+  int norm_f64_per8;  /* mixed form, double-single residual: the share of the residual kernel's
+                         blocks that use double-precision instructions, so that the FP64 pipe works
+                         beside the single-precision ones: n/128 for n in 0..7 (default 3), all of
+                         them for 8 */
   int small_tile_w, small_tile_h; /* 2D mixed form: tile interior on the smaller levels */
   int small_tile_threads;         /* (default 16 x 8 cells on 256 threads) and its block size */
   int quad_passes;    /* 3D mixed form: 1 (default) runs the colour passes of levels whose x extent

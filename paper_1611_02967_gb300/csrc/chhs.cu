@@ -71,9 +71,8 @@ int level_fields(int dim, bool single) {
   return kBaseFields + (dim == 3 ? 14 : 12) + (single ? 1 + (dim == 2 ? 6 : 0) : 0);
 }
 
-// The mixed form's residual kernel: of every 8 tiles, this many are evaluated
-// with double-precision instructions and the rest in double-single
-// arithmetic, so that both kinds of pipes are busy (chhs_norm_df.cuh).
+// The mixed form's residual kernel: the share of its blocks evaluated with
+// double-precision instructions, in 128ths (chhs_norm_df.cuh).
 constexpr int kNormF64Per8 = 3;
 
 // Tiles of the 2D single-precision levels: a level of at least
@@ -118,9 +117,9 @@ Layout make_layout(int dim, const int n[3], int coarsest, int precision) {
   off += align_up(sizeof(DevState));
   int nf = L.shapes[0].n[0] * L.shapes[0].n[1] * L.shapes[0].n[2];
   // partial-sum slots: six per 256-cell block (the reductions), and three per
-  // block of the double-single norm (tiles of 32 x 8 cells)
-  L.nparts = (int)std::max<long long>(nblocks(nf),
-                                      (ndf_blocks(L.shapes[0].n[0], L.shapes[0].n[1], L.shapes[0].n[2]) + 1) / 2);
+  // block of the double-single norm (at most one per 32 x 8 cells of a plane)
+  const long long tiles = (long long)ndf_blocks_x(L.shapes[0].n[0]) * ndf_blocks_y(L.shapes[0].n[1]) * L.shapes[0].n[2];
+  L.nparts = (int)std::max<long long>(nblocks(nf), (tiles + 1) / 2);
   L.partial_off = off;
   off += align_up(sizeof(double) * 6 * (size_t)L.nparts);
   L.phimm1_off = off;
@@ -214,7 +213,7 @@ struct chhs {
   // block size; chhs_autotune)
   int tile_w = kLargeTileW, tile_h = kLargeTileH;
   int stile_w = kSmallTileW, stile_h = kSmallTileH, stile_threads = kSmallTileThreads;
-  int norm_f64_per8 = kNormF64Per8;      // blocks of 8 whose residual runs on the FP64 pipe (mixed form)
+  int norm_f64_per8 = kNormF64Per8;      // share of the residual's blocks on the FP64 pipe (mixed form)
   int quad_passes = 1;              // 3D mixed form: x-quad colour passes where nx % 4 == 0 (k_smooth_c4)
   Tail<double> tail{};              // its levels (double-precision V-cycles)
   Tail<float> tail32{};             // (single-precision inner V-cycles)
@@ -603,11 +602,10 @@ struct Enqueue {
     const Level<double>& L = run->lev[0];
     const int nb = run->norm_blocks;
     launch(run, s, CHHS_K_NORM, L.ncell, [&] {
-      if (mixed(run) && !run->opts.f64_residual)
-        pdl(k_norm_mixed_df<DIM>, (int)ndf_blocks(L.nx, L.ny, L.nz), kNdfTX * kNdfTY, s, L, df_coefs(run), K,
-            run->norm_f64_per8, run->lev32[0], run->partials, run->st, cond, mode, use_cond);
-      else if (mixed(run))
-        pdl(k_norm_mixed<DIM>, nb, kBlock, s, L, K, run->lev32[0], run->partials, run->st, cond, mode, use_cond);
+      if (mixed(run))
+        pdl(run->opts.f64_residual ? k_norm_mixed_df<DIM, true> : k_norm_mixed_df<DIM, false>,
+            (int)ndf_blocks<DIM>(L.nx, L.ny, L.nz), kNdfTX * kNdfTY, s, L, df_coefs(run), K, run->norm_f64_per8,
+            run->lev32[0], run->partials, run->st, cond, mode, use_cond);
       else
         pdl(k_norm<double, DIM>, nb, kBlock, s, L, K, run->partials, run->st, cond, mode, use_cond);
     });
@@ -1902,16 +1900,13 @@ struct BatchStep {
   void norm(cudaStream_t s, bool use_cond, int mode) {
     const BatchConds* cc = use_cond ? b->d_conds : nullptr;
     JobList<NormJob> jl;
-    const bool df = !b->opts.f64_residual;
     for (chhs_t* r : b->runs) {
       const Level<double>& L = r->lev[0];
       jl.add(NormJob{L, r->lev32[0], k64(r), Enqueue<DIM>::df_coefs(r), r->partials, r->st, r->norm_f64_per8},
-             df ? (int)ndf_blocks(L.nx, L.ny, L.nz) : r->norm_blocks);
+             (int)ndf_blocks<DIM>(L.nx, L.ny, L.nz));
     }
-    if (df)
-      go(CHHS_K_NORM, jl, kb_norm_mixed_df<DIM>, kNdfTX * kNdfTY, 0, s, b->d_ticket, cc, mode, b->d_ticket + 1);
-    else
-      go(CHHS_K_NORM, jl, kb_norm_mixed<DIM>, kBlock, 0, s, b->d_ticket, cc, mode, b->d_ticket + 1);
+    go(CHHS_K_NORM, jl, b->opts.f64_residual ? kb_norm_mixed_df<DIM, true> : kb_norm_mixed_df<DIM, false>,
+       kNdfTX * kNdfTY, 0, s, b->d_ticket, cc, mode, b->d_ticket + 1);
   }
 
   void vcycle(cudaStream_t s) {

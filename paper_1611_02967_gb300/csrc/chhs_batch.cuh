@@ -161,23 +161,8 @@ __device__ __forceinline__ void batch_norm_epilogue(const NormJob* jobs, int njo
 // The stopping norms of all runs (mode 0: start of a step, every run; mode 1:
 // after a V-cycle, the runs still iterating).  Each run's last block takes
 // that run's decision.
-template <int DIM>
-__global__ void __launch_bounds__(kBlock) kb_norm_mixed(const NormJob* jobs, const int* start, int njobs,
-                                                        unsigned int* ticket, const BatchConds* cc, int mode,
-                                                        unsigned int* any_out) {
-  pdl_enter();
-  const int j = job_of(start, njobs, blockIdx.x);
-  const NormJob& J = job_in_smem(jobs, j);
-  const int lb = blockIdx.x - start[j];
-  bool reports = lb == 0;
-  if (mode == 0 || gate_open(&J.st->go))
-    reports = norm_mixed_body<DIM>(lb, start[j + 1] - start[j], J.L, J.K, J.G, J.partials, J.st, 0, mode, 0);
-  batch_norm_epilogue(jobs, njobs, reports, ticket, cc, any_out);
-}
-
-// The same with the double-single residual (chhs_norm_df.cuh).
-template <int DIM>
-__global__ void __launch_bounds__(kNdfTX * kNdfTY) kb_norm_mixed_df(const NormJob* jobs, const int* start, int njobs,
+template <int DIM, bool F64>
+__global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) kb_norm_mixed_df(const NormJob* jobs, const int* start, int njobs,
                                                                   unsigned int* ticket, const BatchConds* cc,
                                                                   int mode, unsigned int* any_out) {
   pdl_enter();
@@ -186,7 +171,7 @@ __global__ void __launch_bounds__(kNdfTX * kNdfTY) kb_norm_mixed_df(const NormJo
   const int lb = blockIdx.x - start[j];
   bool reports = lb == 0;
   if (mode == 0 || gate_open(&J.st->go))
-    reports = norm_mixed_df_body<DIM>(lb, start[j + 1] - start[j], J.L, J.Kdf, J.K, J.f64_per8, J.G, J.partials,
+    reports = norm_mixed_df_body<DIM, F64>(lb, start[j + 1] - start[j], J.L, J.Kdf, J.K, J.f64_per8, J.G, J.partials,
                                       J.st, 0, mode, 0);
   batch_norm_epilogue(jobs, njobs, reports, ticket, cc, any_out);
 }

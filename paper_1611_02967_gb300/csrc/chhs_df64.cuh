@@ -143,6 +143,25 @@ DF_HD df64 df_mul(df64 x, df64 y) {
   return df_quick_sum(p, e);
 }
 
+// Sum and product without the renormalisation, for sums of differences: the
+// high parts' sum with its error, the low parts added to it.  Exact to 2^-46
+// of the larger operand like df_add and df_mul, but after a cancellation the
+// result's low part may be as large as its high part (every operation here
+// takes such pairs); 8 and 4 instructions instead of 11 and 7.
+DF_HD df64 df_add_raw(df64 x, df64 y) {
+  const df64 s = df_two_sum(x.hi, y.hi);
+  return df64{s.hi, df_fadd(s.lo, df_fadd(x.lo, y.lo))};
+}
+
+DF_HD df64 df_sub_raw(df64 x, df64 y) { return df_add_raw(x, df_neg(y)); }
+
+DF_HD df64 df_mul_raw(df64 x, df64 y) {
+  const float p = df_fmul(x.hi, y.hi);
+  float e = df_ffma(x.hi, y.hi, -p);
+  e = df_ffma(x.hi, y.lo, e);
+  return df64{p, df_ffma(x.lo, y.hi, e)};
+}
+
 DF_HD float df_to_float(df64 x) { return df_fadd(x.hi, x.lo); }
 
 DF_HD double df_to_double(df64 x) { return (double)x.hi + (double)x.lo; }

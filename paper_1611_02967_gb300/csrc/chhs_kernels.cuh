@@ -1082,63 +1082,6 @@ __global__ void __launch_bounds__(kBlock) k_coef_restrict_f32(Level<double> F, L
   coef_restrict_f32_body<DIM>(blockIdx.x, F, G, K, Gn, has_next);
 }
 
-// The stopping norm of the double-precision iterate, as k_norm, and the
-// right-hand side of the next inner solve: f32 = r cut to single precision,
-// e = 0, phi_b = phi cut to single precision.
-template <int DIM>
-__device__ __forceinline__ bool norm_mixed_body(int bx, int nbx, const Level<double>& L, const Coefs<double>& K,
-                                                const Level<float>& G,
-                                                       double* partials, DevState* st,
-                                                       cudaGraphConditionalHandle cond, int mode, int use_cond) {
-  __shared__ bool last;
-  double acc[2] = {0.0, 0.0};
-  double mx = 0.0;
-  const int stride = nbx * blockDim.x;
-  for (int c = bx * blockDim.x + threadIdx.x; c < L.ncell; c += stride) {
-    int i, j, k;
-    cell_ijk(c, L.nx, L.ny, i, j, k);
-    double n1, n2, n3;
-    eval_N<double, DIM, false>(L, K, L.phi, L.mu, L.p, c, i, j, k, n1, n2, n3);
-    double r1 = L.fphi[c] - n1, r2 = L.fmu[c] - n2, r3 = L.fp[c] - n3;
-    double r3s = K.s * r3;
-    acc[0] = fma(r1, r1, acc[0]);
-    acc[0] = fma(r2, r2, acc[0]);
-    acc[0] = fma(r3s, r3s, acc[0]);
-    acc[1] += L.p[c];
-    mx = fmax(mx, row_max(r1, r2, r3s));
-    G.fphi[c] = f64_to_f32_rz(r1);
-    G.fmu[c] = f64_to_f32_rz(r2);
-    G.fp[c] = f64_to_f32_rz(r3);
-    G.phi[c] = 0.f;
-    G.mu[c] = 0.f;
-    G.p[c] = 0.f;
-    G.phib[c] = f64_to_f32_rz(L.phi[c]);
-  }
-  block_sum<2>(acc);
-  mx = block_max(mx);
-  if (threadIdx.x == 0) {
-    partials[3 * bx] = acc[0];
-    partials[3 * bx + 1] = acc[1];
-    partials[3 * bx + 2] = mx;
-    __threadfence();
-    last = atomicAdd(&st->ticket, 1u) == nbx - 1;
-  }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  norm_finish(partials, nbx, L.ncell, st, cond, mode, use_cond);
-  return true;
-}
-
-template <int DIM>
-__global__ void __launch_bounds__(kBlock) k_norm_mixed(const __grid_constant__ Level<double> L, Coefs<double> K,
-                                                       const __grid_constant__ Level<float> G,
-                                                       double* partials, DevState* st,
-                                                       cudaGraphConditionalHandle cond, int mode, int use_cond) {
-  pdl_enter();
-  norm_mixed_body<DIM>(blockIdx.x, gridDim.x, L, K, G, partials, st, cond, mode, use_cond);
-}
-
 // u <- u + e in double precision.
 static __device__ __forceinline__ void mixed_update_body(int bx, Level<double> L, Level<float> G) {
   int c = bx * blockDim.x + threadIdx.x;

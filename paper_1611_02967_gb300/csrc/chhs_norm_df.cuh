@@ -2,38 +2,70 @@
 // f - N(u) of the double-precision iterate, evaluated in double-single
 // arithmetic (chhs_df64.cuh) on the single-precision pipes.
 //
-// Same outputs as k_norm_mixed: the stopping norm and the pointwise residual
-// (the loop decision of the step graph), the mean of p, and the next inner
-// solve's right-hand side (r rounded to single precision, e = 0,
-// phi_b = phi cut to single precision).  The residual is formed in the
-// difference form of Eqs. 2.5-2.7,
-//   N1 = phi - s/h^2 sum_f [M_f (mu_e - mu_c) + a_f (p_e - p_c)]
-//   N2 = mu + (3/4) eps^2/h^2 sum_f (phi_e - phi_c) - phi (phi^2 + phi phi^m + (phi^m)^2)/4
-//   N3 = -1/h^2 sum_f [(p_e - p_c) + gamma a_f (mu_e - mu_c)]
+// Outputs: the stopping norm and the pointwise residual (the loop decision of
+// the step graph), the mean of p, and the next inner solve's right-hand side
+// (r rounded to single precision, e = 0, phi_b = phi cut to single
+// precision).  The residual is formed from the fluxes of the faces between
+// two cells c and e, with a = (phi*_c + phi*_e)/2 and d the difference e - c,
+//   w = dp + gamma a dmu,          v = dmu + a w  ( = M dmu + a dp ),
+//   N1 = phi - s/h^2 sum_f v,      N3 = -1/h^2 sum_f w,
+//   N2 = mu + (3/4) eps^2/h^2 sum_f dphi - phi (phi^2 + phi phi^m + (phi^m)^2)/4
 // (N2 and f_mu carry the same constant shift (phi^m)^3/4 as the
-// double-precision kernels, see cubic_P), with every double input split
-// into hi + lo and every operation a double-single one: the residual is
-// exact to ~1e-14 relative to the terms, far below the 1e-10 stopping
-// tolerance, at a quarter of the issue slots of double precision on GB300.
+// double-precision kernels, see cubic_P; f_phi = phi^m and f_p = 0 on the
+// finest level), with every double input split into hi + lo and every
+// operation a double-single one: the residual is exact to ~1e-14 relative to
+// the terms, far below the 1e-10 stopping tolerance.
 //
-// Each block takes a tile of 32 x 8 cells of one z-plane: the double state
-// (phi, mu, p) and the +x/+y face coefficients of the tile and its one-cell
-// ring are split once into shared memory; z-neighbours (3D) are split where
-// they are read.
+// What bounds it: issue slots (a double-single addition is 8 instructions),
+// so the work per cell is kept small.  In 3D a block takes a column of 32 x 8
+// cells and marches through up to 16 planes: every double is split once (the
+// tile's one-cell ring adds 31 %), every face's flux is formed once and given
+// to both of its cells (x and y through shared memory, z in registers), and
+// the coefficients come from phi* (w above needs no stored M).  In 2D a warp
+// marches up a strip of 32 cells, x neighbours by shuffles, without shared
+// memory or block barriers.
+//
+// Measured per launch (GB300, kernel by kernel with events), against a kernel
+// of one plane per block that read the stored a and M, formed each flux on
+// both sides and ran three of eight tiles on the FP64 pipe (~1 460
+// instructions per cell): 256^3 1056 -> 491 us, 128^3 159 -> 93 us,
+// 2048^2 231 -> 136 us.
 #pragma once
+#include <type_traits>
+
 #include "chhs_df64.cuh"
 #include "chhs_kernels.cuh"
 
 namespace chhs_dev {
 
-constexpr int kNdfTX = 32, kNdfTY = 8;  // 256 threads, one cell each
+constexpr int kNdfTX = 32, kNdfTY = 8;  // 256 threads, one cell of the plane each
 constexpr int kNdfSW = kNdfTX + 2, kNdfSH = kNdfTY + 2, kNdfSN = kNdfSW * kNdfSH;
+constexpr int kNdfRing = 2 * (kNdfTX + kNdfTY);  // ring cells without the corners
 
-// Blocks of the double-single norm on an nx x ny x nz grid.
+// Planes a block marches through, and the blocks of an nx x ny x nz grid.
 __host__ __device__ inline int ndf_blocks_x(int nx) { return (nx + kNdfTX - 1) / kNdfTX; }
 __host__ __device__ inline int ndf_blocks_y(int ny) { return (ny + kNdfTY - 1) / kNdfTY; }
+__host__ __device__ inline int ndf_planes(int nx, int ny, int nz) {
+  const long long columns = (long long)ndf_blocks_x(nx) * ndf_blocks_y(ny);
+  int planes = 16;
+  while (planes > 2 && columns * ((nz + planes - 1) / planes) < 900) planes >>= 1;
+  return planes;
+}
+// Rows a warp marches through in 2D; a block's eight warps take eight such
+// runs of rows of one strip.
+__host__ __device__ inline int ndf_rows(int nx, int ny) {
+  int rows = 16;
+  while (rows > 1 && (long long)ndf_blocks_x(nx) * ((ny + 8 * rows - 1) / (8 * rows)) < 300) rows >>= 1;
+  return rows;
+}
+template <int DIM>
 __host__ __device__ inline long long ndf_blocks(int nx, int ny, int nz) {
-  return (long long)ndf_blocks_x(nx) * ndf_blocks_y(ny) * nz;
+  if (DIM == 2) {
+    const int run = 8 * ndf_rows(nx, ny);
+    return (long long)ndf_blocks_x(nx) * ((ny + run - 1) / run);
+  }
+  const int planes = ndf_planes(nx, ny, nz);
+  return (long long)ndf_blocks_x(nx) * ndf_blocks_y(ny) * ((nz + planes - 1) / planes);
 }
 
 // The level's scalar coefficients as double-single numbers (host-split).
@@ -41,6 +73,59 @@ struct DfCoefs {
   df64 sih2, ih2, e34ih2, gamma;
   float s;
 };
+
+// The residual's arithmetic: double-single, or double precision for the share
+// of the blocks that runs on the FP64 pipe (chhs_tuning.norm_f64_per8, or all
+// with chhs_opts.f64_residual).  Both are 8 bytes a value.  A block on the
+// FP64 pipe takes ~5 times as long as one beside it, so the share's unit is
+// small, n/128 of the blocks, and they are the launch's first (256^3: 497 us
+// without, 499 us with 3/128, 581 with 3/32, 919 with 3/8; a share of 3/8 had
+// paid while the double-single blocks spent twice the instructions).
+struct NdfSingle {
+  using V = df64;
+  static __device__ __forceinline__ V from(double x) { return df_split(x); }
+  static __device__ __forceinline__ V add(V a, V b) { return df_add_raw(a, b); }
+  static __device__ __forceinline__ V sub(V a, V b) { return df_sub_raw(a, b); }
+  static __device__ __forceinline__ V mul(V a, V b) { return df_mul_raw(a, b); }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return df_add_raw(df_mul_raw(a, b), c); }
+  static __device__ __forceinline__ V half(V a) { return df64{0.5f * a.hi, 0.5f * a.lo}; }
+  static __device__ __forceinline__ V zero() { return df64{0.f, 0.f}; }
+  static __device__ __forceinline__ float cut(V a) { return df_to_float(a); }
+  static __device__ __forceinline__ float base(V a) { return a.hi; }
+};
+struct NdfDouble {
+  using V = double;
+  static __device__ __forceinline__ V from(double x) { return x; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
+  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return ::fma(a, b, c); }
+  static __device__ __forceinline__ V half(V a) { return 0.5 * a; }
+  static __device__ __forceinline__ V zero() { return 0.0; }
+  static __device__ __forceinline__ float cut(V a) { return f64_to_f32_rz(a); }
+  static __device__ __forceinline__ float base(V a) { return f64_to_f32_rz(a); }
+};
+
+// A face's fluxes from the cell below it to the one above, and the four
+// fields of a cell (phi, mu, p, phi*).
+template <class A>
+struct NdfFlux {
+  typename A::V v, w, d;
+};
+template <class A>
+struct NdfCell {
+  typename A::V phi, mu, p, ps;
+};
+
+template <class A>
+__device__ __forceinline__ NdfFlux<A> ndf_face(const NdfCell<A>& lo, const NdfCell<A>& hi, typename A::V gamma) {
+  NdfFlux<A> F;
+  const typename A::V a = A::half(A::add(lo.ps, hi.ps)), dmu = A::sub(hi.mu, lo.mu);
+  F.d = A::sub(hi.phi, lo.phi);
+  F.w = A::fma(gamma, A::mul(a, dmu), A::sub(hi.p, lo.p));
+  F.v = A::fma(a, F.w, dmu);
+  return F;
+}
 
 // Block sums: thread 0 returns the sum of squares, the double-single sum of
 // p and the maximum.
@@ -70,141 +155,299 @@ __device__ __forceinline__ void ndf_block_reduce(float& sq, df64& ps, float& mx)
   __syncthreads();
 }
 
-// The double-precision pipe and the single-precision/integer pipes work at
-// the same time: a share of the blocks (f64_per8 of every 8) evaluates its
-// tile's residual with double-precision instructions (eval_N), the others in
-// double-single arithmetic; on one SM the former wait on the FP64 pipe while
-// the latter fill the issue slots.  Both write the same outputs, and the
-// residual is exact to far below the stopping tolerance either way.
-//
-// bx: the block's index among the run's nbx blocks (x-tiles fastest, then
-// y-tiles, then z-planes).  Returns true in the run's last block (which took
-// the loop decision).
-template <int DIM>
-__device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<double>& L, const DfCoefs& K,
-                                                   const Coefs<double>& K64, int f64_per8, const Level<float>& G,
-                                                   double* partials, DevState* st, cudaGraphConditionalHandle cond,
-                                                   int mode, int use_cond) {
-  __shared__ df64 sP[kNdfSN], sU[kNdfSN], sQ[kNdfSN], sAx[kNdfSN], sMx[kNdfSN], sAy[kNdfSN], sMy[kNdfSN];
-  __shared__ bool last;
-  const int nx = L.nx, ny = L.ny, nz = L.nz;
-  const int gx = ndf_blocks_x(nx), gy = ndf_blocks_y(ny);
-  const int tx_blk = bx % gx;
-  const int rest = bx / gx;
-  const int ty_blk = rest % gy, k = rest / gy;
-  const int x0 = tx_blk * kNdfTX, y0 = ty_blk * kNdfTY;
-  const int sz = nx * ny;
-  if ((bx & 7) < f64_per8) {  // this tile in double precision
-    const int tx = threadIdx.x % kNdfTX, ty = threadIdx.x / kNdfTX;
-    const int i = x0 + tx, j = y0 + ty;
-    float sq = 0.f, mx = 0.f;
-    df64 ps{0.f, 0.f};
-    if (i < nx && j < ny) {
-      const int c = i + nx * j + sz * k;
-      double n1, n2, n3;
-      eval_N<double, DIM, false>(L, K64, L.phi, L.mu, L.p, c, i, j, k, n1, n2, n3);
-      const double r1 = L.fphi[c] - n1, r2 = L.fmu[c] - n2, r3 = L.fp[c] - n3;
-      const float r1f = f64_to_f32_rz(r1), r2f = f64_to_f32_rz(r2), r3f = f64_to_f32_rz(r3);
-      const float r3s = K.s * r3f;
-      sq = r1f * r1f + r2f * r2f + r3s * r3s;
-      mx = fmaxf(fmaxf(fabsf(r1f), fabsf(r2f)), fabsf(r3s));
-      const double pc = L.p[c];
-      ps = df_split(pc);
-      G.fphi[c] = r1f;
-      G.fmu[c] = r2f;
-      G.fp[c] = r3f;
-      G.phi[c] = 0.f;
-      G.mu[c] = 0.f;
-      G.p[c] = 0.f;
-      G.phib[c] = f64_to_f32_rz(L.phi[c]);
-    }
-    ndf_block_reduce(sq, ps, mx);
-    if (threadIdx.x == 0) {
-      partials[3 * bx] = (double)sq;
-      partials[3 * bx + 1] = df_to_double(ps);
-      partials[3 * bx + 2] = (double)mx;
-      __threadfence();
-      last = atomicAdd(&st->ticket, 1u) == nbx - 1;
-    }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    norm_finish(partials, nbx, L.ncell, st, cond, mode, use_cond);
-    return true;
-  }
-  // the tile and its ring, split once
-  for (int q = threadIdx.x; q < kNdfSN; q += blockDim.x) {
-    const int qy = q / kNdfSW, qx = q - qy * kNdfSW;
-    const int i = x0 - 1 + qx, j = y0 - 1 + qy;
-    if (i < 0 || j < 0 || i >= nx || j >= ny) continue;
-    const int c = i + nx * j + sz * k;
-    sP[q] = df_split(L.phi[c]);
-    sU[q] = df_split(L.mu[c]);
-    sQ[q] = df_split(L.p[c]);
-    sAx[q] = df_split(L.ax[c]);
-    sMx[q] = df_split(L.Mx[c]);
-    sAy[q] = df_split(L.ay[c]);
-    sMy[q] = df_split(L.My[c]);
-  }
-  __syncthreads();
-  const int tx = threadIdx.x % kNdfTX, ty = threadIdx.x / kNdfTX;
-  const int i = x0 + tx, j = y0 + ty;
+// Sums of a block's cells: in single precision (p double-single) beside the
+// double-single residual, in double precision with f64_residual.
+struct NdfSums32 {
   float sq = 0.f, mx = 0.f;
   df64 ps{0.f, 0.f};
-  if (i < nx && j < ny) {
-    const int c = i + nx * j + sz * k;
-    const int s = (tx + 1) + kNdfSW * (ty + 1);
-    const df64 phic = sP[s], muc = sU[s], pc = sQ[s];
-    df64 S1{0.f, 0.f}, Sa{0.f, 0.f}, Sp{0.f, 0.f}, Sphi{0.f, 0.f};
-    auto face = [&](df64 phe, df64 mue, df64 pe, df64 a, df64 M) {
-      const df64 dmu = df_sub(mue, muc), dp = df_sub(pe, pc), dphi = df_sub(phe, phic);
-      S1 = df_add(S1, df_add(df_mul(M, dmu), df_mul(a, dp)));
-      Sa = df_add(Sa, df_mul(a, dmu));
-      Sp = df_add(Sp, dp);
-      Sphi = df_add(Sphi, dphi);
-    };
-    if (i > 0) face(sP[s - 1], sU[s - 1], sQ[s - 1], sAx[s - 1], sMx[s - 1]);
-    if (i + 1 < nx) face(sP[s + 1], sU[s + 1], sQ[s + 1], sAx[s], sMx[s]);
-    if (j > 0) face(sP[s - kNdfSW], sU[s - kNdfSW], sQ[s - kNdfSW], sAy[s - kNdfSW], sMy[s - kNdfSW]);
-    if (j + 1 < ny) face(sP[s + kNdfSW], sU[s + kNdfSW], sQ[s + kNdfSW], sAy[s], sMy[s]);
-    if (DIM == 3) {
-      if (k > 0) {
-        const int e = c - sz;
-        face(df_split(L.phi[e]), df_split(L.mu[e]), df_split(L.p[e]), df_split(L.az[e]), df_split(L.Mz[e]));
-      }
-      if (k + 1 < nz) {
-        const int e = c + sz;
-        face(df_split(L.phi[e]), df_split(L.mu[e]), df_split(L.p[e]), df_split(L.az[c]), df_split(L.Mz[c]));
-      }
+  __device__ __forceinline__ void add(float r1, float r2, float r3s) {
+    sq += r1 * r1 + r2 * r2 + r3s * r3s;
+    mx = fmaxf(mx, fmaxf(fmaxf(fabsf(r1), fabsf(r2)), fabsf(r3s)));
+  }
+  __device__ __forceinline__ void finish(double (&out)[3]) {
+    ndf_block_reduce(sq, ps, mx);
+    out[0] = (double)sq;
+    out[1] = df_to_double(ps);
+    out[2] = (double)mx;
+  }
+};
+struct NdfSums64 {
+  double acc[2] = {0.0, 0.0}, mx = 0.0;
+  __device__ __forceinline__ void add(double r1, double r2, double r3s) {
+    acc[0] = ::fma(r1, r1, acc[0]);
+    acc[0] = ::fma(r2, r2, acc[0]);
+    acc[0] = ::fma(r3s, r3s, acc[0]);
+    mx = fmax(mx, row_max(r1, r2, r3s));
+  }
+  __device__ __forceinline__ void finish(double (&out)[3]) {
+    block_sum<2>(acc);
+    out[0] = acc[0];
+    out[1] = acc[1];
+    out[2] = block_max(mx);
+  }
+};
+
+struct NdfShared {
+  df64 cell[4][kNdfSN];                      // phi, mu, p, phi* of the tile and its ring
+  df64 fx[3][kNdfTY * (kNdfTX + 1)];         // v, w, d of the x faces
+  df64 fy[3][(kNdfTY + 1) * kNdfTX];         // ... and of the y faces
+};
+
+// A cell's residual from its summed fluxes (sv, sw, sd), and what the next
+// inner solve reads; c: its index.
+template <class A, class SUMS>
+struct NdfOut {
+  using V = typename A::V;
+  const Level<float>& G;
+  V sih2, ih2, e34ih2;
+  float s32;
+  double s64;
+  SUMS& sums;
+  __device__ __forceinline__ void cell(int c, const NdfCell<A>& u, V sv, V sw, V sd, double pm64, double fmu64) {
+    const V pm = A::from(pm64);
+    const V r1 = A::fma(sih2, sv, A::sub(pm, u.phi));
+    const V quad = A::fma(u.phi, A::add(u.phi, pm), A::mul(pm, pm));
+    const V cub = A::half(A::half(A::mul(u.phi, quad)));
+    const V r2 = A::sub(A::add(A::sub(A::from(fmu64), u.mu), cub), A::mul(e34ih2, sd));
+    const V r3 = A::mul(ih2, sw);
+    const float r1f = A::cut(r1), r2f = A::cut(r2), r3f = A::cut(r3);
+    if constexpr (std::is_same<SUMS, NdfSums64>::value) {
+      sums.add(r1, r2, s64 * r3);
+      sums.acc[1] += u.p;
+    } else {
+      sums.add(r1f, r2f, s32 * r3f);
+      if constexpr (std::is_same<A, NdfSingle>::value) sums.ps = df_add(sums.ps, u.p);
+      else sums.ps = df_add(sums.ps, df_split(u.p));
     }
-    const df64 pm = df_split(L.phim[c]);
-    // N1, N3 and the shifted N2 (see above)
-    const df64 n1 = df_sub(phic, df_mul(K.sih2, S1));
-    const df64 n3 = df_neg(df_mul(K.ih2, df_add(Sp, df_mul(K.gamma, Sa))));
-    const df64 quad = df_add(df_mul(phic, df_add(phic, pm)), df_mul(pm, pm));
-    const df64 cub = df_mul(df_mul(phic, quad), df64{0.25f, 0.f});
-    const df64 n2 = df_sub(df_add(muc, df_mul(K.e34ih2, Sphi)), cub);
-    const df64 r1 = df_sub(df_split(L.fphi[c]), n1);
-    const df64 r2 = df_sub(df_split(L.fmu[c]), n2);
-    const df64 r3 = df_sub(df_split(L.fp[c]), n3);
-    const float r1f = df_to_float(r1), r2f = df_to_float(r2), r3f = df_to_float(r3);
-    const float r3s = K.s * r3f;
-    sq = r1f * r1f + r2f * r2f + r3s * r3s;
-    mx = fmaxf(fmaxf(fabsf(r1f), fabsf(r2f)), fabsf(r3s));
-    ps = pc;
     G.fphi[c] = r1f;
     G.fmu[c] = r2f;
     G.fp[c] = r3f;
     G.phi[c] = 0.f;
     G.mu[c] = 0.f;
     G.p[c] = 0.f;
-    G.phib[c] = phic.hi;  // phi with its significand cut to 24 bits
+    G.phib[c] = A::base(u.phi);  // phi with its significand cut to 24 bits
   }
-  ndf_block_reduce(sq, ps, mx);
+};
+
+__device__ __forceinline__ df64 ndf_shfl_up(df64 v) {
+  return df64{__shfl_up_sync(0xffffffffu, v.hi, 1), __shfl_up_sync(0xffffffffu, v.lo, 1)};
+}
+__device__ __forceinline__ double ndf_shfl_up(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ df64 ndf_shfl_down(df64 v) {
+  return df64{__shfl_down_sync(0xffffffffu, v.hi, 1), __shfl_down_sync(0xffffffffu, v.lo, 1)};
+}
+__device__ __forceinline__ double ndf_shfl_down(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+// 2D: one warp's strip, the cells x0 .. x0+31 of the rows j0 .. j1-1.
+template <class A, class SUMS>
+__device__ __forceinline__ void ndf_strip(int x0, int j0, int j1, const Level<double>& L, typename A::V gamma,
+                                          NdfOut<A, SUMS>& out) {
+  using V = typename A::V;
+  using Cell = NdfCell<A>;
+  using Flux = NdfFlux<A>;
+  const Flux none{A::zero(), A::zero(), A::zero()};
+  const Cell empty{A::zero(), A::zero(), A::zero(), A::zero()};
+  const int nx = L.nx, lane = threadIdx.x & 31, i = x0 + lane;
+  const bool in = i < nx;
+  const int col = in ? i : 0;
+  auto load = [&](int c) { return Cell{A::from(L.phi[c]), A::from(L.mu[c]), A::from(L.p[c]), A::from(L.phis[c])}; };
+  // the cells beside the strip, held by its first and last lane
+  const int rcol = lane == 0 ? x0 - 1 : x0 + 32;
+  const bool ring = (lane == 0 && x0 > 0) || (lane == 31 && x0 + 32 < nx);
+  Cell cur = empty;
+  Flux below = none;
+  if (j0 < j1 && in) {
+    cur = load(col + nx * j0);
+    if (j0 > 0) below = ndf_face<A>(load(col + nx * (j0 - 1)), cur, gamma);
+  }
+  for (int j = j0; j < j1; ++j) {
+    const int c = col + nx * j;
+    const bool up = in && j + 1 < L.ny;
+    double nxt[4], pm64 = 0.0, fmu64 = 0.0;
+    if (up) {
+      nxt[0] = L.phi[c + nx];
+      nxt[1] = L.mu[c + nx];
+      nxt[2] = L.p[c + nx];
+      nxt[3] = L.phis[c + nx];
+    }
+    if (in) {
+      pm64 = L.phim[c];
+      fmu64 = L.fmu[c];
+    }
+    const Cell side = ring ? load(rcol + nx * j) : empty;
+    Cell left{ndf_shfl_up(cur.phi), ndf_shfl_up(cur.mu), ndf_shfl_up(cur.p), ndf_shfl_up(cur.ps)};
+    if (lane == 0) left = side;
+    const Flux W = in && i > 0 ? ndf_face<A>(left, cur, gamma) : none;
+    Flux E{ndf_shfl_down(W.v), ndf_shfl_down(W.w), ndf_shfl_down(W.d)};
+    if (lane == 31) E = ring ? ndf_face<A>(cur, side, gamma) : none;
+    Cell above = empty;
+    Flux N = none;
+    if (up) {
+      above = Cell{A::from(nxt[0]), A::from(nxt[1]), A::from(nxt[2]), A::from(nxt[3])};
+      N = ndf_face<A>(cur, above, gamma);
+    }
+    if (in)
+      out.cell(c, cur, A::add(A::sub(E.v, W.v), A::sub(N.v, below.v)), A::add(A::sub(E.w, W.w), A::sub(N.w, below.w)),
+               A::add(A::sub(E.d, W.d), A::sub(N.d, below.d)), pm64, fmu64);
+    cur = above;
+    below = N;
+  }
+}
+
+// 3D: one block's column, the cells of its tile on the planes k0 .. k1-1.
+template <class A, class SUMS>
+__device__ __forceinline__ void ndf_column(NdfShared& sh, int x0, int y0, int k0, int k1, const Level<double>& L,
+                                           typename A::V gamma, NdfOut<A, SUMS>& out) {
+  using V = typename A::V;
+  using Cell = NdfCell<A>;
+  using Flux = NdfFlux<A>;
+  V* const cP = reinterpret_cast<V*>(sh.cell[0]);
+  V* const cU = reinterpret_cast<V*>(sh.cell[1]);
+  V* const cQ = reinterpret_cast<V*>(sh.cell[2]);
+  V* const cS = reinterpret_cast<V*>(sh.cell[3]);
+  auto put = [](df64 (&f)[3][kNdfTY * (kNdfTX + 1)], int q, const Flux& F) {
+    reinterpret_cast<V*>(f[0])[q] = F.v;
+    reinterpret_cast<V*>(f[1])[q] = F.w;
+    reinterpret_cast<V*>(f[2])[q] = F.d;
+  };
+  auto puty = [](df64 (&f)[3][(kNdfTY + 1) * kNdfTX], int q, const Flux& F) {
+    reinterpret_cast<V*>(f[0])[q] = F.v;
+    reinterpret_cast<V*>(f[1])[q] = F.w;
+    reinterpret_cast<V*>(f[2])[q] = F.d;
+  };
+  auto cell_at = [&](int q) { return Cell{cP[q], cU[q], cQ[q], cS[q]}; };
+  auto store_cell = [&](int q, const Cell& c) {
+    cP[q] = c.phi;
+    cU[q] = c.mu;
+    cQ[q] = c.p;
+    cS[q] = c.ps;
+  };
+  const Flux none{A::zero(), A::zero(), A::zero()};
+  const int nx = L.nx, ny = L.ny, nz = L.nz, sz = nx * ny;
+  const int tx = threadIdx.x % kNdfTX, ty = threadIdx.x / kNdfTX;
+  const int i = x0 + tx, j = y0 + ty, q = (tx + 1) + kNdfSW * (ty + 1);
+  const bool in = i < nx && j < ny;
+  const int c2 = in ? i + nx * j : 0;  // the cell in its plane
+  auto load = [&](int c) { return Cell{A::from(L.phi[c]), A::from(L.mu[c]), A::from(L.p[c]), A::from(L.phis[c])}; };
+  // ring cells: the columns left and right of the tile, the rows below and above
+  const int t = threadIdx.x;
+  const int rx = t < kNdfTY ? -1 : t < 2 * kNdfTY ? kNdfTX : (t - 2 * kNdfTY) % kNdfTX;
+  const int ry = t < 2 * kNdfTY ? t % kNdfTY : t < 2 * kNdfTY + kNdfTX ? -1 : kNdfTY;
+  const bool ring = t < kNdfRing && x0 + rx >= 0 && x0 + rx < nx && y0 + ry >= 0 && y0 + ry < ny;
+  const int rq = (rx + 1) + kNdfSW * (ry + 1), rc = ring ? (x0 + rx) + nx * (y0 + ry) : 0;
+  // the faces right of the tile's last column and above its last row
+  const bool extra = t < kNdfTX + kNdfTY;
+  const int ex = t < kNdfTX ? t : kNdfTX - 1, ey = t < kNdfTX ? kNdfTY - 1 : t - kNdfTX;
+  const int eq = (ex + 1) + kNdfSW * (ey + 1);
+  const bool ein = extra && (t < kNdfTX ? x0 + ex < nx && y0 + kNdfTY < ny : x0 + kNdfTX < nx && y0 + ey < ny);
+
+  Cell cur{A::zero(), A::zero(), A::zero(), A::zero()};
+  Flux zlow = none;
+  if (in) {
+    cur = load(c2 + sz * k0);
+    if (k0 > 0) zlow = ndf_face<A>(load(c2 + sz * (k0 - 1)), cur, gamma);
+    store_cell(q, cur);
+  }
+  if (ring) store_cell(rq, load(rc + sz * k0));
+  for (int k = k0; k < k1; ++k) {
+    __syncthreads();
+    const int c = c2 + sz * k;
+    double nxt[4], rng[4], pm64 = 0.0, fmu64 = 0.0;  // the next plane's cells, loaded before they are needed
+    const bool up = k + 1 < nz;
+    if (in) {
+      pm64 = L.phim[c];
+      fmu64 = L.fmu[c];
+      if (up) {
+        nxt[0] = L.phi[c + sz];
+        nxt[1] = L.mu[c + sz];
+        nxt[2] = L.p[c + sz];
+        nxt[3] = L.phis[c + sz];
+      }
+    }
+    const bool more = k + 1 < k1;
+    if (ring && more) {
+      const int r = rc + sz * (k + 1);
+      rng[0] = L.phi[r];
+      rng[1] = L.mu[r];
+      rng[2] = L.p[r];
+      rng[3] = L.phis[r];
+    }
+    const Flux W = in && i > 0 ? ndf_face<A>(cell_at(q - 1), cur, gamma) : none;
+    const Flux S = in && j > 0 ? ndf_face<A>(cell_at(q - kNdfSW), cur, gamma) : none;
+    put(sh.fx, tx + (kNdfTX + 1) * ty, W);
+    puty(sh.fy, tx + kNdfTX * ty, S);
+    if (extra) {
+      const Flux E = ein ? ndf_face<A>(cell_at(eq), cell_at(t < kNdfTX ? eq + kNdfSW : eq + 1), gamma) : none;
+      if (t < kNdfTX) puty(sh.fy, t + kNdfTX * kNdfTY, E);
+      else put(sh.fx, kNdfTX + (kNdfTX + 1) * ey, E);
+    }
+    Cell above{A::zero(), A::zero(), A::zero(), A::zero()};
+    Flux zup = none;
+    if (in && up) {
+      above = Cell{A::from(nxt[0]), A::from(nxt[1]), A::from(nxt[2]), A::from(nxt[3])};
+      zup = ndf_face<A>(cur, above, gamma);
+    }
+    __syncthreads();
+    if (in) {
+      auto fx = [&](int m) { return reinterpret_cast<const V*>(sh.fx[m])[tx + 1 + (kNdfTX + 1) * ty]; };
+      auto fy = [&](int m) { return reinterpret_cast<const V*>(sh.fy[m])[tx + kNdfTX * (ty + 1)]; };
+      V sv = A::add(A::sub(fx(0), W.v), A::sub(fy(0), S.v));
+      V sw = A::add(A::sub(fx(1), W.w), A::sub(fy(1), S.w));
+      V sd = A::add(A::sub(fx(2), W.d), A::sub(fy(2), S.d));
+      sv = A::add(sv, A::sub(zup.v, zlow.v));
+      sw = A::add(sw, A::sub(zup.w, zlow.w));
+      sd = A::add(sd, A::sub(zup.d, zlow.d));
+      out.cell(c, cur, sv, sw, sd, pm64, fmu64);
+    }
+    if (more) {
+      if (in) store_cell(q, above);
+      if (ring) store_cell(rq, Cell{A::from(rng[0]), A::from(rng[1]), A::from(rng[2]), A::from(rng[3])});
+      cur = above;
+      zlow = zup;
+    }
+  }
+}
+
+// bx: the block's index among the run's nbx blocks (x-tiles fastest, then
+// y-tiles, then the chunks of planes; in 2D strips, then runs of rows).  F64: every block and the sums in
+// double precision (f64_residual).  Returns true in the run's last block
+// (which took the loop decision).
+template <int DIM, bool F64>
+__device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<double>& L, const DfCoefs& K,
+                                                   const Coefs<double>& K64, int f64_per8, const Level<float>& G,
+                                                   double* partials, DevState* st, cudaGraphConditionalHandle cond,
+                                                   int mode, int use_cond) {
+  __shared__ __align__(16) unsigned char raw[DIM == 3 ? sizeof(NdfShared) : 16];
+  __shared__ bool last;
+  const int gx = ndf_blocks_x(L.nx);
+  const int rest = bx / gx, x0 = (bx - rest * gx) * kNdfTX;
+  auto residual = [&](auto arith, auto& sums, auto sih2, auto ih2, auto e34ih2, auto gamma) {
+    using A = decltype(arith);
+    NdfOut<A, std::remove_reference_t<decltype(sums)>> out{G, sih2, ih2, e34ih2, K.s, K64.s, sums};
+    if constexpr (DIM == 2) {
+      const int rows = ndf_rows(L.nx, L.ny), j0 = (rest * (kNdfTX * kNdfTY / 32) + (threadIdx.x >> 5)) * rows;
+      ndf_strip<A>(x0, j0, min(j0 + rows, L.ny), L, gamma, out);
+    } else {
+      const int gy = ndf_blocks_y(L.ny), chunk = rest / gy;
+      const int planes = ndf_planes(L.nx, L.ny, L.nz), k0 = chunk * planes;
+      ndf_column<A>(reinterpret_cast<NdfShared&>(raw), x0, (rest - chunk * gy) * kNdfTY, k0, min(k0 + planes, L.nz), L, gamma, out);
+    }
+  };
+  double out[3];
+  if constexpr (F64) {
+    NdfSums64 sums;
+    residual(NdfDouble{}, sums, L.sih2, L.ih2, L.e34ih2, K64.gamma);
+    sums.finish(out);
+  } else {
+    NdfSums32 sums;
+    if (f64_per8 == 8 || bx < (int)((long long)nbx * f64_per8 / 128)) residual(NdfDouble{}, sums, L.sih2, L.ih2, L.e34ih2, K64.gamma);
+    else residual(NdfSingle{}, sums, K.sih2, K.ih2, K.e34ih2, K.gamma);
+    sums.finish(out);
+  }
   if (threadIdx.x == 0) {
-    partials[3 * bx] = (double)sq;
-    partials[3 * bx + 1] = df_to_double(ps);
-    partials[3 * bx + 2] = (double)mx;
+    partials[3 * bx] = out[0];
+    partials[3 * bx + 1] = out[1];
+    partials[3 * bx + 2] = out[2];
     __threadfence();
     last = atomicAdd(&st->ticket, 1u) == nbx - 1;
   }
@@ -215,15 +458,15 @@ __device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<
   return true;
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(kNdfTX * kNdfTY) k_norm_mixed_df(const __grid_constant__ Level<double> L,
+template <int DIM, bool F64>
+__global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) k_norm_mixed_df(const __grid_constant__ Level<double> L,
                                                                  DfCoefs K, Coefs<double> K64, int f64_per8,
                                                                  const __grid_constant__ Level<float> G,
                                                                  double* partials, DevState* st,
                                                                  cudaGraphConditionalHandle cond, int mode,
                                                                  int use_cond) {
   pdl_enter();
-  norm_mixed_df_body<DIM>(blockIdx.x, gridDim.x, L, K, K64, f64_per8, G, partials, st, cond, mode, use_cond);
+  norm_mixed_df_body<DIM, F64>(blockIdx.x, gridDim.x, L, K, K64, f64_per8, G, partials, st, cond, mode, use_cond);
 }
 
 }  // namespace chhs_dev
