@@ -915,13 +915,24 @@ __device__ __forceinline__ void sum_partials(const double* partials, int nparts,
 // ~0.8 more norms per step and no fewer V-cycles on the benchmark
 // workloads); at least 1, at most max_inner and the V-cycles left under
 // max_v.  Every stop is still decided by a norm of the iterate.
+//
+// The prediction runs in single precision, with log2 of a double taken from
+// its exponent and its leading significand bits: on one thread at the end of
+// a norm, FP64 log, pow and division (each a chain of FP64 instructions of
+// ~64 cycles) took ~8 us per norm, on the critical path of every iteration.
+__device__ __forceinline__ float log2_f64(double x) {  // x > 0, normal
+  const int hi = __double2hiint(x);
+  const float m = __uint_as_float(0x3F800000u | (((unsigned)hi & 0xFFFFFu) << 3) | ((unsigned)__double2loint(x) >> 29));
+  return (float)((hi >> 20) - 1023) + log2f(m);
+}
+
 __device__ __forceinline__ int next_inner(const DevState* st, double r, double rmax) {
   const int cap = min(st->max_inner, st->max_v - st->vcycles);
   if (cap <= 1 || !(st->rho > 0.0 && st->rho < 1.0)) return 1;
-  const double lr = log(st->rho);
-  double need = r > st->tol ? log(st->tol / r) / lr : 0.0;
-  if (rmax > st->tol_max) need = fmax(need, log(st->tol_max / rmax) / lr);
-  return max(1, min(cap, (int)floor(need + 0.5)));
+  const float lr = log2_f64(st->rho), lt = log2_f64(st->tol);
+  float need = r > st->tol ? (lt - log2_f64(r)) / lr : 0.f;
+  if (rmax > st->tol_max) need = fmaxf(need, (log2_f64(st->tol_max) - log2_f64(rmax)) / lr);
+  return max(1, min(cap, (int)floorf(need + 0.5f)));
 }
 
 __device__ __forceinline__ unsigned int loop_decision(DevState* st, double r, double rmax, int mode) {
@@ -943,9 +954,9 @@ __device__ __forceinline__ unsigned int loop_decision(DevState* st, double r, do
       st->checks += 1;
       // contraction per V-cycle over the iteration just finished (kept across
       // steps: the next step's first iteration starts from it)
-      if (st->rprev > 0.0 && r > 0.0 && isfinite(r))
-        st->rho = fmin(fmax(pow(r / st->rprev, 1.0 / ran), 1e-3), 0.9);
-      bool finite = isfinite(r);
+      const bool finite = isfinite(r);
+      if (st->rprev > 0.0 && r > 0.0 && finite)
+        st->rho = (double)fminf(fmaxf(exp2f((log2_f64(r) - log2_f64(st->rprev)) / (float)ran), 1e-3f), 0.9f);
       if (!finite || r > 1e8 * (st->r0 + 1.0)) {
         st->failed = 5;  // CHHS_ERR_DIVERGED
       } else if (above) {
@@ -961,19 +972,25 @@ __device__ __forceinline__ unsigned int loop_decision(DevState* st, double r, do
   return go;
 }
 
+// The larger of two values >= 0, compared as integers: their bits order as
+// the values do, and a comparison of doubles would cost an FP64 instruction.
+__device__ __forceinline__ double max_pos(double a, double b) {
+  return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+
 // Largest of the three rows' residuals at a cell (the pointwise guard).
 __device__ __forceinline__ double row_max(double r1, double r2, double r3s) {
-  return fmax(fmax(fabs(r1), fabs(r2)), fabs(r3s));
+  return max_pos(max_pos(fabs(r1), fabs(r2)), fabs(r3s));
 }
 
 // Block maximum of v (v >= 0); thread 0 returns it.
 __device__ __forceinline__ double block_max(double v) {
   __shared__ double shm[32];
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
+  for (int o = 16; o > 0; o >>= 1) v = max_pos(v, __shfl_down_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, shm[w]);
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = max_pos(v, shm[w]);
   __syncthreads();
   return v;
 }
@@ -987,14 +1004,20 @@ __device__ __forceinline__ void norm_finish(const double* partials, int nparts, 
   for (int b = threadIdx.x; b < nparts; b += blockDim.x) {
     tot[0] += __ldcg(partials + 3 * b);
     tot[1] += __ldcg(partials + 3 * b + 1);
-    mx = fmax(mx, __ldcg(partials + 3 * b + 2));
+    mx = max_pos(mx, __ldcg(partials + 3 * b + 2));
   }
   block_sum<2>(tot);
   mx = block_max(mx);
   if (threadIdx.x != 0) return;
   st->ticket = 0;
-  st->pmean = tot[1] / ncell;
-  unsigned int go = loop_decision(st, sqrt(tot[0] / ncell), mx, mode);
+  // 1/ncell by Newton's iteration from single precision: five FP64
+  // instructions where a division takes ~20
+  const double n = (double)ncell;
+  double inv = (double)(1.0f / (float)ncell);
+  inv = ::fma(inv, ::fma(-n, inv, 1.0), inv);
+  inv = ::fma(inv, ::fma(-n, inv, 1.0), inv);
+  st->pmean = tot[1] * inv;
+  unsigned int go = loop_decision(st, sqrt(tot[0] * inv), mx, mode);
   if (use_cond) {
     cudaGraphSetConditional(cond, go);
     for (int q = 0; q < st->use_if; ++q) cudaGraphSetConditional(st->cond_if[q], st->inner >= 2 + q ? 1u : 0u);
@@ -1030,7 +1053,7 @@ __global__ void __launch_bounds__(kBlock) k_norm(Level<T> L, Coefs<T> K, double*
     acc[0] = fma(r2, r2, acc[0]);
     acc[0] = fma(r3, r3, acc[0]);
     acc[1] += double(L.p[c]);
-    mx = fmax(mx, row_max(r1, r2, r3));
+    mx = max_pos(mx, row_max(r1, r2, r3));
   }
   block_sum<2>(acc);
   mx = block_max(mx);

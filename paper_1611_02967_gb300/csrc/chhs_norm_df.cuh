@@ -177,7 +177,7 @@ struct NdfSums64 {
     acc[0] = ::fma(r1, r1, acc[0]);
     acc[0] = ::fma(r2, r2, acc[0]);
     acc[0] = ::fma(r3s, r3s, acc[0]);
-    mx = fmax(mx, row_max(r1, r2, r3s));
+    mx = max_pos(mx, row_max(r1, r2, r3s));
   }
   __device__ __forceinline__ void finish(double (&out)[3]) {
     block_sum<2>(acc);
