@@ -641,11 +641,31 @@ struct Enqueue {
     frame_coefs(run, s);
   }
 
+  // Mixed form with the finest level above the tail: k_setup_mixed (such a
+  // level coarsens, so its extents are even).
+  static bool setup_mixed(const chhs_t* run) { return mixed(run) && run->tail_start > 0; }
+  static int setup_mixed_blocks(const Level<float>& Gn) { return (Gn.ncell + kSetupBlock - 1) / kSetupBlock; }
+
+  // Single-precision levels whose kernels read stored coefficients: the tail's,
+  // and in 3D those without a pre-smoothing sweep (k_coarse_rhs).  The others
+  // recompute them from phi*.
+  static bool stored_coefs(const chhs_t* run, int l) {
+    return l >= run->tail_start || (DIM == 3 && nu_pre(run, l) == 0);
+  }
+
   static void frame_setup(chhs_t* run, cudaStream_t s) {
     const Level<double>& F = run->lev[0];
     const Coefs<double> K = coefs<double>(run);
     const std::vector<Level<double>>& D = run->lev;
     const int nd = (int)D.size();
+    if (setup_mixed(run)) {
+      const std::vector<Level<float>>& G = run->lev32;
+      launch(run, s, CHHS_K_FRAME, 1.0, [&] {
+        pdl(k_setup_mixed<DIM>, setup_mixed_blocks(G[1]), kSetupBlock, s, F, run->phimm1, run->eps * run->eps, run->st,
+            G[0], G[1]);
+      });
+      return;
+    }
     launch(run, s, CHHS_K_FRAME, 1.0, [&] {
       pdl(k_setup_coef<DIM>, nblocks(F.ncell), kBlock, s, F, run->phimm1, run->eps * run->eps, run->st, K,
           nd > 1 ? D[1] : D[0], nd > 1 ? 1 : 0);
@@ -660,20 +680,21 @@ struct Enqueue {
     for (int l = 1; l < nd; ++l)
       launch(run, s, CHHS_K_FRAME, 1.0, [&] {
         pdl(k_coef_restrict<double, DIM>, nblocks(D[l].ncell), kBlock, s, D[l], K, l + 1 < nd ? D[l + 1] : D[l],
-            l + 1 < nd ? 1 : 0);
+            l + 1 < nd ? 1 : 0, 1);
       });
     if (!mixed(run)) return;
     const std::vector<Level<float>>& G = run->lev32;
     const int ng = (int)G.size();
     const Coefs<float> K32 = coefs<float>(run);
-    launch(run, s, CHHS_K_FRAME, 1.0, [&] {
-      pdl(k_coef_restrict_f32<DIM>, nblocks(F.ncell), kBlock, s, F, G[0], K32, ng > 1 ? G[1] : G[0],
-          ng > 1 ? 1 : 0);
-    });
+    if (!setup_mixed(run))
+      launch(run, s, CHHS_K_FRAME, 1.0, [&] {
+        pdl(k_coef_restrict_f32<DIM>, nblocks(F.ncell), kBlock, s, F, G[0], K32, ng > 1 ? G[1] : G[0],
+            ng > 1 ? 1 : 0);
+      });
     for (int l = 1; l < ng; ++l)
       launch(run, s, CHHS_K_FRAME, 1.0, [&] {
         pdl(k_coef_restrict<float, DIM>, nblocks(G[l].ncell), kBlock, s, G[l], K32, l + 1 < ng ? G[l + 1] : G[l],
-            l + 1 < ng ? 1 : 0);
+            l + 1 < ng ? 1 : 0, stored_coefs(run, l) ? 1 : 0);
       });
   }
 
@@ -1285,6 +1306,13 @@ chhs_status chhs_profile_smooth(chhs_t* run, int npasses, double* ms_per_pass) {
   CU(cudaMemcpyAsync(L.phi0, L.phi, bytes, cudaMemcpyDeviceToDevice, run->stream));
   CU(cudaMemcpyAsync(L.mu0, L.mu, bytes, cudaMemcpyDeviceToDevice, run->stream));
   CU(cudaMemcpyAsync(L.p0, L.p, bytes, cudaMemcpyDeviceToDevice, run->stream));
+  // a mixed-precision step leaves the finest level's double-precision coefficients unset
+  if (run->opts.precision == 1) {
+    if (run->dim == 2)
+      pdl(k_coef_restrict<double, 2>, nblocks(L.ncell), kBlock, run->stream, L, K, L, 0, 1);
+    else
+      pdl(k_coef_restrict<double, 3>, nblocks(L.ncell), kBlock, run->stream, L, K, L, 0, 1);
+  }
   // one untimed pass, then npasses timed ones back to back
   for (int k = 0; k <= npasses; ++k) {
     if (k == 1) CU(cudaEventRecord(ev.a, run->stream));
@@ -1868,10 +1896,17 @@ struct BatchStep {
 
   void setup(cudaStream_t s) {
     JobList<SetupJob> jl;
+    JobList<SetupMixedJob> jm;
     for (chhs_t* r : b->runs) {
       const Level<double>& F = r->lev[0];
+      if (Enqueue<DIM>::setup_mixed(r)) {
+        jm.add(SetupMixedJob{F, r->lev32[0], r->lev32[1], r->phimm1, r->eps * r->eps, r->st},
+               Enqueue<DIM>::setup_mixed_blocks(r->lev32[1]));
+        continue;
+      }
       jl.add(SetupJob{F, F, r->phimm1, r->eps * r->eps, r->st, k64(r), 0}, nblocks(F.ncell));
     }
+    go(CHHS_K_FRAME, jm, kb_setup_mixed<DIM>, kSetupBlock, 0, s);
     go(CHHS_K_FRAME, jl, kb_setup_coef<DIM>, kBlock, 0, s);
   }
 
@@ -1881,6 +1916,7 @@ struct BatchStep {
     for (chhs_t* r : b->runs) {
       const int ng = (int)r->lev32.size();
       maxng = std::max(maxng, ng);
+      if (Enqueue<DIM>::setup_mixed(r)) continue;
       jf.add(CoefF32Job{r->lev[0], r->lev32[0], ng > 1 ? r->lev32[1] : r->lev32[0], k32(r), ng > 1 ? 1 : 0},
              nblocks(r->lev[0].ncell));
     }
@@ -1891,7 +1927,9 @@ struct BatchStep {
         const int ng = (int)r->lev32.size();
         if (l >= ng) continue;
         const Level<float>& G = r->lev32[l];
-        jl.add(CoefJob{G, l + 1 < ng ? r->lev32[l + 1] : G, k32(r), l + 1 < ng ? 1 : 0}, nblocks(G.ncell));
+        jl.add(CoefJob{G, l + 1 < ng ? r->lev32[l + 1] : G, k32(r), l + 1 < ng ? 1 : 0,
+                       Enqueue<DIM>::stored_coefs(r, l) ? 1 : 0},
+               nblocks(G.ncell));
       }
       go(CHHS_K_FRAME, jl, kb_coef_restrict<DIM>, kBlock, 0, s);
     }

@@ -67,6 +67,22 @@ __global__ void __launch_bounds__(kBlock) kb_setup_coef(const SetupJob* jobs, co
   setup_coef_body<DIM>(blockIdx.x - start[j], J.L, J.phimm1, J.eps2, J.st, J.K, J.Cn, J.has_next);
 }
 
+struct SetupMixedJob {
+  Level<double> L;
+  Level<float> G, Gn;
+  const double* phimm1;
+  double eps2;
+  const DevState* st;
+};
+
+template <int DIM>
+__global__ void __launch_bounds__(kSetupBlock) kb_setup_mixed(const SetupMixedJob* jobs, const int* start, int njobs) {
+  pdl_enter();
+  const int j = job_of(start, njobs, blockIdx.x);
+  const SetupMixedJob& J = job_in_smem(jobs, j);
+  setup_mixed_body<DIM>(blockIdx.x - start[j], J.L, J.phimm1, J.eps2, J.st, J.G, J.Gn);
+}
+
 struct CoefF32Job {
   Level<double> F;
   Level<float> G, Gn;
@@ -86,7 +102,7 @@ __global__ void __launch_bounds__(kBlock) kb_coef_restrict_f32(const CoefF32Job*
 struct CoefJob {
   Level<float> L, Cn;
   Coefs<float> K;
-  int has_next;
+  int has_next, full;
 };
 
 template <int DIM>
@@ -94,7 +110,7 @@ __global__ void __launch_bounds__(kBlock) kb_coef_restrict(const CoefJob* jobs, 
   pdl_enter();
   const int j = job_of(start, njobs, blockIdx.x);
   const CoefJob& J = jobs[j];
-  coef_restrict_body<float, DIM>(blockIdx.x - start[j], J.L, J.K, J.Cn, J.has_next);
+  coef_restrict_body<float, DIM>(blockIdx.x - start[j], J.L, J.K, J.Cn, J.has_next, J.full);
 }
 
 struct NormJob {

@@ -28,6 +28,7 @@ namespace chhs_dev {
 
 constexpr int kBlock = 256;        // block size of the plain per-cell kernels
 constexpr int kSmoothBlock = 128;  // block size of the smoother (more, smaller blocks per SM)
+constexpr int kSetupBlock = 128;   // block size of the mixed form's set-up (a thread per coarse cell)
 constexpr int kTailThreads = 512;  // one block runs the coarse tail of a V-cycle
 constexpr int kTailMaxLevels = 12;
 
@@ -357,24 +358,27 @@ __device__ __forceinline__ void restrict_coef_at(const Level<U>& F, const Level<
   C.phis[q] = w * b;
 }
 
-// A level's coefficients, and the restriction of phi^m and phi* to the next
-// level (has_next), in one pass.
+// A level's coefficients (full: the levels whose kernels read them; the
+// others recompute them from phi*), and the restriction of phi^m and phi* to
+// the next level (has_next), in one pass.
 template <typename T, int DIM>
-__device__ __forceinline__ void coef_restrict_body(int bx, Level<T> L, Coefs<T> K, Level<T> Cn, int has_next) {
+__device__ __forceinline__ void coef_restrict_body(int bx, Level<T> L, Coefs<T> K, Level<T> Cn, int has_next,
+                                                   int full) {
   int c = bx * blockDim.x + threadIdx.x;
   if (c >= L.ncell) return;
   int i, j, k;
   cell_ijk(c, L.nx, L.ny, i, j, k);
   auto ps = [&](int e) { return L.phis[e]; };
   auto pm = [&](int e) { return L.phim[e]; };
-  coef_at<T, DIM>(L, K, c, i, j, k, ps, pm(c));
+  if (full) coef_at<T, DIM>(L, K, c, i, j, k, ps, pm(c));
   if (has_next && !(i & 1) && !(j & 1) && (DIM == 2 || !(k & 1))) restrict_coef_at<T, T, DIM>(L, Cn, i, j, k, pm, ps);
 }
 
 template <typename T, int DIM>
-__global__ void __launch_bounds__(kBlock) k_coef_restrict(Level<T> L, Coefs<T> K, Level<T> Cn, int has_next) {
+__global__ void __launch_bounds__(kBlock) k_coef_restrict(Level<T> L, Coefs<T> K, Level<T> Cn, int has_next,
+                                                          int full) {
   pdl_enter();
-  coef_restrict_body<T, DIM>(blockIdx.x, L, K, Cn, has_next);
+  coef_restrict_body<T, DIM>(blockIdx.x, L, K, Cn, has_next, full);
 }
 
 // ---------------------------------------------------------------- smoother
@@ -1166,6 +1170,112 @@ __global__ void __launch_bounds__(kBlock) k_setup_coef(Level<double> L, const do
                                                        int has_next) {
   pdl_enter();
   setup_coef_body<DIM>(blockIdx.x, L, phimm1, eps2, st, K, Cn, has_next);
+}
+
+// The set-up of a mixed-precision step whose finest level is above the tail:
+// phi*, f_mu and the initial guess in double precision (the residual kernel
+// forms the coefficients from phi*, takes f_phi = phi^m and f_p = 0), phi^m
+// and phi* rounded for the finest single-precision level, and their
+// restriction to the next.
+//
+// What bounds it: the FP64 pipe.  k_setup_coef with k_coef_restrict_f32 also
+// wrote 16 double- and 15 single-precision coefficient arrays that no kernel
+// of these levels reads, formed phi* of every neighbour again, and had every
+// warp run the restriction for its few even cells: ~85 FP64 instructions per
+// cell.  Here a thread takes the 2^d children of a coarse cell: phi* once per
+// cell, the differences inside the block once, the rounding and the
+// restriction on the integer and single-precision pipes: ~18.
+// Measured, with the rest of the step unchanged: a 256^3 step 25.8 -> 22.9 ms,
+// three of 128^3 10.8 -> 10.0 ms, two of 2048^2 11.4 -> 10.4 ms.
+//
+// Double to single precision rounded to nearest with integer instructions
+// (ties away from zero), a conversion costing as much as an FP64 FMA;
+// magnitudes below the smallest normal single give 0, beyond its range
+// infinity.
+__device__ __forceinline__ float f64_to_f32_rn(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7FFu) - 896;
+  const unsigned mag = ((unsigned)e << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29) + ((lo >> 28) & 1u);
+  return __uint_as_float((hi & 0x80000000u) | (e <= 0 ? 0u : e >= 255 ? 0x7F800000u : mag));
+}
+
+template <int DIM>
+__device__ __forceinline__ void setup_mixed_body(int bx, const Level<double>& L, const double* phimm1, double eps2,
+                                                 const DevState* st, const Level<float>& G, const Level<float>& Gn) {
+  if (st->failed) return;
+  const int t = bx * blockDim.x + threadIdx.x;
+  if (t >= Gn.ncell) return;
+  int I, J, KK;
+  if (t < (1 << 21)) {
+    cell_ijk_small(t, Gn, I, J, KK);
+  } else {
+    cell_ijk(t, Gn.nx, Gn.ny, I, J, KK);
+  }
+  constexpr int NZ = DIM == 3 ? 2 : 1;
+  const int sy = L.nx, sz = L.nx * L.ny;
+  const int i = 2 * I, c0 = i + sy * 2 * J + (DIM == 3 ? sz * 2 * KK : 0);
+  const bool xm = I > 0, xp = i + 2 < L.nx, ym = J > 0, yp = 2 * J + 2 < L.ny;
+  const bool zm = DIM == 3 && KK > 0, zp = DIM == 3 && 2 * KK + 2 < L.nz;
+  auto ld2 = [](const double* a, int x) { return *reinterpret_cast<const double2*>(a + x); };
+  double2 b[NZ][2];  // phi^{m-1} of the block's x-pairs
+#pragma unroll
+  for (int dk = 0; dk < NZ; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) b[dk][dj] = ld2(phimm1, c0 + dj * sy + dk * sz);
+  const double c34 = 0.25 * eps2 * L.ih2;
+  float a32 = 0.f, b32 = 0.f;
+#pragma unroll
+  for (int dk = 0; dk < NZ; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) {
+      const int c = c0 + dj * sy + dk * sz;
+      const double2 o = b[dk][dj], pm = ld2(L.phim, c);
+      const double dx = o.y - o.x;
+      double lx = dx, ly = -dx;
+      if (xm) lx += phimm1[c - 1] - o.x;
+      if (xp) ly += phimm1[c + 2] - o.y;
+      auto row = [&](bool in, const double2& e) {
+        if (!in) return;
+        lx += e.x - o.x;
+        ly += e.y - o.y;
+      };
+      row(true, b[dk][1 - dj]);
+      if (dj == 0) row(ym, ym ? ld2(phimm1, c - sy) : o);
+      else row(yp, yp ? ld2(phimm1, c + sy) : o);
+      if (DIM == 3) {
+        row(true, b[NZ - 1 - dk][dj]);
+        if (dk == 0) row(zm, zm ? ld2(phimm1, c - sz) : o);
+        else row(zp, zp ? ld2(phimm1, c + sz) : o);
+      }
+      auto fmu = [&](double p, double ps, double lap) {
+        return ::fma(0.25 * p * p, p, -::fma(c34, lap, ps));
+      };
+      const double2 ps = make_double2(1.5 * pm.x - 0.5 * o.x, 1.5 * pm.y - 0.5 * o.y);
+      auto put = [&](double* a, double x, double y) { *reinterpret_cast<double2*>(a + c) = make_double2(x, y); };
+      put(L.phis, ps.x, ps.y);
+      put(L.fmu, fmu(pm.x, ps.x, lx), fmu(pm.y, ps.y, ly));
+      put(L.phi, 2.0 * pm.x - o.x, 2.0 * pm.y - o.y);
+      const float2 pf = make_float2(f64_to_f32_rn(pm.x), f64_to_f32_rn(pm.y));
+      const float2 sf = make_float2(f64_to_f32_rn(ps.x), f64_to_f32_rn(ps.y));
+      *reinterpret_cast<float2*>(G.phim + c) = pf;
+      *reinterpret_cast<float2*>(G.phis + c) = sf;
+      a32 += pf.x;
+      a32 += pf.y;
+      b32 += sf.x;
+      b32 += sf.y;
+    }
+  const float w = DIM == 3 ? 0.125f : 0.25f;
+  Gn.phim[t] = w * a32;
+  Gn.phis[t] = w * b32;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kSetupBlock) k_setup_mixed(const __grid_constant__ Level<double> L,
+                                                             const double* phimm1, double eps2, const DevState* st,
+                                                             const __grid_constant__ Level<float> G,
+                                                             const __grid_constant__ Level<float> Gn) {
+  pdl_enter();
+  setup_mixed_body<DIM>(blockIdx.x, L, phimm1, eps2, st, G, Gn);
 }
 
 // Accept the step: phi^{m-1} <- phi^m, phi^m <- phi^{m+1}, p <- p - mean(p).
