@@ -371,6 +371,64 @@ struct Enqueue {
       }
   }
 
+  // The tile launches of a level's smoothing.  No launch writes what its own
+  // tiles read: each takes the state from one of its two copies (phi, phi2)
+  // and writes the other, the first with a right-hand side to complete (rhs)
+  // writes that to fc.  More than kTileMaxPasses passes take several launches;
+  // the post-smoothing launches end in phi, with a launch of no passes where
+  // their number would not.
+  struct TileStep {
+    Level<float> L;
+    int npass, rhs, prolong, restrict_out;
+    TileOut out;
+  };
+  static int tile_chunks(int npass) { return std::max(1, (npass + kTileMaxPasses - 1) / kTileMaxPasses); }
+  static TileStep tile_step(const Level<float>& L, int from, bool fc, int npass) {
+    TileStep q{L, npass, 0, 0, 0, TileOut{}};
+    if (from) {
+      q.L.phi = L.phi2;
+      q.L.mu = L.mu2;
+      q.L.p = L.p2;
+    }
+    if (fc) {
+      q.L.fphi = L.fc1;
+      q.L.fmu = L.fc2;
+      q.L.fp = L.fc3;
+    }
+    q.out = from ? TileOut{L.phi, L.mu, L.p, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}
+                 : TileOut{L.phi2, L.mu2, L.p2, L.fc1, L.fc2, L.fc3, nullptr, nullptr, nullptr};
+    return q;
+  }
+  static std::vector<TileStep> tile_pre(const Level<float>& L, int npass, bool rhs) {
+    std::vector<TileStep> steps;
+    const int n = tile_chunks(npass);
+    for (int k = 0; k < n; ++k) {
+      TileStep q = tile_step(L, k & 1, rhs && k > 0, std::min(kTileMaxPasses, npass - k * kTileMaxPasses));
+      q.rhs = rhs && k == 0;
+      q.restrict_out = k == n - 1;
+      steps.push_back(q);
+    }
+    return steps;
+  }
+  static std::vector<TileStep> tile_post(const Level<float>& L, int npass_pre, int npass, bool rhs,
+                                         const Level<double>* u) {
+    std::vector<TileStep> steps;
+    const int from = tile_chunks(npass_pre) & 1;
+    int n = tile_chunks(npass);
+    if ((n & 1) != from) ++n;
+    for (int k = 0; k < n; ++k) {
+      TileStep q = tile_step(L, (from + k) & 1, rhs, std::max(0, std::min(kTileMaxPasses, npass - k * kTileMaxPasses)));
+      q.prolong = k == 0;
+      if (u && k == n - 1) {
+        q.out.phi64 = u->phi;
+        q.out.mu64 = u->mu;
+        q.out.p64 = u->p;
+      }
+      steps.push_back(q);
+    }
+    return steps;
+  }
+
   // One FAS V(nu1, nu2)-cycle from level l down, on a hierarchy of either precision.
   template <typename T, bool CORR>
   static void vcycle(chhs_t* run, cudaStream_t s, const std::vector<Level<T>>& lev, const Tail<T>& tail,
@@ -400,38 +458,22 @@ struct Enqueue {
       // restriction in one tiled launch, prolongation + post-smoothing in another
       const bool large = L.ncell >= kLargeTileCells;
       const int tw = large ? run->tile_w : run->stile_w, th = large ? run->tile_h : run->stile_h;
-      const int tt = large ? run->tile_threads : run->stile_threads;
-      const dim3 grid((L.nx + tw - 1) / tw, (L.ny + th - 1) / th);
-      const int nf = tile_nfields<CORR>();
+      const int kind = l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH;
+      auto tiles = [&](const std::vector<TileStep>& steps) {
+        for (const TileStep& q : steps) {
+          const TileShape ts = tile_shape(tw, th, q.npass, q.restrict_out);
+          const dim3 grid((L.nx + ts.tw - 1) / ts.tw, (L.ny + ts.th - 1) / ts.th);
+          launch(run, s, kind, (double)L.ncell * q.npass / 2, [&] {
+            pdl_grid(k_tile, grid, ts.threads(), ts.smem(), s, q.L, C, K, q.npass, q.rhs, q.prolong, q.restrict_out,
+                     q.out, (const int*)nullptr, ts);
+          });
+        }
+      };
       const int np1 = 2 * nu_pre(run, l), np2 = 2 * nu_post(run, l);
-      // the pre-smoothing launch writes the second copy of the state (and the
-      // completed right-hand side), the post-smoothing launch reads them and
-      // writes the state back: no launch writes what its own tiles read
-      const TileOut<T> to_copy{L.phi2, L.mu2, L.p2, L.fc1, L.fc2, L.fc3, nullptr, nullptr, nullptr};
-      Level<T> Lb = L;
-      Lb.phi = L.phi2;
-      Lb.mu = L.mu2;
-      Lb.p = L.p2;
-      if (rhs) {
-        Lb.fphi = L.fc1;
-        Lb.fmu = L.fc2;
-        Lb.fp = L.fc3;
-      }
-      TileOut<T> to_state{L.phi, L.mu, L.p, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-      if (l == 0 && fused_update(run) && run->vc_update) {  // the finished correction goes straight into u
-        to_state.phi64 = run->lev[0].phi;
-        to_state.mu64 = run->lev[0].mu;
-        to_state.p64 = run->lev[0].p;
-      }
-      launch(run, s, l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, (double)L.ncell * nu_pre(run, l), [&] {
-        pdl_grid(k_tile<T, CORR>, grid, tt, tile_smem_bytes(np1 + 1, nf, sizeof(T), tw, th), s, L, C,
-                 K, np1, np1 + 1, rhs ? 1 : 0, 0, 1, to_copy, (const int*)nullptr, tw, th);
-      });
+      tiles(tile_pre(L, np1, rhs));
       vcycle<T, CORR>(run, s, lev, tail, l + 1);
-      launch(run, s, l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, (double)L.ncell * nu_post(run, l), [&] {
-        pdl_grid(k_tile<T, CORR>, grid, tt, tile_smem_bytes(np2, nf, sizeof(T), tw, th), s, Lb, C, K,
-                 np2, np2, 0, 1, 0, to_state, (const int*)nullptr, tw, th);
-      });
+      // the finished correction of the finest level goes straight into u
+      tiles(tile_post(L, np1, np2, rhs, l == 0 && fused_update(run) && run->vc_update ? &run->lev[0] : nullptr));
       return;
     }
     if (rhs && nu_pre(run, l) == 0)
@@ -578,13 +620,13 @@ struct Enqueue {
                   "the grid does not coarsen to a coarsest level small enough for the one-block solve");
     CU(raise_to(ktail, smem));
     if constexpr (use_tiles<T>()) {
+      // the accepted sweep counts: tiles with their halo in nine shared fields
       const int halo = 2 * std::max(std::max(run->opts.nu1, run->opts.nu2), std::max(run->nu1c, run->nu2c)) + 1;
-      const size_t tb = std::max(tile_smem_bytes(halo, tile_nfields<CORR>(), sizeof(T), run->tile_w, run->tile_h),
-                                 tile_smem_bytes(halo, tile_nfields<CORR>(), sizeof(T), run->stile_w, run->stile_h));
-      const void* ktile = reinterpret_cast<const void*>(k_tile<T, CORR>);
-      if (!fits(ktile, tb))
+      if (std::max(tile_limit_bytes(halo, run->tile_w, run->tile_h),
+                   tile_limit_bytes(halo, run->stile_w, run->stile_h)) > (size_t)optin)
         return fail(run, CHHS_ERR_INVALID_ARG, "nu1/nu2 too large for the single-precision tiles");
-      CU(raise_to(ktile, tb));
+      if (std::max(run->tile_threads, run->stile_threads) > kTileThreads)
+        return fail(run, CHHS_ERR_CUDA, "more threads than a tile's block has");
     }
     return CHHS_OK;
   }
@@ -1362,12 +1404,11 @@ chhs_status chhs_profile_smooth32(chhs_t* run, int npasses, double* ms_per_launc
   CU(cudaMemcpyAsync(L.p0, L.p, bytes, cudaMemcpyDeviceToDevice, run->stream));
   const int threads = ((L.nx + 1) / 2) * L.ny * L.nz;
   const int blocks = (threads + kSmoothBlock - 1) / kSmoothBlock;
-  const int np1 = 2 * run->opts.nu1;
-  const TileOut<float> to_copy{L.phi2, L.mu2, L.p2, L.fc1, L.fc2, L.fc3, nullptr, nullptr, nullptr};
   const bool large = L.ncell >= kLargeTileCells;
-  const int tw = large ? run->tile_w : run->stile_w, th = large ? run->tile_h : run->stile_h;
-  const int tt = large ? run->tile_threads : run->stile_threads;
-  const dim3 grid((L.nx + tw - 1) / tw, (L.ny + th - 1) / th);
+  const Enqueue<2>::TileStep q = Enqueue<2>::tile_pre(L, 2 * run->opts.nu1, false)[0];
+  const TileShape T = tile_shape(large ? run->tile_w : run->stile_w, large ? run->tile_h : run->stile_h, q.npass,
+                                 q.restrict_out);
+  const dim3 grid((L.nx + T.tw - 1) / T.tw, (L.ny + T.th - 1) / T.th);
   for (int k = 0; k <= npasses; ++k) {
     if (k == 1) CU(cudaEventRecord(ev.a, run->stream));
     if (run->dim == 3 && Enqueue<3>::quad_level(run, L))
@@ -1376,8 +1417,8 @@ chhs_status chhs_profile_smooth32(chhs_t* run, int npasses, double* ms_per_launc
     else if (run->dim == 3)
       pdl(k_smooth_c<3>, blocks, kSmoothBlock, run->stream, L, C, K, k & 1, 0, 0, Level<double>{});
     else
-      pdl_grid(k_tile<float, true>, grid, tt, tile_smem_bytes(np1 + 1, tile_nfields<true>(), 4, tw, th),
-               run->stream, L, C, K, np1, np1 + 1, 0, 0, 1, to_copy, (const int*)nullptr, tw, th);
+      pdl_grid(k_tile, grid, T.threads(), T.smem(), run->stream, q.L, C, K, q.npass, q.rhs, q.prolong, q.restrict_out,
+               q.out, (const int*)nullptr, T);
   }
   CU(cudaGetLastError());
   CU(cudaEventRecord(ev.b, run->stream));
@@ -1831,7 +1872,7 @@ struct BatchStep {
   std::vector<size_t> offs;         // table offsets in emission order
   size_t cur = 0;
   int* counter = nullptr;           // launches, while capturing
-  size_t tile_smem = 0, tile_smem_big = 0, tail_smem = 0;
+  size_t tail_smem = 0;
 
   size_t put(const void* p, size_t n) {
     const size_t off = align_up(buf.size());
@@ -1970,15 +2011,15 @@ struct BatchStep {
   // constant bank; a batched launch would hold them in registers and
   // re-derive them per block (measured 35-50% slower on 512^2-1024^2 levels).
   // The smaller levels of all runs share one batched launch.
-  static constexpr int kSoloTileBlocks = 128;  // a level of 512 x 256 cells or more
-  void go_tile(int kind, const TileJob<float>& J, int blocks, cudaStream_t s) {
+  static constexpr int kSoloTileCells = 128 * kTileW * kTileH;  // a level of 512 x 128 cells or more
+  void go_tile(int kind, const TileJob& J, cudaStream_t s) {
     if (!capture) return;
     if (counter) ++*counter;
-    const int tw = b->big_tw, th = b->big_th;
-    const dim3 grid((unsigned)((J.L.nx + tw - 1) / tw), (unsigned)((J.L.ny + th - 1) / th));
+    const TileShape T = tile_shape(b->big_tw, b->big_th, J.npass, J.restrict_out);
+    const dim3 grid((unsigned)((J.L.nx + T.tw - 1) / T.tw), (unsigned)((J.L.ny + T.th - 1) / T.th));
     timed(kind, [&] {
-      pdl_grid(k_tile<float, true>, grid, b->big_tt, tile_smem_big, s, J.L, J.C, J.K, J.npass, J.halo, J.rhs,
-               J.prolong, J.restrict_out, J.out, J.gate, tw, th);
+      pdl_grid(k_tile, grid, T.threads(), T.smem(), s, J.L, J.C, J.K, J.npass, J.rhs, J.prolong, J.restrict_out, J.out,
+               J.gate, T);
     }, s);
   }
   // Side streams of the capture: the big per-run tile launches of one phase
@@ -1988,13 +2029,20 @@ struct BatchStep {
   cudaStream_t branch[kBranches] = {};
   cudaEvent_t fork_ev = nullptr, join_ev[kBranches] = {};
 
-  void tiles(int kind, const JobList<TileJob<float>>& all, cudaStream_t s) {
-    JobList<TileJob<float>> small;
+  // A level of each run as the tile job of launch q of its smoothing.
+  void add_tile(JobList<TileJob>& jl, const chhs_t* r, const typename Enqueue<DIM>::TileStep& q, int l) {
+    const TileShape T = tile_shape(kTileW, kTileH, q.npass, q.restrict_out);
+    const int gx = (q.L.nx + T.tw - 1) / T.tw, gy = (q.L.ny + T.th - 1) / T.th;
+    jl.add(TileJob{q.L, r->lev32[l + 1], k32(r), q.out, gate(r), q.npass, q.rhs, q.prolong, q.restrict_out, gx, T}, gx * gy);
+  }
+
+  void tiles(int kind, const JobList<TileJob>& all, cudaStream_t s) {
+    JobList<TileJob> small;
     std::vector<int> big;
     for (int q = 0; q < all.njobs(); ++q) {
-      const int blocks = all.start[q + 1] - all.start[q];
-      if (blocks >= kSoloTileBlocks) big.push_back(q);
-      else small.add(all.jobs[q], blocks);
+      const Level<float>& L = all.jobs[q].L;
+      if (L.ncell >= kSoloTileCells) big.push_back(q);
+      else small.add(all.jobs[q], all.start[q + 1] - all.start[q]);
     }
     const bool fan = capture && branch[0] && big.size() > 1;
     const int nb = fan ? std::min<int>(kBranches, (int)big.size()) : 0;
@@ -2004,9 +2052,12 @@ struct BatchStep {
     }
     for (size_t q = 0; q < big.size(); ++q) {
       const int jq = big[q];
-      go_tile(kind, all.jobs[jq], all.start[jq + 1] - all.start[jq], fan ? branch[q % nb] : s);
+      go_tile(kind, all.jobs[jq], fan ? branch[q % nb] : s);
     }
-    go(kind, small, kb_tile<float, true>, kTileThreads, tile_smem, s);
+    if (!small.jobs.empty()) {
+      const TileShape T = small.jobs[0].T;  // the same passes, so the same shape, for every run
+      go(kind, small, kb_tile, T.threads(), T.smem(), s);
+    }
     if (fan)
       for (int q = 0; q < nb; ++q) {
         cudaEventRecord(join_ev[q], branch[q]);
@@ -2016,17 +2067,13 @@ struct BatchStep {
 
   void pre(cudaStream_t s, int l, int nu1) {
     if (DIM == 2) {
-      JobList<TileJob<float>> jl;
-      const int np1 = 2 * nu1;
-      for (chhs_t* r : b->runs) {
-        if (l >= r->tail_start) continue;
-        const Level<float>& L = r->lev32[l];
-        const TileOut<float> to_copy{L.phi2, L.mu2, L.p2, L.fc1, L.fc2, L.fc3, nullptr, nullptr, nullptr};
-        const int gx = (L.nx + kTileW - 1) / kTileW, gy = (L.ny + kTileH - 1) / kTileH;
-        jl.add(TileJob<float>{L, r->lev32[l + 1], k32(r), to_copy, gate(r), np1, np1 + 1, l > 0 ? 1 : 0, 0, 1, gx},
-               gx * gy);
+      const int n = Enqueue<DIM>::tile_chunks(2 * nu1);
+      for (int k = 0; k < n; ++k) {
+        JobList<TileJob> jl;
+        for (chhs_t* r : b->runs)
+          if (l < r->tail_start) add_tile(jl, r, Enqueue<DIM>::tile_pre(r->lev32[l], 2 * nu1, l > 0)[k], l);
+        tiles(l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, jl, s);
       }
-      tiles(l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, jl, s);
       return;
     }
     auto runs_at = [&](auto add) {
@@ -2060,30 +2107,17 @@ struct BatchStep {
 
   void post(cudaStream_t s, int l, int nu2) {
     if (DIM == 2) {
-      JobList<TileJob<float>> jl;
-      const int np2 = 2 * nu2;
-      for (chhs_t* r : b->runs) {
-        if (l >= r->tail_start) continue;
-        const Level<float>& L = r->lev32[l];
-        Level<float> Lb = L;
-        Lb.phi = L.phi2;
-        Lb.mu = L.mu2;
-        Lb.p = L.p2;
-        if (l > 0) {
-          Lb.fphi = L.fc1;
-          Lb.fmu = L.fc2;
-          Lb.fp = L.fc3;
+      const int np1 = 2 * (l == 0 ? b->opts.nu1 : b->runs[0]->nu1c);
+      const size_t n = Enqueue<DIM>::tile_post(Level<float>{}, np1, 2 * nu2, false, nullptr).size();
+      for (size_t k = 0; k < n; ++k) {
+        JobList<TileJob> jl;
+        for (chhs_t* r : b->runs) {
+          if (l >= r->tail_start) continue;
+          const Level<double>* u = l == 0 && Enqueue<DIM>::fused_update(r) && vk == 1 ? &r->lev[0] : nullptr;
+          add_tile(jl, r, Enqueue<DIM>::tile_post(r->lev32[l], np1, 2 * nu2, l > 0, u)[k], l);
         }
-        TileOut<float> to_state{L.phi, L.mu, L.p, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-        if (l == 0 && Enqueue<DIM>::fused_update(r) && vk == 1) {
-          to_state.phi64 = r->lev[0].phi;
-          to_state.mu64 = r->lev[0].mu;
-          to_state.p64 = r->lev[0].p;
-        }
-        const int gx = (L.nx + kTileW - 1) / kTileW, gy = (L.ny + kTileH - 1) / kTileH;
-        jl.add(TileJob<float>{Lb, r->lev32[l + 1], k32(r), to_state, gate(r), np2, np2, 0, 1, 0, gx}, gx * gy);
+        tiles(l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, jl, s);
       }
-      tiles(l == 0 ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH, jl, s);
       return;
     }
     auto runs_at = [&](auto add) {
@@ -2140,10 +2174,11 @@ struct BatchStep {
     BCU(cudaGetDevice(&dev));
     BCU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     for (chhs_t* r : b->runs) tail_smem = std::max(tail_smem, Enqueue<DIM>::template tail_bytes<float, true>(r->tail32));
-    if (DIM == 2) {
+    if (DIM == 2) {  // the accepted sweep counts and shapes, as Enqueue::prepare_tail
       const int halo = 2 * std::max(std::max(b->opts.nu1, b->opts.nu2), std::max(b->runs[0]->nu1c, b->runs[0]->nu2c)) + 1;
-      tile_smem = tile_smem_bytes(halo, tile_nfields<true>(), sizeof(float));
-      tile_smem_big = tile_smem_bytes(halo, tile_nfields<true>(), sizeof(float), b->big_tw, b->big_th);
+      if (std::max(tile_limit_bytes(halo, kTileW, kTileH), tile_limit_bytes(halo, b->big_tw, b->big_th)) > (size_t)optin)
+        return bfail(b, CHHS_ERR_INVALID_ARG, "a run's coarse tail or tiles need more shared memory than a block has");
+      if (b->big_tt > kTileThreads) return bfail(b, CHHS_ERR_CUDA, "more threads than a tile's block has");
     }
     auto raise_to = [&](const void* fn, size_t dyn) -> chhs_status {
       cudaFuncAttributes fa;
@@ -2156,12 +2191,6 @@ struct BatchStep {
     };
     chhs_status st = raise_to(reinterpret_cast<const void*>(kb_tail<float, DIM, true>), tail_smem);
     if (st != CHHS_OK) return st;
-    if (DIM == 2) {
-      st = raise_to(reinterpret_cast<const void*>(kb_tile<float, true>), tile_smem);
-      if (st != CHHS_OK) return st;
-      st = raise_to(reinterpret_cast<const void*>(k_tile<float, true>), std::max(tile_smem, tile_smem_big));
-      if (st != CHHS_OK) return st;
-    }
     return CHHS_OK;
   }
 

@@ -192,25 +192,24 @@ __global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) kb_norm_mix
   batch_norm_epilogue(jobs, njobs, reports, ticket, cc, any_out);
 }
 
-template <typename T>
 struct TileJob {
-  Level<T> L, C;
-  Coefs<T> K;
-  TileOut<T> out;
+  Level<float> L, C;
+  Coefs<float> K;
+  TileOut out;
   const int* gate;
-  int npass, halo, rhs, prolong, restrict_out;
-  int gx;  // tiles per row of the level
+  int npass, rhs, prolong, restrict_out;
+  int gx;       // tiles per row of the level
+  TileShape T;  // of the batched launch
 };
 
-template <typename T, bool CORR>
-__global__ void __launch_bounds__(kTileThreads, 3) kb_tile(const TileJob<T>* jobs, const int* start, int njobs) {
+static __global__ void __launch_bounds__(kTileThreads) kb_tile(const TileJob* jobs, const int* start, int njobs) {
   pdl_enter();
   const int j = job_of(start, njobs, blockIdx.x);
-  const TileJob<T>& J = job_in_smem(jobs, j);
+  const TileJob& J = job_in_smem(jobs, j);
   if (!gate_open(J.gate)) return;
   const int lb = blockIdx.x - start[j];
   const int by = lb / J.gx, bx = lb - by * J.gx;
-  tile_body<T, CORR>(bx, by, J.L, J.C, J.K, J.npass, J.halo, J.rhs, J.prolong, J.restrict_out, J.out);
+  tile_body(bx, by, J.L, J.C, J.K, J.npass, J.rhs, J.prolong, J.restrict_out, J.out, J.T);
 }
 
 template <typename T>

@@ -1,27 +1,42 @@
-// chhs_tile.cuh -- several smoothing passes fused per shared-memory tile (2D).
+// chhs_tile.cuh -- several smoothing passes fused per tile (2D, single
+// precision, correction form), a thread per 2 x 2 cells.
 //
-// One block loads a tile of kTileW x kTileH cells of a level plus a halo of
-// `halo` cells into shared memory and runs npass red-black colour passes of
-// the smoother there.  Pass k (k = 1..npass) updates the cells of its colour
-// in the tile grown by (halo - k) cells: every neighbour of those cells lies
-// in the region that pass k-1 left exact, so after npass passes the tile
-// grown by (halo - npass) cells holds exactly what npass grid-wide colour
-// passes would give (cells of a colour are updated from the other colour's
-// previous values either way).  The price is the recomputed halo cells; in
-// single precision that is cheaper than the launches and global round trips
-// it removes.
+// One block takes a tile of a level and a halo around it, a thread holds 2 x 2
+// cells of it in registers -- state, right-hand sides, the face values a_f of
+// phi*, the smoother's constants -- and runs npass red-black colour passes.
+// Only (phi, mu, p) of the cells passes through shared memory, so that a pass
+// is: read the four neighbour cells that other threads own, update the two
+// cells of the colour (they only couple to the thread's other two and to those
+// four), store them, block barrier.  Pass k (k = 1 .. npass) leaves the cells
+// within halo - k of the tile exactly as npass grid-wide colour passes would
+// (cells of a colour are updated from the other colour's previous values either
+// way); the cells further out are given up.  The price is the recomputed halo.
 //
 // Optional steps fused around the passes:
 //   prolong  -- on load, u += P(u_c - u_c^0) (the FAS correction from the
-//               next coarser level, piecewise constant);
-//   rhs      -- before the first pass, f += N(u) on the cells that need it,
-//               completing the FAS right-hand side R r + N_c(R u) (the tile's
-//               u still equals R u at that point);
-//   restrict -- after the passes (halo = npass + 1, so the ring around the
-//               tile is exact too), the residual r = f - N(u) on the tile and
-//               its restriction: u_c = u_c^0 = R u, f_c = R r, phi_b,c = R phi_b.
-// The per-step face coefficients are recomputed from phi* in shared memory
-// (cheap in single precision) instead of being read from global memory.
+//               next coarser level, piecewise constant: one value per thread);
+//   rhs      -- before the first pass, f += N(u), completing the FAS
+//               right-hand side R r + N_c(R u) (the tile's u still equals R u);
+//   restrict -- after the passes (one more cell of halo), the residual summed
+//               over the thread's 2 x 2 cells and its mean: u_c = u_c^0 = R u,
+//               f_c = R r, phi_b,c = R phi_b.  The fluxes of the faces inside
+//               the 2 x 2 cells cancel in that sum and are not formed.
+//
+// N is evaluated from face differences (d = neighbour - cell): with w = dp +
+// gamma a dmu and v = dmu + a w (= M dmu + a dp),
+//   N1 = phi - s/h^2 sum v,  N3 = -1/h^2 sum w,  N2 = mu - chi + (3/4) eps^2/h^2 sum dphi.
+// A face on the boundary has the cell itself as its neighbour (a mirrored copy
+// in the shared-memory slot outside the domain), so all its differences vanish.
+//
+// What bounds it: latency -- on small levels the load, the passes' block
+// barriers and the update's dependent chain, on large ones too: 124 registers
+// leave one block of 16 warps per SM, which issues 44 % of the time (ncu,
+// 2048^2: 67 M warp instructions, global loads the largest stall).  Two blocks
+// at 64 or three at 85 registers spill or cut smaller tiles and are slower
+// (2048^2 step 4.77 ms, 5.88 and 5.58).
+// One cell per thread with all fields in shared memory and the coefficients
+// recomputed in every pass took twice the instructions; its 512^2 step 835 us
+// against 683, 640 x 384 1.12 -> 0.94 ms, batch of 24 15.4 -> 14.2 ms.
 //
 // A tile reads its halo from global memory while other tiles of the same
 // launch write their results, so a launch never writes the arrays it reads:
@@ -34,293 +49,348 @@
 
 namespace chhs_dev {
 
-constexpr int kTileW = 32, kTileH = 16;  // default tile interior (even, so restriction stays inside);
-                                         // chhs_autotune may pick 32 x 32 or 64 x 16
-constexpr int kTileThreads = 512;
+constexpr int kTileW = 32, kTileH = 16;  // tile of the batched launches
+constexpr int kTileThreads = 512;        // most threads of a block (2 x 2 cells each, halo included)
+constexpr int kTileMaxPasses = 8;        // more colour passes are split over several launches
 
-template <bool CORR>
-__host__ __device__ constexpr int tile_nfields() { return CORR ? 9 : 8; }
-
-__host__ __device__ inline size_t tile_smem_bytes(int halo, int nfields, size_t elem, int tw = kTileW,
-                                                  int th = kTileH) {
-  return (size_t)(tw + 2 * halo) * (th + 2 * halo) * nfields * elem;
+// Shared memory of the limit on sweep counts (chhs_create): a tile of tw x th
+// with its halo in nine shared fields, the size up to which sweep counts are
+// accepted.
+__host__ __device__ inline size_t tile_limit_bytes(int halo, int tw, int th) {
+  return (size_t)(tw + 2 * halo) * (th + 2 * halo) * 9 * sizeof(float);
 }
 
-// Coefficients of cell (i, j) from phi* in shared memory: face values a_f,
-// M_f for the interior faces, their sums and the smoother's Ae, C/Dn, G
-// (the formulas of k_coef).
-template <typename T>
-struct LocalCoef {
-  T aW, aE, aS, aN, MW, ME, MS, MN;  // zero on boundary faces
-  T sM, sa, Ae, CD, G;
-  int m;
+// A tile launch's shape: interior tw x th (even), halo in 2 x 2 blocks hb,
+// threads bx by by (one per 2 x 2 cells) rounded up to whole warps.
+struct TileShape {
+  int tw, th, hb;
+  __host__ __device__ int bx() const { return tw / 2 + 2 * hb; }
+  __host__ __device__ int by() const { return th / 2 + 2 * hb; }
+  __host__ __device__ int threads() const { return (bx() * by() + 31) / 32 * 32; }
+  __host__ __device__ size_t smem() const { return (size_t)bx() * by() * 4 * sizeof(float4); }
 };
 
-template <typename T>
-__device__ __forceinline__ void local_coef(const T* ps, int s, int SW, int i, int j, int nx, int ny,
-                                           const Level<T>& L, const Coefs<T>& K, LocalCoef<T>& C) {
-  const T pc = ps[s];
-  // branch-free: a missing face reads the cell itself and gets a = M = 0
-  auto face = [&](bool inside, int e, T& a, T& M) {
-    const T af = T(0.5) * (pc + ps[inside ? e : s]);
-    a = inside ? af : T(0);
-    M = inside ? T(1) + K.gamma * af * af : T(0);
-  };
-  face(i > 0, s - 1, C.aW, C.MW);
-  face(i + 1 < nx, s + 1, C.aE, C.ME);
-  face(j > 0, s - SW, C.aS, C.MS);
-  face(j + 1 < ny, s + SW, C.aN, C.MN);
-  C.m = (i > 0) + (i + 1 < nx) + (j > 0) + (j + 1 < ny);
-  C.sM = (C.MW + C.ME) + (C.MS + C.MN);
-  C.sa = (C.aW + C.aE) + (C.aS + C.aN);
-  const T im = inv_count<T>(C.m);
-  C.Ae = L.sih2 * (C.sM - K.gamma * C.sa * C.sa * im);
-  C.CD = K.s * C.sa * im;
-  C.G = K.gamma * L.ih2 * C.sa;
+// The shape for npass passes (and the residual, restrict_out): the asked
+// interior, at least 16 x 16 (512^2 step with 16 x 16 tiles below the finest
+// level 669 us, 16 x 8 683, 8 x 8 698), its longer side halved until the block
+// has room for the halo.  Shapes cut the passes into blocks and change no
+// result.  On the finest level 32 x 32 is best (2048^2: 147 us a launch, 32 x
+// 16 165, 16 x 16 178): its halo makes 1.9 threads per 2 x 2 cells of it
+// against 2.4 and 3.1.
+__host__ __device__ inline TileShape tile_shape(int tw, int th, int npass, int restrict_out) {
+  TileShape s{tw > 16 ? tw : 16, th > 16 ? th : 16, (npass + (restrict_out ? 1 : 0) + 1) / 2};
+  while (s.threads() > kTileThreads && (s.tw > 2 || s.th > 2)) {
+    if (s.tw >= s.th) s.tw = s.tw / 4 * 2 > 2 ? s.tw / 4 * 2 : 2;
+    else s.th = s.th / 4 * 2 > 2 ? s.th / 4 * 2 : 2;
+  }
+  return s;
 }
 
 // Where a tile launch writes its interior: (phi, mu, p) and, with rhs, the
 // completed right-hand side.  On the finest level of the mixed form the
 // post-smoothing launch instead adds the finished correction to the
 // double-precision iterate (phi64, mu64, p64 non-null): u <- u + e.
-template <typename T>
 struct TileOut {
-  T *phi, *mu, *p, *f1, *f2, *f3;
+  float *phi, *mu, *p, *f1, *f2, *f3;
   double *phi64, *mu64, *p64;
 };
 
-// Shared-memory views of one tile's fields.
-template <typename T, bool CORR>
-struct TileView {
-  T *phi, *mu, *p, *phim, *phis, *f1, *f2, *f3, *phib;
+struct TileCell {
+  float phi, mu, p;
 };
 
-// N(u) at shared-memory cell s (global (i, j)).
-template <typename T, bool CORR>
-__device__ __forceinline__ void tile_N(const TileView<T, CORR>& V, int s, int SW, int i, int j, int nx, int ny,
-                                       const Level<T>& L, const Coefs<T>& K, const LocalCoef<T>& C, T& n1, T& n2,
-                                       T& n3) {
-  T Mmu = 0, ap = 0, amu = 0, sphi = 0, sp = 0;
-  // branch-free: a missing face (a = M = 0 from local_coef) reads the cell itself
-  auto face = [&](bool inside, int e, T a, T M) {
-    const int es = inside ? e : s;
-    const T mue = V.mu[es], pe = V.p[es], phie = V.phi[es];
-    Mmu += M * mue;
-    ap += a * pe;
-    amu += a * mue;
-    sphi += inside ? phie : T(0);
-    sp += inside ? pe : T(0);
-  };
-  face(i > 0, s - 1, C.aW, C.MW);
-  face(i + 1 < nx, s + 1, C.aE, C.ME);
-  face(j > 0, s - SW, C.aS, C.MS);
-  face(j + 1 < ny, s + SW, C.aN, C.MN);
-  const T phic = V.phi[s], muc = V.mu[s], pc = V.p[s], pm = V.phim[s], mm = count_value<T>(C.m);
-  T chi_v;
-  if (CORR) {
-    T b = V.phib[s];
-    chi_v = T(0.25) * phic * (T(3) * b * b + T(2) * b * pm + pm * pm + (T(3) * b + pm) * phic + phic * phic);
-  } else {
-    chi_v = chi(phic, pm);
-  }
-  n1 = phic - L.sih2 * ((Mmu - C.sM * muc) + (ap - C.sa * pc));
-  n2 = muc - chi_v + L.e34ih2 * (sphi - mm * phic);
-  n3 = -L.ih2 * ((sp - mm * pc) + K.gamma * (amu - C.sa * muc));
+// Adds the fluxes of the face to neighbour n (coefficient a) of cell c.
+__device__ __forceinline__ void tile_face(const TileCell& c, const TileCell& n, float a, float gamma, float& sv,
+                                          float& sw) {
+  const float dmu = n.mu - c.mu, dp = n.p - c.p;
+  const float w = fmaf(gamma, __fmul_rn(a, dmu), dp);
+  sv += fmaf(a, w, dmu);
+  sw += w;
 }
 
-template <typename T, bool CORR>
-__device__ __forceinline__ void tile_body(int bx, int by, const Level<T>& L, const Level<T>& Cl,
-                                          const Coefs<T>& K, int npass, int halo, int rhs, int prolong,
-                                          int restrict_out, const TileOut<T>& out, int tw = kTileW,
-                                          int th = kTileH) {
-  // The tiles serve the correction-form (single-precision) levels only: the
-  // plain form's right-hand side f_mu carries the shift of cubic_P, which
-  // tile_N does not.
-  static_assert(CORR, "k_tile runs the correction form only");
-  extern __shared__ __align__(16) unsigned char tile_smem[];
-  const int SW = tw + 2 * halo, SH = th + 2 * halo, SN = SW * SH;
-  TileView<T, CORR> V;
-  {
-    T* base = reinterpret_cast<T*>(tile_smem);
-    V.phi = base; V.mu = base + SN; V.p = base + 2 * SN; V.phim = base + 3 * SN; V.phis = base + 4 * SN;
-    V.f1 = base + 5 * SN; V.f2 = base + 6 * SN; V.f3 = base + 7 * SN;
-    V.phib = CORR ? base + 8 * SN : nullptr;
-  }
-  const int nx = L.nx, ny = L.ny;
-  const int tx0 = bx * tw, ty0 = by * th;  // tile origin (global)
-  const int gx0 = tx0 - halo, gy0 = ty0 - halo;                      // shared-memory origin (global)
+// A cell's constants: chi(phi_b + e, phi^m) - chi(phi_b, phi^m) = e (q0 + e (q1 + e/4));
+// x = sum a / n_c, hn = h^2 / n_c, em = (3/4) eps^2 n_c / h^2.
+struct TileConst {
+  float q0, q1, Ae, x, hn, em;
+};
 
-  // load the tile and its halo (cells outside the domain are never read);
-  // thread-to-cell maps use small_div (every index here is below 2^21)
-  const float rSW = __frcp_rn((float)SW);
-  for (int s = threadIdx.x; s < SN; s += blockDim.x) {
-    int sy = small_div(s, rSW), sx = s - sy * SW;
-    int i = gx0 + sx, j = gy0 + sy;
-    if (i < 0 || j < 0 || i >= nx || j >= ny) continue;
-    int c = i + nx * j;
-    T phi = L.phi[c], mu = L.mu[c], p = L.p[c];
+__device__ __forceinline__ float tile_chi(float e, const TileConst& k) {
+  return __fmul_rn(e, fmaf(e, fmaf(0.25f, e, k.q1), k.q0));
+}
+
+// One Newton step of cell c (the update of cell_update: the pressure row
+// eliminated) with neighbours n0..n3 across faces a0..a3.
+__device__ __forceinline__ void tile_update(TileCell& c, const TileCell& n0, const TileCell& n1, const TileCell& n2,
+                                            const TileCell& n3, float a0, float a1, float a2, float a3, float f1,
+                                            float f2, float f3, const TileConst& k, const Level<float>& L,
+                                            const Coefs<float>& K) {
+  float sv = 0.f, sw = 0.f;
+  tile_face(c, n0, a0, K.gamma, sv, sw);
+  tile_face(c, n1, a1, K.gamma, sv, sw);
+  tile_face(c, n2, a2, K.gamma, sv, sw);
+  tile_face(c, n3, a3, K.gamma, sv, sw);
+  const float sd = fmaf(-4.f, c.phi, (n0.phi + n1.phi) + (n2.phi + n3.phi));
+  const float R1 = fmaf(L.sih2, sv, f1 - c.phi);
+  const float R2 = fmaf(-L.e34ih2, sd, (f2 - c.mu) + tile_chi(c.phi, k));
+  const float R3 = fmaf(L.ih2, sw, f3);
+  const float B = fmaf(c.phi, fmaf(0.75f, c.phi, k.q1 + k.q1), k.q0 + k.em);
+  const float num = fmaf(-__fmul_rn(K.s, k.x), R3, fmaf(-k.Ae, R2, R1));
+  const float dphi = __fmul_rn(num, rcp_approx(fmaf(k.Ae, B, 1.f)));
+  const float dmu = fmaf(B, dphi, R2);
+  c.phi += dphi;
+  c.mu += dmu;
+  c.p += fmaf(-__fmul_rn(K.gamma, k.x), dmu, __fmul_rn(k.hn, R3));
+}
+
+__device__ __forceinline__ void tile_body(int bx, int by, const Level<float>& L, const Level<float>& Cl,
+                                          const Coefs<float>& K, int npass, int rhs, int prolong, int restrict_out,
+                                          const TileOut& out, const TileShape& T) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  const int BX = T.bx(), NB = BX * T.by(), t = threadIdx.x;
+  float4* const sA = reinterpret_cast<float4*>(tile_smem);  // cells (0,0) of the 2 x 2 blocks: phi, mu, p, phi*
+  float4* const sB = sA + NB;                               // (1,0)
+  float4* const sC = sB + NB;                               // (0,1)
+  float4* const sD = sC + NB;                               // (1,1)
+  const int ty = small_div(t, __frcp_rn((float)BX)), tx = t - ty * BX;
+  const int hx = L.nx >> 1, hy = L.ny >> 1;                       // 2 x 2 blocks of the level
+  const int I = bx * (T.tw >> 1) - T.hb + tx, J = by * (T.th >> 1) - T.hb + ty;
+  const bool in = t < NB && I >= 0 && J >= 0 && I < hx && J < hy;
+  // distance of the block from the tile, in blocks
+  const int ddx = max(T.hb - tx, tx - (BX - 1 - T.hb)), ddy = max(T.hb - ty, ty - (T.by() - 1 - T.hb));
+  const int dist = max(max(ddx, ddy), 0);
+  const bool inner = in && dist == 0;
+  // neighbour slots (the thread's own at the region's rim, whose cells are given up)
+  const int iW = tx > 0 ? t - 1 : t, iE = tx < BX - 1 ? t + 1 : t;
+  const int iS = ty > 0 ? t - BX : t, iN = ty < T.by() - 1 ? t + BX : t;
+  // boundary faces whose mirrored cell lives in a slot outside the domain
+  const bool eW = in && I == 0, eE = in && I == hx - 1, eS = in && J == 0, eN = in && J == hy - 1;
+  const bool gW = eW && iW != t, gE = eE && iE != t, gS = eS && iS != t, gN = eN && iN != t;
+  const bool ghosts = gW || gE || gS || gN;
+  const int c0 = in ? 2 * I + L.nx * 2 * J : 0, c1 = c0 + L.nx;
+
+  TileCell A{0.f, 0.f, 0.f}, B = A, C = A, D = A;
+  float f1[4], f2[4], f3[4], pm[4], pb[4], ps[4];  // of A, B, C, D
+  auto ld = [&](const float* a, float (&v)[4]) {
+    const float2 lo = *reinterpret_cast<const float2*>(a + c0), hi = *reinterpret_cast<const float2*>(a + c1);
+    v[0] = lo.x;
+    v[1] = lo.y;
+    v[2] = hi.x;
+    v[3] = hi.y;
+  };
+  if (in) {
+    float u[4], v[4], w[4];
+    ld(L.phi, u);
+    ld(L.mu, v);
+    ld(L.p, w);
+    ld(L.phis, ps);
+    ld(L.fphi, f1);
+    ld(L.fmu, f2);
+    ld(L.fp, f3);
+    ld(L.phim, pm);
+    ld(L.phib, pb);
     if (prolong) {
-      int q = (i >> 1) + Cl.nx * (j >> 1);
-      phi += Cl.phi[q] - Cl.phi0[q];
-      mu += Cl.mu[q] - Cl.mu0[q];
-      p += Cl.p[q] - Cl.p0[q];
+      const int q = I + Cl.nx * J;
+      const float dphi = Cl.phi[q] - Cl.phi0[q], dmu = Cl.mu[q] - Cl.mu0[q], dp = Cl.p[q] - Cl.p0[q];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        u[m] += dphi;
+        v[m] += dmu;
+        w[m] += dp;
+      }
     }
-    V.phi[s] = phi;
-    V.mu[s] = mu;
-    V.p[s] = p;
-    V.phim[s] = L.phim[c];
-    V.phis[s] = L.phis[c];
-    V.f1[s] = L.fphi[c];
-    V.f2[s] = L.fmu[c];
-    V.f3[s] = L.fp[c];
-    if (CORR) V.phib[s] = L.phib[c];
+    A = TileCell{u[0], v[0], w[0]};
+    B = TileCell{u[1], v[1], w[1]};
+    C = TileCell{u[2], v[2], w[2]};
+    D = TileCell{u[3], v[3], w[3]};
+  }
+  auto put = [](float4* s, int q, const TileCell& c) {
+    s[q].x = c.phi;
+    s[q].y = c.mu;
+    s[q].z = c.p;
+  };
+  auto get = [](const float4* s, int q) {
+    const float4 v = s[q];
+    return TileCell{v.x, v.y, v.z};
+  };
+  // the mirrored copies of the red (A, D) or black (B, C) cells
+  auto mirror_red = [&]() {
+    if (gW) put(sB, iW, A);
+    if (gS) put(sC, iS, A);
+    if (gE) put(sC, iE, D);
+    if (gN) put(sB, iN, D);
+  };
+  auto mirror_black = [&]() {
+    if (gE) put(sA, iE, B);
+    if (gS) put(sD, iS, B);
+    if (gW) put(sD, iW, C);
+    if (gN) put(sA, iN, C);
+  };
+  if (in) {
+    sA[t] = make_float4(A.phi, A.mu, A.p, ps[0]);
+    sB[t] = make_float4(B.phi, B.mu, B.p, ps[1]);
+    sC[t] = make_float4(C.phi, C.mu, C.p, ps[2]);
+    sD[t] = make_float4(D.phi, D.mu, D.p, ps[3]);
+    if (ghosts) {
+      mirror_red();
+      mirror_black();
+    }
   }
   __syncthreads();
+  // face values a_f: inside the block AB, CD, AC, BD; outside AW, CW, BE, DE, AS, BS, CN, DN
+  float aAB = 0.f, aCD = 0.f, aAC = 0.f, aBD = 0.f, aAW = 0.f, aCW = 0.f, aBE = 0.f, aDE = 0.f, aAS = 0.f, aBS = 0.f,
+        aCN = 0.f, aDN = 0.f;
+  TileConst kA{}, kB{}, kC{}, kD{};
+  if (in) {
+    auto avg = [](float x, float y) { return 0.5f * (x + y); };
+    aAB = avg(ps[0], ps[1]);
+    aCD = avg(ps[2], ps[3]);
+    aAC = avg(ps[0], ps[2]);
+    aBD = avg(ps[1], ps[3]);
+    // zero on boundary faces
+    aAW = eW ? 0.f : avg(ps[0], sB[iW].w);
+    aCW = eW ? 0.f : avg(ps[2], sD[iW].w);
+    aBE = eE ? 0.f : avg(ps[1], sA[iE].w);
+    aDE = eE ? 0.f : avg(ps[3], sC[iE].w);
+    aAS = eS ? 0.f : avg(ps[0], sC[iS].w);
+    aBS = eS ? 0.f : avg(ps[1], sD[iS].w);
+    aCN = eN ? 0.f : avg(ps[2], sA[iN].w);
+    aDN = eN ? 0.f : avg(ps[3], sB[iN].w);
+    auto constants = [&](int m, float a0, float a1, float a2, float a3, int faces) {
+      TileConst k;
+      const float n = (float)faces, im = rcp_approx(n), sa = (a0 + a1) + (a2 + a3);
+      const float sM = fmaf(K.gamma, fmaf(a0, a0, fmaf(a1, a1, fmaf(a2, a2, __fmul_rn(a3, a3)))), n);
+      k.x = __fmul_rn(sa, im);
+      k.Ae = __fmul_rn(L.sih2, fmaf(-__fmul_rn(K.gamma, sa), k.x, sM));
+      k.hn = __fmul_rn(L.h2, im);
+      k.em = __fmul_rn(L.e34ih2, n);
+      k.q0 = __fmul_rn(0.25f, fmaf(pm[m], pm[m], __fmul_rn(pb[m], fmaf(3.f, pb[m], pm[m] + pm[m]))));
+      k.q1 = __fmul_rn(0.25f, fmaf(3.f, pb[m], pm[m]));
+      return k;
+    };
+    const int w = eW ? 0 : 1, e = eE ? 0 : 1, s = eS ? 0 : 1, n = eN ? 0 : 1;
+    kA = constants(0, aAB, aAC, aAW, aAS, 2 + w + s);
+    kB = constants(1, aAB, aBD, aBE, aBS, 2 + e + s);
+    kC = constants(2, aCD, aAC, aCW, aCN, 2 + w + n);
+    kD = constants(3, aCD, aBD, aDE, aDN, 2 + e + n);
+  }
 
-  // the cells of region "tile grown by g" inside the domain: [x0, x1) x [y0, y1)
-  auto region = [&](int g, int& x0, int& x1, int& y0, int& y1) {
-    x0 = max(tx0 - g, 0);
-    x1 = min(tx0 + tw + g, nx);
-    y0 = max(ty0 - g, 0);
-    y1 = min(ty0 + th + g, ny);
+  if (rhs && in) {  // f += N(R u)
+    const TileCell AW = get(sB, iW), CW = get(sD, iW), BE = get(sA, iE), DE = get(sC, iE);
+    const TileCell AS = get(sC, iS), BS = get(sD, iS), CN = get(sA, iN), DN = get(sB, iN);
+    auto add_N = [&](int m, const TileCell& c, const TileCell& n0, const TileCell& n1, const TileCell& n2,
+                     const TileCell& n3, float a0, float a1, float a2, float a3, const TileConst& k) {
+      float sv = 0.f, sw = 0.f;
+      tile_face(c, n0, a0, K.gamma, sv, sw);
+      tile_face(c, n1, a1, K.gamma, sv, sw);
+      tile_face(c, n2, a2, K.gamma, sv, sw);
+      tile_face(c, n3, a3, K.gamma, sv, sw);
+      const float sd = fmaf(-4.f, c.phi, (n0.phi + n1.phi) + (n2.phi + n3.phi));
+      f1[m] += fmaf(-L.sih2, sv, c.phi);
+      f2[m] += fmaf(L.e34ih2, sd, c.mu - tile_chi(c.phi, k));
+      f3[m] = fmaf(-L.ih2, sw, f3[m]);
+    };
+    add_N(0, A, B, C, AW, AS, aAB, aAC, aAW, aAS, kA);
+    add_N(1, B, A, D, BE, BS, aAB, aBD, aBE, aBS, kB);
+    add_N(2, C, D, A, CW, CN, aCD, aAC, aCW, aCN, kC);
+    add_N(3, D, C, B, DE, DN, aCD, aBD, aDE, aDN, kD);
+  }
+  // the pass writes what the right-hand side's threads may still read
+  if (rhs) __syncthreads();
+
+  for (int k = 1; k <= npass; k += 2) {
+    // a block takes part while a cell of it is still needed (within npass - k
+    // of the tile, one more for the residual)
+    const int need = npass - k + (restrict_out ? 1 : 0);
+    if (in && 2 * dist - 1 <= need) {
+      tile_update(A, B, C, get(sB, iW), get(sC, iS), aAB, aAC, aAW, aAS, f1[0], f2[0], f3[0], kA, L, K);
+      tile_update(D, C, B, get(sC, iE), get(sB, iN), aCD, aBD, aDE, aDN, f1[3], f2[3], f3[3], kD, L, K);
+      put(sA, t, A);
+      put(sD, t, D);
+      if (ghosts) mirror_red();
+    }
+    __syncthreads();
+    if (k == npass) break;
+    if (in && 2 * dist - 1 <= need - 1) {
+      tile_update(B, A, D, get(sA, iE), get(sD, iS), aAB, aBD, aBE, aBS, f1[1], f2[1], f3[1], kB, L, K);
+      tile_update(C, D, A, get(sD, iW), get(sA, iN), aCD, aAC, aCW, aCN, f1[2], f2[2], f3[2], kC, L, K);
+      put(sB, t, B);
+      put(sC, t, C);
+      if (ghosts) mirror_black();
+    }
+    __syncthreads();
+  }
+
+  if (!inner) return;
+  auto st = [&](float* a, float x0, float x1, float x2, float x3) {
+    *reinterpret_cast<float2*>(a + c0) = make_float2(x0, x1);
+    *reinterpret_cast<float2*>(a + c1) = make_float2(x2, x3);
   };
-
-  if (rhs) {  // f += N(R u) wherever pass 1 needs f
-    int x0, x1, y0, y1;
-    region(halo - 1, x0, x1, y0, y1);
-    const int w = x1 - x0, total = w * (y1 - y0);
-    const float rw = __frcp_rn((float)w);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int q = small_div(t, rw);
-      int j = y0 + q, i = x0 + (t - q * w);
-      int s = (i - gx0) + SW * (j - gy0);
-      LocalCoef<T> C;
-      local_coef(V.phis, s, SW, i, j, nx, ny, L, K, C);
-      T n1, n2, n3;
-      tile_N<T, CORR>(V, s, SW, i, j, nx, ny, L, K, C, n1, n2, n3);
-      V.f1[s] += n1;
-      V.f2[s] += n2;
-      V.f3[s] += n3;
-    }
-    __syncthreads();
+  if (out.phi64) {
+    auto upd = [&](double* a, float x0, float x1, float x2, float x3) {
+      double2* lo = reinterpret_cast<double2*>(a + c0);
+      double2* hi = reinterpret_cast<double2*>(a + c1);
+      double2 l = *lo, h = *hi;
+      l.x += (double)x0;
+      l.y += (double)x1;
+      h.x += (double)x2;
+      h.y += (double)x3;
+      *lo = l;
+      *hi = h;
+    };
+    upd(out.phi64, A.phi, B.phi, C.phi, D.phi);
+    upd(out.mu64, A.mu, B.mu, C.mu, D.mu);
+    upd(out.p64, A.p, B.p, C.p, D.p);
+  } else {
+    st(out.phi, A.phi, B.phi, C.phi, D.phi);
+    st(out.mu, A.mu, B.mu, C.mu, D.mu);
+    st(out.p, A.p, B.p, C.p, D.p);
   }
-
-  for (int k = 1; k <= npass; ++k) {
-    const int colour = (k - 1) & 1;
-    int x0, x1, y0, y1;
-    region(halo - k, x0, x1, y0, y1);
-    const int hw = (x1 - x0 + 1) >> 1, total = hw * (y1 - y0);
-    const float rhw = __frcp_rn((float)hw);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int q = small_div(t, rhw);
-      int j = y0 + q;
-      int i = x0 + 2 * (t - q * hw);
-      i += (i + j + colour) & 1;
-      if (i >= x1) continue;
-      int s = (i - gx0) + SW * (j - gy0);
-      LocalCoef<T> C;
-      local_coef(V.phis, s, SW, i, j, nx, ny, L, K, C);
-      T n1, n2, n3;
-      tile_N<T, CORR>(V, s, SW, i, j, nx, ny, L, K, C, n1, n2, n3);
-      const T phic = V.phi[s], pm = V.phim[s];
-      T R1 = V.f1[s] - n1, R2 = V.f2[s] - n2, R3 = V.f3[s] - n3;
-      T dchi = CORR ? dchi_da(V.phib[s] + phic, pm) : dchi_da(phic, pm);
-      T B = dchi + L.e34ih2 * count_value<T>(C.m);
-      T dphi = (R1 - C.Ae * R2 - C.CD * R3) * rcp_approx(T(1) + C.Ae * B);
-      T dmu = R2 + B * dphi;
-      T dp = (R3 - C.G * dmu) * (L.h2 * inv_count<T>(C.m));
-      V.phi[s] = phic + dphi;
-      V.mu[s] += dmu;
-      V.p[s] += dp;
-    }
-    __syncthreads();
+  if (rhs) {
+    st(out.f1, f1[0], f1[1], f1[2], f1[3]);
+    st(out.f2, f2[0], f2[1], f2[2], f2[3]);
+    st(out.f3, f3[0], f3[1], f3[2], f3[3]);
   }
-
-  // write the tile back
-  {
-    int x0, x1, y0, y1;
-    region(0, x0, x1, y0, y1);
-    const int w = x1 - x0, total = w * (y1 - y0);
-    const float rw = __frcp_rn((float)w);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int q = small_div(t, rw);
-      int j = y0 + q, i = x0 + (t - q * w);
-      int s = (i - gx0) + SW * (j - gy0), c = i + nx * j;
-      if (out.phi64) {
-        out.phi64[c] += (double)V.phi[s];
-        out.mu64[c] += (double)V.mu[s];
-        out.p64[c] += (double)V.p[s];
-      } else {
-        out.phi[c] = V.phi[s];
-        out.mu[c] = V.mu[s];
-        out.p[c] = V.p[s];
-      }
-      if (rhs) {
-        out.f1[c] = V.f1[s];
-        out.f2[c] = V.f2[s];
-        out.f3[c] = V.f3[s];
-      }
-    }
-  }
-
   if (restrict_out) {
-    // residual on the tile and its restriction: one thread per fine cell,
-    // the four children of a coarse cell in adjacent lanes (child d = t mod 4),
-    // summed by shuffles in a fixed order; the round count is uniform so
-    // every thread takes part in the shuffles
-    constexpr int NV = CORR ? 7 : 6;
-    const int cw = tw / 2, chh = th / 2, total = 4 * cw * chh;
-    for (int r = 0; r < total; r += blockDim.x) {
-      const int t = r + threadIdx.x, qq = t >> 2, d = t & 3;
-      const int I = (tx0 >> 1) + qq % cw, J = (ty0 >> 1) + qq / cw;
-      const bool act = t < total && I < Cl.nx && J < Cl.ny;
-      T v[NV];
-#pragma unroll
-      for (int m = 0; m < NV; ++m) v[m] = T(0);
-      if (act) {
-        const int i = 2 * I + (d & 1), j = 2 * J + (d >> 1);
-        const int s = (i - gx0) + SW * (j - gy0);
-        LocalCoef<T> C;
-        local_coef(V.phis, s, SW, i, j, nx, ny, L, K, C);
-        T n1, n2, n3;
-        tile_N<T, CORR>(V, s, SW, i, j, nx, ny, L, K, C, n1, n2, n3);
-        v[0] = V.f1[s] - n1;
-        v[1] = V.f2[s] - n2;
-        v[2] = V.f3[s] - n3;
-        v[3] = V.phi[s];
-        v[4] = V.mu[s];
-        v[5] = V.p[s];
-        if (CORR) v[NV - 1] = V.phib[s];
-      }
-#pragma unroll
-      for (int o = 1; o < 4; o <<= 1)
-#pragma unroll
-        for (int m = 0; m < NV; ++m) v[m] += __shfl_xor_sync(0xffffffffu, v[m], o);
-      if (act && d == 0) {
-        const int q = I + Cl.nx * J;
-        Cl.fphi[q] = T(0.25) * v[0];
-        Cl.fmu[q] = T(0.25) * v[1];
-        Cl.fp[q] = T(0.25) * v[2];
-        Cl.phi[q] = Cl.phi0[q] = T(0.25) * v[3];
-        Cl.mu[q] = Cl.mu0[q] = T(0.25) * v[4];
-        Cl.p[q] = Cl.p0[q] = T(0.25) * v[5];
-        if (CORR) Cl.phib[q] = T(0.25) * v[NV - 1];
-      }
-    }
+    float sv = 0.f, sw = 0.f;
+    tile_face(A, get(sB, iW), aAW, K.gamma, sv, sw);
+    tile_face(C, get(sD, iW), aCW, K.gamma, sv, sw);
+    tile_face(B, get(sA, iE), aBE, K.gamma, sv, sw);
+    tile_face(D, get(sC, iE), aDE, K.gamma, sv, sw);
+    tile_face(A, get(sC, iS), aAS, K.gamma, sv, sw);
+    tile_face(B, get(sD, iS), aBS, K.gamma, sv, sw);
+    tile_face(C, get(sA, iN), aCN, K.gamma, sv, sw);
+    tile_face(D, get(sB, iN), aDN, K.gamma, sv, sw);
+    const float uphi = (A.phi + B.phi) + (C.phi + D.phi), umu = (A.mu + B.mu) + (C.mu + D.mu);
+    const float up = (A.p + B.p) + (C.p + D.p);
+    // the outer neighbours' differences of phi; those inside cancel
+    const float sd = ((sB[iW].x - A.phi) + (sD[iW].x - C.phi)) + ((sA[iE].x - B.phi) + (sC[iE].x - D.phi)) +
+                     (((sC[iS].x - A.phi) + (sD[iS].x - B.phi)) + ((sA[iN].x - C.phi) + (sB[iN].x - D.phi)));
+    const float r1 = fmaf(L.sih2, sv, ((f1[0] - A.phi) + (f1[1] - B.phi)) + ((f1[2] - C.phi) + (f1[3] - D.phi)));
+    const float m2 = (((f2[0] - A.mu) + tile_chi(A.phi, kA)) + ((f2[1] - B.mu) + tile_chi(B.phi, kB))) +
+                     (((f2[2] - C.mu) + tile_chi(C.phi, kC)) + ((f2[3] - D.mu) + tile_chi(D.phi, kD)));
+    const float r2 = fmaf(-L.e34ih2, sd, m2);
+    const float r3 = fmaf(L.ih2, sw, (f3[0] + f3[1]) + (f3[2] + f3[3]));
+    const int q = I + Cl.nx * J;
+    Cl.fphi[q] = 0.25f * r1;
+    Cl.fmu[q] = 0.25f * r2;
+    Cl.fp[q] = 0.25f * r3;
+    Cl.phi[q] = Cl.phi0[q] = 0.25f * uphi;
+    Cl.mu[q] = Cl.mu0[q] = 0.25f * umu;
+    Cl.p[q] = Cl.p0[q] = 0.25f * up;
+    Cl.phib[q] = 0.25f * ((pb[0] + pb[1]) + (pb[2] + pb[3]));
   }
 }
 
 // gate (nullable): the run's loop flag; the launch does nothing once the
 // run has stopped iterating (a run of a batch that has converged).
-template <typename T, bool CORR>
-__global__ void __launch_bounds__(kTileThreads) k_tile(const __grid_constant__ Level<T> L,
-                                                      const __grid_constant__ Level<T> Cl, Coefs<T> K, int npass,
-                                                      int halo, int rhs, int prolong, int restrict_out,
-                                                      const __grid_constant__ TileOut<T> out, const int* gate,
-                                                      int tw, int th) {
+static __global__ void __launch_bounds__(kTileThreads) k_tile(const __grid_constant__ Level<float> L,
+                                                             const __grid_constant__ Level<float> Cl, Coefs<float> K,
+                                                             int npass, int rhs, int prolong, int restrict_out,
+                                                             const __grid_constant__ TileOut out, const int* gate,
+                                                             TileShape T) {
   pdl_enter();
   if (gate && *(volatile const int*)gate == 0) return;
-  tile_body<T, CORR>(blockIdx.x, blockIdx.y, L, Cl, K, npass, halo, rhs, prolong, restrict_out, out, tw, th);
+  tile_body(blockIdx.x, blockIdx.y, L, Cl, K, npass, rhs, prolong, restrict_out, out, T);
 }
 
 }  // namespace chhs_dev
