@@ -27,6 +27,7 @@
 #include "../../include/chhs.h"
 #include "chhs_kernels.cuh"
 #include "chhs_cluster.cuh"
+#include "chhs_tail2.cuh"
 #include "chhs_tile.cuh"
 #include "chhs_corr3.cuh"
 #include "chhs_norm_df.cuh"

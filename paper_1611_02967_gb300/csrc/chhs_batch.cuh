@@ -15,6 +15,7 @@
 #include "chhs_corr3.cuh"
 #include "chhs_kernels.cuh"
 #include "chhs_norm_df.cuh"
+#include "chhs_tail2.cuh"
 #include "chhs_tile.cuh"
 
 namespace chhs_dev {
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) kb_tail(const TailJob<T>* job
   pdl_enter();
   const TailJob<T>& J = jobs[blockIdx.x];
   if (!gate_open(J.gate)) return;
-  tail_body<T, DIM, CORR>(J.tl, J.K);
+  tail_run<T, DIM, CORR>(J.tl, J.K);
 }
 
 struct SmoothCJob {

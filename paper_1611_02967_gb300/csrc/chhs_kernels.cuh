@@ -1567,17 +1567,13 @@ __host__ __device__ inline size_t tail_smem_bytes(const int* ncell, int n, int c
   return b;
 }
 
-// Level l of the tail with its arrays in shared memory.  Every thread forms
-// the pointers itself from the shared-memory base, so the compiler sees
-// shared-memory accesses (no level table in memory, no generic loads).
+// A level with its arrays in shared memory from `base` on.
 template <typename T, int DIM, bool CORR>
-__device__ __forceinline__ Level<T> tail_level(const Tail<T>& tl, int l, unsigned char* smem) {
-  size_t off = 0;
-  for (int q = 0; q < l; ++q) off += tail_fields<DIM, CORR>() * tail_align(sizeof(T) * tl.lev[q].ncell);
-  Level<T> L = tl.lev[l];
+__device__ __forceinline__ Level<T> tail_carve(const Level<T>& G, unsigned char* base) {
+  Level<T> L = G;
   const size_t st = tail_align(sizeof(T) * L.ncell);
   int q = 0;
-  auto carve = [&]() { return reinterpret_cast<T*>(smem + off + (q++) * st); };
+  auto carve = [&]() { return reinterpret_cast<T*>(base + (q++) * st); };
   L.phi = carve(); L.mu = carve(); L.p = carve();
   L.fphi = carve(); L.fmu = carve(); L.fp = carve();
   L.phim = carve(); L.phi0 = carve(); L.mu0 = carve(); L.p0 = carve();
@@ -1588,6 +1584,16 @@ __device__ __forceinline__ Level<T> tail_level(const Tail<T>& tl, int l, unsigne
   if (CORR) L.phib = carve();
   L.phis = nullptr;
   return L;
+}
+
+// Level l of the tail with its arrays in shared memory.  Every thread forms
+// the pointers itself from the shared-memory base, so the compiler sees
+// shared-memory accesses (no level table in memory, no generic loads).
+template <typename T, int DIM, bool CORR>
+__device__ __forceinline__ Level<T> tail_level(const Tail<T>& tl, int l, unsigned char* smem) {
+  size_t off = 0;
+  for (int q = 0; q < l; ++q) off += tail_fields<DIM, CORR>() * tail_align(sizeof(T) * tl.lev[q].ncell);
+  return tail_carve<T, DIM, CORR>(tl.lev[l], smem + off);
 }
 
 // The coarsest solve of a single-precision correction-form V-cycle carried
@@ -1703,12 +1709,6 @@ __device__ __forceinline__ void tail_body(const Tail<T>& tl, const Coefs<T>& K) 
   copy(G.phi, S.phi, G.ncell);
   copy(G.mu, S.mu, G.ncell);
   copy(G.p, S.p, G.ncell);
-}
-
-template <typename T, int DIM, bool CORR>
-__global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ Tail<T> tl, Coefs<T> K) {
-  pdl_enter();
-  tail_body<T, DIM, CORR>(tl, K);
 }
 
 // ---------------------------------------------------------------- diagnostics

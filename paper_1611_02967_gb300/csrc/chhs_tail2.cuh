@@ -1,0 +1,450 @@
+// chhs_tail2.cuh -- the one-block coarse tail of the 2D single-precision
+// (correction-form) V-cycles, a thread per 2 x 2 cells.
+//
+// The levels of the tail (at most 32 x 32 cells by default, down to the
+// coarsest) are latency: a colour pass of the general tail (tail_smooth) took
+// 700-1000 cycles, most of it index arithmetic, the loads of 25 stored fields
+// and a chain through them.  Here a thread keeps the 2 x 2 cells of a level in
+// registers through all its passes as in chhs_tile.cuh (the same arithmetic):
+// a pass reads four neighbour cells, updates two and stores them.  Levels of
+// at most 32 threads (16 x 16 cells has 64, 8 x 8 has 16) are one warp's, with
+// a warp barrier between passes; the coarsest grid of at most 32 cells is a
+// cell per lane, its neighbours by shuffles.  A larger coarsest grid, and its
+// double-precision solve (coarsest_f64), run on the general tail's code.
+// Measured: FIGURES.
+#pragma once
+#include "chhs_tile.cuh"
+
+namespace chhs_dev {
+
+// Shared memory of a level above the coarsest, nb blocks of 2 x 2 cells:
+// per cell position (phi, mu, p, phi*), the restricted iterate R u, the
+// right-hand sides, phi^m and phi_b.
+struct Tail2Level {
+  float4* s0;  // (phi, mu, p, phi*): position m (of 4) of block q at m nb + q
+  float *u, *fs, *pms, *pbs;  // field k, position m of block q at (4 k + m) nb + q
+  int hx, hy, nb;             // blocks per row, rows, blocks
+  __device__ __forceinline__ float4* s(int m, int q) const { return s0 + m * nb + q; }
+  __device__ __forceinline__ float& u0(int k, int m, int q) const { return u[(4 * k + m) * nb + q]; }
+  __device__ __forceinline__ float& f(int k, int m, int q) const { return fs[(4 * k + m) * nb + q]; }
+  __device__ __forceinline__ float& pm(int m, int q) const { return pms[m * nb + q]; }
+  __device__ __forceinline__ float& pb(int m, int q) const { return pbs[m * nb + q]; }
+};
+
+__host__ __device__ inline size_t tail2_level_bytes(int nb) { return tail_align((size_t)nb * 48 * sizeof(float)); }
+
+__device__ __forceinline__ Tail2Level tail2_level(const Tail<float>& tl, int l, unsigned char* smem) {
+  size_t off = 0;
+  for (int q = 0; q < l; ++q) off += tail2_level_bytes(tl.lev[q].ncell >> 2);
+  Tail2Level T;
+  T.hx = tl.lev[l].nx >> 1;
+  T.hy = tl.lev[l].ny >> 1;
+  T.nb = T.hx * T.hy;
+  float* a = reinterpret_cast<float*>(smem + off);
+  T.s0 = reinterpret_cast<float4*>(a);
+  T.u = a + 16 * T.nb;
+  T.fs = a + 28 * T.nb;
+  T.pms = a + 40 * T.nb;
+  T.pbs = a + 44 * T.nb;
+  return T;
+}
+
+// One thread's 2 x 2 cells of a level: registers and the neighbour cells'
+// places (a cell's own on a boundary face, so its differences vanish).
+struct Tail2Block {
+  TileCell c[4];
+  float f1[4], f2[4], f3[4];
+  TileConst k[4];
+  float a01, a23, a02, a13;                          // faces inside
+  float aw0, aw2, ae1, ae3, as0, as1, an2, an3;      // faces outside, zero on the boundary
+  const float4 *w0, *w2, *e1, *e3, *s0, *s1, *n2, *n3;
+};
+
+__device__ __forceinline__ TileCell tail2_get(const float4* p) {
+  const float4 v = *p;
+  return TileCell{v.x, v.y, v.z};
+}
+__device__ __forceinline__ void tail2_put(float4* p, const TileCell& c) {
+  p->x = c.phi;
+  p->y = c.mu;
+  p->z = c.p;
+}
+
+// Geometry, face values and constants of thread t's block from phi*, phi^m
+// and phi_b in shared memory.
+__device__ __forceinline__ void tail2_setup(Tail2Block& b, const Tail2Level& T, int t, const Level<float>& L,
+                                            const Coefs<float>& K) {
+  const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+  const bool eW = I == 0, eE = I == T.hx - 1, eS = J == 0, eN = J == T.hy - 1;
+  b.w0 = eW ? T.s(0, t) : T.s(1, t) - 1;
+  b.w2 = eW ? T.s(2, t) : T.s(3, t) - 1;
+  b.e1 = eE ? T.s(1, t) : T.s(0, t) + 1;
+  b.e3 = eE ? T.s(3, t) : T.s(2, t) + 1;
+  b.s0 = eS ? T.s(0, t) : T.s(2, t) - T.hx;
+  b.s1 = eS ? T.s(1, t) : T.s(3, t) - T.hx;
+  b.n2 = eN ? T.s(2, t) : T.s(0, t) + T.hx;
+  b.n3 = eN ? T.s(3, t) : T.s(1, t) + T.hx;
+  float ps[4];
+  for (int m = 0; m < 4; ++m) ps[m] = T.s(m, t)->w;
+  auto avg = [](float x, float y) { return 0.5f * (x + y); };
+  b.a01 = avg(ps[0], ps[1]);
+  b.a23 = avg(ps[2], ps[3]);
+  b.a02 = avg(ps[0], ps[2]);
+  b.a13 = avg(ps[1], ps[3]);
+  b.aw0 = eW ? 0.f : avg(ps[0], b.w0->w);
+  b.aw2 = eW ? 0.f : avg(ps[2], b.w2->w);
+  b.ae1 = eE ? 0.f : avg(ps[1], b.e1->w);
+  b.ae3 = eE ? 0.f : avg(ps[3], b.e3->w);
+  b.as0 = eS ? 0.f : avg(ps[0], b.s0->w);
+  b.as1 = eS ? 0.f : avg(ps[1], b.s1->w);
+  b.an2 = eN ? 0.f : avg(ps[2], b.n2->w);
+  b.an3 = eN ? 0.f : avg(ps[3], b.n3->w);
+  const int w = eW ? 0 : 1, e = eE ? 0 : 1, s = eS ? 0 : 1, n = eN ? 0 : 1;
+  b.k[0] = tile_constants(L, K, T.pm(0, t), T.pb(0, t), b.a01, b.a02, b.aw0, b.as0, 2 + w + s);
+  b.k[1] = tile_constants(L, K, T.pm(1, t), T.pb(1, t), b.a01, b.a13, b.ae1, b.as1, 2 + e + s);
+  b.k[2] = tile_constants(L, K, T.pm(2, t), T.pb(2, t), b.a23, b.a02, b.aw2, b.an2, 2 + w + n);
+  b.k[3] = tile_constants(L, K, T.pm(3, t), T.pb(3, t), b.a23, b.a13, b.ae3, b.an3, 2 + e + n);
+}
+
+// The barrier between passes: the block's, or warp 0's on a level of one warp.
+__device__ __forceinline__ void tail2_sync(bool warp) {
+  if (warp) __syncwarp();
+  else __syncthreads();
+}
+
+// npass colour passes (even) of a level; every thread of the block (or of
+// warp 0) calls it, act says whether it holds a block.
+__device__ __forceinline__ void tail2_passes(Tail2Block& b, const Tail2Level& T, int t, bool act, bool warp, int npass,
+                                             const Level<float>& L, const Coefs<float>& K) {
+  for (int k = 0; k < npass; k += 2) {
+    if (act) {
+      tile_update(b.c[0], b.c[1], b.c[2], tail2_get(b.w0), tail2_get(b.s0), b.a01, b.a02, b.aw0, b.as0, b.f1[0],
+                  b.f2[0], b.f3[0], b.k[0], L, K);
+      tile_update(b.c[3], b.c[2], b.c[1], tail2_get(b.e3), tail2_get(b.n3), b.a23, b.a13, b.ae3, b.an3, b.f1[3],
+                  b.f2[3], b.f3[3], b.k[3], L, K);
+      tail2_put(T.s(0, t), b.c[0]);
+      tail2_put(T.s(3, t), b.c[3]);
+    }
+    tail2_sync(warp);
+    if (act) {
+      tile_update(b.c[1], b.c[0], b.c[3], tail2_get(b.e1), tail2_get(b.s1), b.a01, b.a13, b.ae1, b.as1, b.f1[1],
+                  b.f2[1], b.f3[1], b.k[1], L, K);
+      tile_update(b.c[2], b.c[3], b.c[0], tail2_get(b.w2), tail2_get(b.n2), b.a23, b.a02, b.aw2, b.an2, b.f1[2],
+                  b.f2[2], b.f3[2], b.k[2], L, K);
+      tail2_put(T.s(1, t), b.c[1]);
+      tail2_put(T.s(2, t), b.c[2]);
+    }
+    tail2_sync(warp);
+  }
+}
+
+// f += N(R u) of the block's cells (the state is still R u).
+__device__ __forceinline__ void tail2_rhs(Tail2Block& b, const Level<float>& L, const Coefs<float>& K) {
+  tile_add_N(b.f1[0], b.f2[0], b.f3[0], b.c[0], b.c[1], b.c[2], tail2_get(b.w0), tail2_get(b.s0), b.a01, b.a02, b.aw0,
+             b.as0, b.k[0], L, K);
+  tile_add_N(b.f1[1], b.f2[1], b.f3[1], b.c[1], b.c[0], b.c[3], tail2_get(b.e1), tail2_get(b.s1), b.a01, b.a13, b.ae1,
+             b.as1, b.k[1], L, K);
+  tile_add_N(b.f1[2], b.f2[2], b.f3[2], b.c[2], b.c[3], b.c[0], tail2_get(b.w2), tail2_get(b.n2), b.a23, b.a02, b.aw2,
+             b.an2, b.k[2], L, K);
+  tile_add_N(b.f1[3], b.f2[3], b.f3[3], b.c[3], b.c[2], b.c[1], tail2_get(b.e3), tail2_get(b.n3), b.a23, b.a13, b.ae3,
+             b.an3, b.k[3], L, K);
+}
+
+// The coarse cell of the block: its restricted residual, state and phi_b.
+struct Tail2Coarse {
+  TileCell u;
+  float f1, f2, f3, pb;
+};
+
+__device__ __forceinline__ Tail2Coarse tail2_restrict(const Tail2Block& b, const Tail2Level& T, int t,
+                                                      const Level<float>& L, const Coefs<float>& K) {
+  const TileOuter o{tail2_get(b.w0), tail2_get(b.w2), tail2_get(b.e1), tail2_get(b.e3),
+                    tail2_get(b.s0), tail2_get(b.s1), tail2_get(b.n2), tail2_get(b.n3)};
+  Tail2Coarse q;
+  tile_block_residual(b.c[0], b.c[1], b.c[2], b.c[3], o, b.aw0, b.aw2, b.ae1, b.ae3, b.as0, b.as1, b.an2, b.an3, b.f1,
+                      b.f2, b.f3, b.k[0], b.k[1], b.k[2], b.k[3], L, K, q.f1, q.f2, q.f3);
+  q.u = TileCell{0.25f * ((b.c[0].phi + b.c[1].phi) + (b.c[2].phi + b.c[3].phi)),
+                 0.25f * ((b.c[0].mu + b.c[1].mu) + (b.c[2].mu + b.c[3].mu)),
+                 0.25f * ((b.c[0].p + b.c[1].p) + (b.c[2].p + b.c[3].p))};
+  q.pb = 0.25f * ((T.pb(0, t) + T.pb(1, t)) + (T.pb(2, t) + T.pb(3, t)));
+  return q;
+}
+
+// The coarsest grid of at most 32 cells: cell c on lane c, the sweeps and the
+// stopping rule of coarsest_solve.  q: the lane's cell after restriction;
+// returns the correction u - R u.
+__device__ __forceinline__ TileCell tail2_coarsest(const Level<float>& L, const Coefs<float>& K, const Tail2Coarse& q,
+                                                   float ps, float pm, int lane) {
+  const unsigned all = 0xffffffffu;
+  const bool act = lane < L.ncell;
+  const int j = small_div(lane, L.rnx), i = lane - j * L.nx;
+  const bool in0 = act && i > 0, in1 = act && i + 1 < L.nx, in2 = act && j > 0, in3 = act && j + 1 < L.ny;
+  const int l0 = in0 ? lane - 1 : lane, l1 = in1 ? lane + 1 : lane, l2 = in2 ? lane - L.nx : lane,
+            l3 = in3 ? lane + L.nx : lane;
+  const float p0 = __shfl_sync(all, ps, l0), p1 = __shfl_sync(all, ps, l1), p2 = __shfl_sync(all, ps, l2),
+              p3 = __shfl_sync(all, ps, l3);
+  const float a0 = in0 ? 0.5f * (ps + p0) : 0.f, a1 = in1 ? 0.5f * (ps + p1) : 0.f, a2 = in2 ? 0.5f * (ps + p2) : 0.f,
+              a3 = in3 ? 0.5f * (ps + p3) : 0.f;
+  const int faces = max(1, (int)in0 + (int)in1 + (int)in2 + (int)in3);
+  const TileConst k = tile_constants(L, K, pm, q.pb, a0, a1, a2, a3, faces);
+  TileCell u = q.u;
+  float f1 = q.f1, f2 = q.f2, f3 = q.f3;
+  auto from = [&](int l) {
+    return TileCell{__shfl_sync(all, u.phi, l), __shfl_sync(all, u.mu, l), __shfl_sync(all, u.p, l)};
+  };
+  {
+    const TileCell n0 = from(l0), n1 = from(l1), n2 = from(l2), n3 = from(l3);
+    tile_add_N(f1, f2, f3, u, n0, n1, n2, n3, a0, a1, a2, a3, k, L, K);
+  }
+  float acc0 = -1.f, prev = 0.f;
+  for (int it = 0; it <= kCoarsestMaxSweeps; ++it) {
+    float tot = 0.f;
+    {
+      const TileCell n0 = from(l0), n1 = from(l1), n2 = from(l2), n3 = from(l3);
+      float r1 = 0.f, r2 = 0.f, r3 = 0.f;
+      tile_add_N(r1, r2, r3, u, n0, n1, n2, n3, a0, a1, a2, a3, k, L, K);
+      r1 = f1 - r1;
+      r2 = f2 - r2;
+      r3 = K.s * (f3 - r3);
+      tot = act ? r1 * r1 + r2 * r2 + r3 * r3 : 0.f;
+    }
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(all, tot, o);
+    if (acc0 < 0.f) acc0 = tot;
+    if (!(tot > kCoarsestTarget2 * acc0) || tot < 1e-37f) break;
+    if (it >= 8 && tot >= prev) break;
+    prev = tot;
+    for (int colour = 0; colour < 2; ++colour) {
+      const TileCell n0 = from(l0), n1 = from(l1), n2 = from(l2), n3 = from(l3);
+      TileCell v = u;
+      tile_update(v, n0, n1, n2, n3, a0, a1, a2, a3, f1, f2, f3, k, L, K);
+      if (((i + j + colour) & 1) == 0) u = v;
+    }
+  }
+  return TileCell{u.phi - q.u.phi, u.mu - q.u.mu, u.p - q.u.p};
+}
+
+// The tail's levels tl.lev[0 .. n-1], n >= 2: those above the coarsest have
+// even extents and level 0 at most blockDim.x blocks of 2 x 2 cells.
+__device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<float>& K, unsigned char* smem) {
+  const int n = tl.n, t = threadIdx.x, lane = t & 31;
+  const Level<float>& Gc = tl.lev[n - 1];
+  const bool lanes = Gc.ncell <= 32 && !tl.coarsest_f64;  // the coarsest grid on the lanes of warp 0
+  size_t coff = 0;  // the general code's coarsest level behind the others
+  for (int q = 0; q + 1 < n; ++q) coff += tail2_level_bytes(tl.lev[q].ncell >> 2);
+  // the coefficients' sources of every level: phi*, phi^m
+  for (int l = 1; l + 1 < n; ++l) {
+    const Tail2Level T = tail2_level(tl, l, smem);
+    const Level<float>& G = tl.lev[l];
+    for (int c = t; c < G.ncell; c += blockDim.x) {
+      const float ps = G.phis[c], pm = G.phim[c];
+      const int j = small_div(c, G.rnx), i = c - j * G.nx, m = (i & 1) + 2 * (j & 1), q = (i >> 1) + T.hx * (j >> 1);
+      T.s(m, q)->w = ps;
+      T.pm(m, q) = pm;
+    }
+  }
+  float cps = 0.f, cpm = 0.f;
+  if (lanes) {
+    if (t < Gc.ncell) {
+      cps = Gc.phis[t];
+      cpm = Gc.phim[t];
+    }
+  } else {
+    const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
+    for (int c = t; c < Gc.ncell; c += blockDim.x) {
+      S.phim[c] = Gc.phim[c]; S.ax[c] = Gc.ax[c]; S.ay[c] = Gc.ay[c]; S.Mx[c] = Gc.Mx[c]; S.My[c] = Gc.My[c];
+      S.sM[c] = Gc.sM[c]; S.sa[c] = Gc.sa[c]; S.cAe[c] = Gc.cAe[c]; S.cC[c] = Gc.cC[c]; S.cGn[c] = Gc.cGn[c];
+      S.cHn[c] = Gc.cHn[c]; S.cQ[c] = Gc.cQ[c]; S.cH[c] = Gc.cH[c];
+    }
+  }
+  const Level<float>& G0 = tl.lev[0];
+  {
+    const Tail2Level T = tail2_level(tl, 0, smem);
+    if (t < T.nb) {
+      const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+      const int c0 = 2 * I + G0.nx * 2 * J, c1 = c0 + G0.nx;
+      auto ld = [&](const float* a, float (&v)[4]) {
+        const float2 lo = *reinterpret_cast<const float2*>(a + c0), hi = *reinterpret_cast<const float2*>(a + c1);
+        v[0] = lo.x;
+        v[1] = lo.y;
+        v[2] = hi.x;
+        v[3] = hi.y;
+      };
+      float u[4], v[4], w[4], ps[4], f1[4], f2[4], f3[4], pm[4], pb[4];
+      ld(G0.phi, u);
+      ld(G0.mu, v);
+      ld(G0.p, w);
+      ld(G0.phis, ps);
+      ld(G0.fphi, f1);
+      ld(G0.fmu, f2);
+      ld(G0.fp, f3);
+      ld(G0.phim, pm);
+      ld(G0.phib, pb);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        *T.s(m, t) = make_float4(u[m], v[m], w[m], ps[m]);
+        T.f(0, m, t) = f1[m];
+        T.f(1, m, t) = f2[m];
+        T.f(2, m, t) = f3[m];
+        T.pm(m, t) = pm[m];
+        T.pb(m, t) = pb[m];
+      }
+    }
+  }
+  __syncthreads();
+
+  Tail2Block b;
+  TileCell corr{0.f, 0.f, 0.f};  // the next coarser level's correction at the block's coarse cell
+  auto down = [&](int l, bool warp) {
+    const Tail2Level T = tail2_level(tl, l, smem);
+    const Level<float>& L = tl.lev[l];
+    const bool act = t < T.nb;
+    const bool rhs = l > 0 || tl.top_rhs;
+    if (act) {
+      tail2_setup(b, T, t, L, K);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        b.c[m] = tail2_get(T.s(m, t));
+        b.f1[m] = T.f(0, m, t);
+        b.f2[m] = T.f(1, m, t);
+        b.f3[m] = T.f(2, m, t);
+      }
+      if (rhs) {
+        tail2_rhs(b, L, K);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          T.f(0, m, t) = b.f1[m];
+          T.f(1, m, t) = b.f2[m];
+          T.f(2, m, t) = b.f3[m];
+        }
+      }
+    }
+    tail2_sync(warp);
+    tail2_passes(b, T, t, act, warp, 2 * tl.nu1, L, K);
+    Tail2Coarse q{};
+    if (act) q = tail2_restrict(b, T, t, L, K);
+    if (l + 2 < n) {
+      if (act) {
+        const Tail2Level C = tail2_level(tl, l + 1, smem);
+        const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+        const int m = (I & 1) + 2 * (J & 1), x = (I >> 1) + C.hx * (J >> 1);
+        tail2_put(C.s(m, x), q.u);
+        C.u0(0, m, x) = q.u.phi;
+        C.u0(1, m, x) = q.u.mu;
+        C.u0(2, m, x) = q.u.p;
+        C.f(0, m, x) = q.f1;
+        C.f(1, m, x) = q.f2;
+        C.f(2, m, x) = q.f3;
+        C.pb(m, x) = q.pb;
+      }
+    } else if (lanes) {
+      corr = tail2_coarsest(Gc, K, q, cps, cpm, lane);  // warp 0 only: this level has at most 32 blocks
+    } else if (act) {
+      const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
+      S.phi[t] = S.phi0[t] = q.u.phi;
+      S.mu[t] = S.mu0[t] = q.u.mu;
+      S.p[t] = S.p0[t] = q.u.p;
+      S.fphi[t] = q.f1;
+      S.fmu[t] = q.f2;
+      S.fp[t] = q.f3;
+      S.phib[t] = q.pb;
+    }
+  };
+  auto up = [&](int l, bool warp) {
+    const Tail2Level T = tail2_level(tl, l, smem);
+    const Level<float>& L = tl.lev[l];
+    const bool act = t < T.nb;
+    if (act) {
+      TileCell d = corr;
+      if (l + 2 < n) {
+        const Tail2Level C = tail2_level(tl, l + 1, smem);
+        const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+        const int m = (I & 1) + 2 * (J & 1), x = (I >> 1) + C.hx * (J >> 1);
+        const TileCell v = tail2_get(C.s(m, x));
+        d = TileCell{v.phi - C.u0(0, m, x), v.mu - C.u0(1, m, x), v.p - C.u0(2, m, x)};
+      }
+      tail2_setup(b, T, t, L, K);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        b.c[m] = tail2_get(T.s(m, t));
+        b.c[m].phi += d.phi;
+        b.c[m].mu += d.mu;
+        b.c[m].p += d.p;
+        tail2_put(T.s(m, t), b.c[m]);
+        b.f1[m] = T.f(0, m, t);
+        b.f2[m] = T.f(1, m, t);
+        b.f3[m] = T.f(2, m, t);
+      }
+    }
+    tail2_sync(warp);
+    tail2_passes(b, T, t, act, warp, 2 * tl.nu2, L, K);
+  };
+  // the levels of more than 32 blocks on the whole block, the smaller ones on warp 0
+  int small = 0;
+  while (small + 1 < n && (tl.lev[small].ncell >> 2) > 32) ++small;
+  for (int l = 0; l < small; ++l) {
+    down(l, false);
+    __syncthreads();
+  }
+  if (t < 32)
+    for (int l = small; l + 1 < n; ++l) {
+      down(l, true);
+      __syncwarp();
+    }
+  if (!lanes) {
+    __syncthreads();
+    const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
+    tail_rhs<float, 2, true>(S, K);
+    if (tl.coarsest_f64)
+      coarsest_solve_f64<2>(S, K, smem + coff + tail_fields<2, true>() * tail_align(sizeof(float) * Gc.ncell));
+    else
+      coarsest_solve<float, 2, true>(S, K);
+    // level n - 2's block t sits on coarse cell t
+    if (t < Gc.ncell) corr = TileCell{S.phi[t] - S.phi0[t], S.mu[t] - S.mu0[t], S.p[t] - S.p0[t]};
+    __syncthreads();
+  }
+  if (t < 32)
+    for (int l = n - 2; l >= small; --l) {
+      up(l, true);
+      __syncwarp();
+    }
+  __syncthreads();
+  for (int l = small - 1; l >= 0; --l) up(l, false);
+  {
+    const Tail2Level T = tail2_level(tl, 0, smem);
+    if (t < T.nb) {
+      const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+      const int c0 = 2 * I + G0.nx * 2 * J, c1 = c0 + G0.nx;
+      auto st = [&](float* a, float x0, float x1, float x2, float x3) {
+        *reinterpret_cast<float2*>(a + c0) = make_float2(x0, x1);
+        *reinterpret_cast<float2*>(a + c1) = make_float2(x2, x3);
+      };
+      const TileCell A = tail2_get(T.s(0, t)), B = tail2_get(T.s(1, t)), C = tail2_get(T.s(2, t)),
+                     D = tail2_get(T.s(3, t));
+      st(G0.phi, A.phi, B.phi, C.phi, D.phi);
+      st(G0.mu, A.mu, B.mu, C.mu, D.mu);
+      st(G0.p, A.p, B.p, C.p, D.p);
+    }
+  }
+}
+
+// The tail as every launch runs it: 2D single-precision levels as above, unless
+// the coarsest grid is all there is.
+template <typename T, int DIM, bool CORR>
+__device__ __forceinline__ void tail_run(const Tail<T>& tl, const Coefs<T>& K) {
+  if constexpr (DIM == 2 && sizeof(T) == 4 && CORR) {
+    if (tl.n >= 2) {
+      extern __shared__ __align__(16) unsigned char tail_smem[];
+      tail2_body(tl, K, tail_smem);
+      return;
+    }
+  }
+  tail_body<T, DIM, CORR>(tl, K);
+}
+
+template <typename T, int DIM, bool CORR>
+__global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ Tail<T> tl, Coefs<T> K) {
+  pdl_enter();
+  tail_run<T, DIM, CORR>(tl, K);
+}
+
+}  // namespace chhs_dev

@@ -142,6 +142,70 @@ __device__ __forceinline__ void tile_update(TileCell& c, const TileCell& n0, con
   c.p += fmaf(-__fmul_rn(K.gamma, k.x), dmu, __fmul_rn(k.hn, R3));
 }
 
+// The constants of a cell from phi^m, phi_b, its face values and its number of
+// interior faces.
+__device__ __forceinline__ TileConst tile_constants(const Level<float>& L, const Coefs<float>& K, float pm, float pb,
+                                                    float a0, float a1, float a2, float a3, int faces) {
+  TileConst k;
+  const float n = (float)faces, im = rcp_approx(n), sa = (a0 + a1) + (a2 + a3);
+  const float sM = fmaf(K.gamma, fmaf(a0, a0, fmaf(a1, a1, fmaf(a2, a2, __fmul_rn(a3, a3)))), n);
+  k.x = __fmul_rn(sa, im);
+  k.Ae = __fmul_rn(L.sih2, fmaf(-__fmul_rn(K.gamma, sa), k.x, sM));
+  k.hn = __fmul_rn(L.h2, im);
+  k.em = __fmul_rn(L.e34ih2, n);
+  k.q0 = __fmul_rn(0.25f, fmaf(pm, pm, __fmul_rn(pb, fmaf(3.f, pb, pm + pm))));
+  k.q1 = __fmul_rn(0.25f, fmaf(3.f, pb, pm));
+  return k;
+}
+
+// f += N at cell c with neighbours n0..n3.
+__device__ __forceinline__ void tile_add_N(float& f1, float& f2, float& f3, const TileCell& c, const TileCell& n0,
+                                           const TileCell& n1, const TileCell& n2, const TileCell& n3, float a0,
+                                           float a1, float a2, float a3, const TileConst& k, const Level<float>& L,
+                                           const Coefs<float>& K) {
+  float sv = 0.f, sw = 0.f;
+  tile_face(c, n0, a0, K.gamma, sv, sw);
+  tile_face(c, n1, a1, K.gamma, sv, sw);
+  tile_face(c, n2, a2, K.gamma, sv, sw);
+  tile_face(c, n3, a3, K.gamma, sv, sw);
+  const float sd = fmaf(-4.f, c.phi, (n0.phi + n1.phi) + (n2.phi + n3.phi));
+  f1 += fmaf(-L.sih2, sv, c.phi);
+  f2 += fmaf(L.e34ih2, sd, c.mu - tile_chi(c.phi, k));
+  f3 = fmaf(-L.ih2, sw, f3);
+}
+
+// The neighbours outside a block of 2 x 2 cells A, B (row below), C, D.
+struct TileOuter {
+  TileCell w0, w2, e1, e3, s0, s1, n2, n3;
+};
+
+// The mean residual of the block: the fluxes of the faces inside it cancel.
+__device__ __forceinline__ void tile_block_residual(const TileCell& A, const TileCell& B, const TileCell& C,
+                                                    const TileCell& D, const TileOuter& o, float aw0, float aw2,
+                                                    float ae1, float ae3, float as0, float as1, float an2, float an3,
+                                                    const float (&f1)[4], const float (&f2)[4], const float (&f3)[4],
+                                                    const TileConst& kA, const TileConst& kB, const TileConst& kC,
+                                                    const TileConst& kD, const Level<float>& L,
+                                                    const Coefs<float>& K, float& r1, float& r2, float& r3) {
+  float sv = 0.f, sw = 0.f;
+  tile_face(A, o.w0, aw0, K.gamma, sv, sw);
+  tile_face(C, o.w2, aw2, K.gamma, sv, sw);
+  tile_face(B, o.e1, ae1, K.gamma, sv, sw);
+  tile_face(D, o.e3, ae3, K.gamma, sv, sw);
+  tile_face(A, o.s0, as0, K.gamma, sv, sw);
+  tile_face(B, o.s1, as1, K.gamma, sv, sw);
+  tile_face(C, o.n2, an2, K.gamma, sv, sw);
+  tile_face(D, o.n3, an3, K.gamma, sv, sw);
+  const float sd = ((o.w0.phi - A.phi) + (o.w2.phi - C.phi)) + ((o.e1.phi - B.phi) + (o.e3.phi - D.phi)) +
+                   (((o.s0.phi - A.phi) + (o.s1.phi - B.phi)) + ((o.n2.phi - C.phi) + (o.n3.phi - D.phi)));
+  const float m1 = ((f1[0] - A.phi) + (f1[1] - B.phi)) + ((f1[2] - C.phi) + (f1[3] - D.phi));
+  const float m2 = (((f2[0] - A.mu) + tile_chi(A.phi, kA)) + ((f2[1] - B.mu) + tile_chi(B.phi, kB))) +
+                   (((f2[2] - C.mu) + tile_chi(C.phi, kC)) + ((f2[3] - D.mu) + tile_chi(D.phi, kD)));
+  r1 = 0.25f * fmaf(L.sih2, sv, m1);
+  r2 = 0.25f * fmaf(-L.e34ih2, sd, m2);
+  r3 = 0.25f * fmaf(L.ih2, sw, (f3[0] + f3[1]) + (f3[2] + f3[3]));
+}
+
 __device__ __forceinline__ void tile_body(int bx, int by, const Level<float>& L, const Level<float>& Cl,
                                           const Coefs<float>& K, int npass, int rhs, int prolong, int restrict_out,
                                           const TileOut& out, const TileShape& T) {
@@ -255,44 +319,20 @@ __device__ __forceinline__ void tile_body(int bx, int by, const Level<float>& L,
     aBS = eS ? 0.f : avg(ps[1], sD[iS].w);
     aCN = eN ? 0.f : avg(ps[2], sA[iN].w);
     aDN = eN ? 0.f : avg(ps[3], sB[iN].w);
-    auto constants = [&](int m, float a0, float a1, float a2, float a3, int faces) {
-      TileConst k;
-      const float n = (float)faces, im = rcp_approx(n), sa = (a0 + a1) + (a2 + a3);
-      const float sM = fmaf(K.gamma, fmaf(a0, a0, fmaf(a1, a1, fmaf(a2, a2, __fmul_rn(a3, a3)))), n);
-      k.x = __fmul_rn(sa, im);
-      k.Ae = __fmul_rn(L.sih2, fmaf(-__fmul_rn(K.gamma, sa), k.x, sM));
-      k.hn = __fmul_rn(L.h2, im);
-      k.em = __fmul_rn(L.e34ih2, n);
-      k.q0 = __fmul_rn(0.25f, fmaf(pm[m], pm[m], __fmul_rn(pb[m], fmaf(3.f, pb[m], pm[m] + pm[m]))));
-      k.q1 = __fmul_rn(0.25f, fmaf(3.f, pb[m], pm[m]));
-      return k;
-    };
     const int w = eW ? 0 : 1, e = eE ? 0 : 1, s = eS ? 0 : 1, n = eN ? 0 : 1;
-    kA = constants(0, aAB, aAC, aAW, aAS, 2 + w + s);
-    kB = constants(1, aAB, aBD, aBE, aBS, 2 + e + s);
-    kC = constants(2, aCD, aAC, aCW, aCN, 2 + w + n);
-    kD = constants(3, aCD, aBD, aDE, aDN, 2 + e + n);
+    kA = tile_constants(L, K, pm[0], pb[0], aAB, aAC, aAW, aAS, 2 + w + s);
+    kB = tile_constants(L, K, pm[1], pb[1], aAB, aBD, aBE, aBS, 2 + e + s);
+    kC = tile_constants(L, K, pm[2], pb[2], aCD, aAC, aCW, aCN, 2 + w + n);
+    kD = tile_constants(L, K, pm[3], pb[3], aCD, aBD, aDE, aDN, 2 + e + n);
   }
 
   if (rhs && in) {  // f += N(R u)
     const TileCell AW = get(sB, iW), CW = get(sD, iW), BE = get(sA, iE), DE = get(sC, iE);
     const TileCell AS = get(sC, iS), BS = get(sD, iS), CN = get(sA, iN), DN = get(sB, iN);
-    auto add_N = [&](int m, const TileCell& c, const TileCell& n0, const TileCell& n1, const TileCell& n2,
-                     const TileCell& n3, float a0, float a1, float a2, float a3, const TileConst& k) {
-      float sv = 0.f, sw = 0.f;
-      tile_face(c, n0, a0, K.gamma, sv, sw);
-      tile_face(c, n1, a1, K.gamma, sv, sw);
-      tile_face(c, n2, a2, K.gamma, sv, sw);
-      tile_face(c, n3, a3, K.gamma, sv, sw);
-      const float sd = fmaf(-4.f, c.phi, (n0.phi + n1.phi) + (n2.phi + n3.phi));
-      f1[m] += fmaf(-L.sih2, sv, c.phi);
-      f2[m] += fmaf(L.e34ih2, sd, c.mu - tile_chi(c.phi, k));
-      f3[m] = fmaf(-L.ih2, sw, f3[m]);
-    };
-    add_N(0, A, B, C, AW, AS, aAB, aAC, aAW, aAS, kA);
-    add_N(1, B, A, D, BE, BS, aAB, aBD, aBE, aBS, kB);
-    add_N(2, C, D, A, CW, CN, aCD, aAC, aCW, aCN, kC);
-    add_N(3, D, C, B, DE, DN, aCD, aBD, aDE, aDN, kD);
+    tile_add_N(f1[0], f2[0], f3[0], A, B, C, AW, AS, aAB, aAC, aAW, aAS, kA, L, K);
+    tile_add_N(f1[1], f2[1], f3[1], B, A, D, BE, BS, aAB, aBD, aBE, aBS, kB, L, K);
+    tile_add_N(f1[2], f2[2], f3[2], C, D, A, CW, CN, aCD, aAC, aCW, aCN, kC, L, K);
+    tile_add_N(f1[3], f2[3], f3[3], D, C, B, DE, DN, aCD, aBD, aDE, aDN, kD, L, K);
   }
   // the pass writes what the right-hand side's threads may still read
   if (rhs) __syncthreads();
@@ -351,29 +391,16 @@ __device__ __forceinline__ void tile_body(int bx, int by, const Level<float>& L,
     st(out.f3, f3[0], f3[1], f3[2], f3[3]);
   }
   if (restrict_out) {
-    float sv = 0.f, sw = 0.f;
-    tile_face(A, get(sB, iW), aAW, K.gamma, sv, sw);
-    tile_face(C, get(sD, iW), aCW, K.gamma, sv, sw);
-    tile_face(B, get(sA, iE), aBE, K.gamma, sv, sw);
-    tile_face(D, get(sC, iE), aDE, K.gamma, sv, sw);
-    tile_face(A, get(sC, iS), aAS, K.gamma, sv, sw);
-    tile_face(B, get(sD, iS), aBS, K.gamma, sv, sw);
-    tile_face(C, get(sA, iN), aCN, K.gamma, sv, sw);
-    tile_face(D, get(sB, iN), aDN, K.gamma, sv, sw);
+    const TileOuter o{get(sB, iW), get(sD, iW), get(sA, iE), get(sC, iE), get(sC, iS), get(sD, iS), get(sA, iN), get(sB, iN)};
+    float r1, r2, r3;
+    tile_block_residual(A, B, C, D, o, aAW, aCW, aBE, aDE, aAS, aBS, aCN, aDN, f1, f2, f3, kA, kB, kC, kD, L, K, r1, r2,
+                        r3);
     const float uphi = (A.phi + B.phi) + (C.phi + D.phi), umu = (A.mu + B.mu) + (C.mu + D.mu);
     const float up = (A.p + B.p) + (C.p + D.p);
-    // the outer neighbours' differences of phi; those inside cancel
-    const float sd = ((sB[iW].x - A.phi) + (sD[iW].x - C.phi)) + ((sA[iE].x - B.phi) + (sC[iE].x - D.phi)) +
-                     (((sC[iS].x - A.phi) + (sD[iS].x - B.phi)) + ((sA[iN].x - C.phi) + (sB[iN].x - D.phi)));
-    const float r1 = fmaf(L.sih2, sv, ((f1[0] - A.phi) + (f1[1] - B.phi)) + ((f1[2] - C.phi) + (f1[3] - D.phi)));
-    const float m2 = (((f2[0] - A.mu) + tile_chi(A.phi, kA)) + ((f2[1] - B.mu) + tile_chi(B.phi, kB))) +
-                     (((f2[2] - C.mu) + tile_chi(C.phi, kC)) + ((f2[3] - D.mu) + tile_chi(D.phi, kD)));
-    const float r2 = fmaf(-L.e34ih2, sd, m2);
-    const float r3 = fmaf(L.ih2, sw, (f3[0] + f3[1]) + (f3[2] + f3[3]));
     const int q = I + Cl.nx * J;
-    Cl.fphi[q] = 0.25f * r1;
-    Cl.fmu[q] = 0.25f * r2;
-    Cl.fp[q] = 0.25f * r3;
+    Cl.fphi[q] = r1;
+    Cl.fmu[q] = r2;
+    Cl.fp[q] = r3;
     Cl.phi[q] = Cl.phi0[q] = 0.25f * uphi;
     Cl.mu[q] = Cl.mu0[q] = 0.25f * umu;
     Cl.p[q] = Cl.p0[q] = 0.25f * up;
