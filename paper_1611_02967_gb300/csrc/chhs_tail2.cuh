@@ -18,34 +18,48 @@
 namespace chhs_dev {
 
 // Shared memory of a level above the coarsest, nb blocks of 2 x 2 cells:
-// per cell position (phi, mu, p, phi*), the restricted iterate R u, the
-// right-hand sides, phi^m and phi_b.
+// per cell position (phi, mu, p), the restricted iterate R u, the right-hand
+// sides, phi^m, phi_b and q0, q1 of TileConst, and per block the constants that
+// do not depend on the V-cycle (the 12 face values, Ae, x, hn, em per cell).
+constexpr int kTail2Consts = 28;
 struct Tail2Level {
-  float4* s0;  // (phi, mu, p, phi*): position m (of 4) of block q at m nb + q
-  float *u, *fs, *pms, *pbs;  // field k, position m of block q at (4 k + m) nb + q
-  int hx, hy, nb;             // blocks per row, rows, blocks
+  float4* s0;  // (phi, mu, p): position m (of 4) of block q at m nb + q
+  float *u, *fs, *pms, *pbs, *qs, *cs;  // field k, position m of block q at (4 k + m) nb + q
+  int hx, hy, nb;                       // blocks per row, rows, blocks
   __device__ __forceinline__ float4* s(int m, int q) const { return s0 + m * nb + q; }
   __device__ __forceinline__ float& u0(int k, int m, int q) const { return u[(4 * k + m) * nb + q]; }
   __device__ __forceinline__ float& f(int k, int m, int q) const { return fs[(4 * k + m) * nb + q]; }
   __device__ __forceinline__ float& pm(int m, int q) const { return pms[m * nb + q]; }
   __device__ __forceinline__ float& pb(int m, int q) const { return pbs[m * nb + q]; }
+  __device__ __forceinline__ float& q01(int k, int m, int q) const { return qs[(4 * k + m) * nb + q]; }
+  __device__ __forceinline__ float& con(int k, int q) const { return cs[k * nb + q]; }
 };
 
-__host__ __device__ inline size_t tail2_level_bytes(int nb) { return tail_align((size_t)nb * 48 * sizeof(float)); }
+__host__ __device__ inline size_t tail2_level_bytes(int nb) {
+  return tail_align((size_t)nb * (16 + 12 + 12 + 4 + 4 + 8 + kTail2Consts) * sizeof(float));
+}
 
-__device__ __forceinline__ Tail2Level tail2_level(const Tail<float>& tl, int l, unsigned char* smem) {
-  size_t off = 0;
-  for (int q = 0; q < l; ++q) off += tail2_level_bytes(tl.lev[q].ncell >> 2);
+// A level's scalars, copied to shared memory once: read with a level index
+// that is not known at compile time, the kernel's parameters come through
+// constant-cache misses (~1 500 cycles per level visit, measured).
+struct Tail2Scalars {
+  float ih2, h2, sih2, e34ih2, rhx;
+  int hx, hy, nb, off;
+};
+
+__device__ __forceinline__ Tail2Level tail2_level(const Tail2Scalars& L, unsigned char* smem) {
   Tail2Level T;
-  T.hx = tl.lev[l].nx >> 1;
-  T.hy = tl.lev[l].ny >> 1;
-  T.nb = T.hx * T.hy;
-  float* a = reinterpret_cast<float*>(smem + off);
+  T.hx = L.hx;
+  T.hy = L.hy;
+  T.nb = L.nb;
+  float* a = reinterpret_cast<float*>(smem + L.off);
   T.s0 = reinterpret_cast<float4*>(a);
   T.u = a + 16 * T.nb;
   T.fs = a + 28 * T.nb;
   T.pms = a + 40 * T.nb;
   T.pbs = a + 44 * T.nb;
+  T.qs = a + 48 * T.nb;
+  T.cs = a + 56 * T.nb;
   return T;
 }
 
@@ -64,17 +78,51 @@ __device__ __forceinline__ TileCell tail2_get(const float4* p) {
   const float4 v = *p;
   return TileCell{v.x, v.y, v.z};
 }
-__device__ __forceinline__ void tail2_put(float4* p, const TileCell& c) {
-  p->x = c.phi;
-  p->y = c.mu;
-  p->z = c.p;
+__device__ __forceinline__ void tail2_put(float4* p, const TileCell& c) { *p = make_float4(c.phi, c.mu, c.p, 0.f); }
+
+// The constants of block q of level L (global phi*, phi^m) into shared memory.
+__device__ __forceinline__ void tail2_constants(const Tail2Level& T, int q, const Level<float>& L,
+                                                const Tail2Scalars& S, const Coefs<float>& K) {
+  const int J = small_div(q, S.rhx), I = q - J * T.hx;
+  const bool eW = I == 0, eE = I == T.hx - 1, eS = J == 0, eN = J == T.hy - 1;
+  const int nx = L.nx, c = 2 * I + nx * 2 * J;
+  const float p0 = L.phis[c], p1 = L.phis[c + 1], p2 = L.phis[c + nx], p3 = L.phis[c + nx + 1];
+  const float w0 = L.phis[eW ? c : c - 1], w2 = L.phis[eW ? c : c + nx - 1];
+  const float e1 = L.phis[eE ? c : c + 2], e3 = L.phis[eE ? c : c + nx + 2];
+  const float s0 = L.phis[eS ? c : c - nx], s1 = L.phis[eS ? c : c - nx + 1];
+  const float n2 = L.phis[eN ? c : c + 2 * nx], n3 = L.phis[eN ? c : c + 2 * nx + 1];
+  const float m0 = L.phim[c], m1 = L.phim[c + 1], m2 = L.phim[c + nx], m3 = L.phim[c + nx + 1];
+  auto avg = [](float x, float y) { return 0.5f * (x + y); };
+  const float a01 = avg(p0, p1), a23 = avg(p2, p3), a02 = avg(p0, p2), a13 = avg(p1, p3);
+  const float aw0 = eW ? 0.f : avg(p0, w0), aw2 = eW ? 0.f : avg(p2, w2);
+  const float ae1 = eE ? 0.f : avg(p1, e1), ae3 = eE ? 0.f : avg(p3, e3);
+  const float as0 = eS ? 0.f : avg(p0, s0), as1 = eS ? 0.f : avg(p1, s1);
+  const float an2 = eN ? 0.f : avg(p2, n2), an3 = eN ? 0.f : avg(p3, n3);
+  const float a[12] = {a01, a23, a02, a13, aw0, aw2, ae1, ae3, as0, as1, an2, an3};
+#pragma unroll
+  for (int k = 0; k < 12; ++k) T.con(k, q) = a[k];
+  const int w = eW ? 0 : 1, e = eE ? 0 : 1, s = eS ? 0 : 1, n = eN ? 0 : 1;
+  auto put = [&](int m, const TileConst& k) {
+    T.con(12 + m, q) = k.Ae;
+    T.con(16 + m, q) = k.x;
+    T.con(20 + m, q) = k.hn;
+    T.con(24 + m, q) = k.em;
+  };
+  put(0, tile_constants(S, K, 0.f, 0.f, a01, a02, aw0, as0, 2 + w + s));
+  put(1, tile_constants(S, K, 0.f, 0.f, a01, a13, ae1, as1, 2 + e + s));
+  put(2, tile_constants(S, K, 0.f, 0.f, a23, a02, aw2, an2, 2 + w + n));
+  put(3, tile_constants(S, K, 0.f, 0.f, a23, a13, ae3, an3, 2 + e + n));
+  T.pm(0, q) = m0;
+  T.pm(1, q) = m1;
+  T.pm(2, q) = m2;
+  T.pm(3, q) = m3;
 }
 
-// Geometry, face values and constants of thread t's block from phi*, phi^m
-// and phi_b in shared memory.
-__device__ __forceinline__ void tail2_setup(Tail2Block& b, const Tail2Level& T, int t, const Level<float>& L,
-                                            const Coefs<float>& K) {
-  const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+// Thread t's block into registers: the neighbour cells' places, the constants,
+// the state and the right-hand side.  On the way down (first) q0 and q1 are
+// formed from phi_b and kept for the way up.
+__device__ __forceinline__ void tail2_setup(Tail2Block& b, const Tail2Level& T, int t, float rhx, bool first) {
+  const int J = small_div(t, rhx), I = t - J * T.hx;
   const bool eW = I == 0, eE = I == T.hx - 1, eS = J == 0, eN = J == T.hy - 1;
   b.w0 = eW ? T.s(0, t) : T.s(1, t) - 1;
   b.w2 = eW ? T.s(2, t) : T.s(3, t) - 1;
@@ -84,26 +132,28 @@ __device__ __forceinline__ void tail2_setup(Tail2Block& b, const Tail2Level& T, 
   b.s1 = eS ? T.s(1, t) : T.s(3, t) - T.hx;
   b.n2 = eN ? T.s(2, t) : T.s(0, t) + T.hx;
   b.n3 = eN ? T.s(3, t) : T.s(1, t) + T.hx;
-  float ps[4];
-  for (int m = 0; m < 4; ++m) ps[m] = T.s(m, t)->w;
-  auto avg = [](float x, float y) { return 0.5f * (x + y); };
-  b.a01 = avg(ps[0], ps[1]);
-  b.a23 = avg(ps[2], ps[3]);
-  b.a02 = avg(ps[0], ps[2]);
-  b.a13 = avg(ps[1], ps[3]);
-  b.aw0 = eW ? 0.f : avg(ps[0], b.w0->w);
-  b.aw2 = eW ? 0.f : avg(ps[2], b.w2->w);
-  b.ae1 = eE ? 0.f : avg(ps[1], b.e1->w);
-  b.ae3 = eE ? 0.f : avg(ps[3], b.e3->w);
-  b.as0 = eS ? 0.f : avg(ps[0], b.s0->w);
-  b.as1 = eS ? 0.f : avg(ps[1], b.s1->w);
-  b.an2 = eN ? 0.f : avg(ps[2], b.n2->w);
-  b.an3 = eN ? 0.f : avg(ps[3], b.n3->w);
-  const int w = eW ? 0 : 1, e = eE ? 0 : 1, s = eS ? 0 : 1, n = eN ? 0 : 1;
-  b.k[0] = tile_constants(L, K, T.pm(0, t), T.pb(0, t), b.a01, b.a02, b.aw0, b.as0, 2 + w + s);
-  b.k[1] = tile_constants(L, K, T.pm(1, t), T.pb(1, t), b.a01, b.a13, b.ae1, b.as1, 2 + e + s);
-  b.k[2] = tile_constants(L, K, T.pm(2, t), T.pb(2, t), b.a23, b.a02, b.aw2, b.an2, 2 + w + n);
-  b.k[3] = tile_constants(L, K, T.pm(3, t), T.pb(3, t), b.a23, b.a13, b.ae3, b.an3, 2 + e + n);
+  float* const a[12] = {&b.a01, &b.a23, &b.a02, &b.a13, &b.aw0, &b.aw2, &b.ae1, &b.ae3, &b.as0, &b.as1, &b.an2, &b.an3};
+#pragma unroll
+  for (int k = 0; k < 12; ++k) *a[k] = T.con(k, t);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    b.k[m].Ae = T.con(12 + m, t);
+    b.k[m].x = T.con(16 + m, t);
+    b.k[m].hn = T.con(20 + m, t);
+    b.k[m].em = T.con(24 + m, t);
+    b.c[m] = tail2_get(T.s(m, t));
+    b.f1[m] = T.f(0, m, t);
+    b.f2[m] = T.f(1, m, t);
+    b.f3[m] = T.f(2, m, t);
+    if (first) {
+      tile_quad(b.k[m], T.pm(m, t), T.pb(m, t));
+      T.q01(0, m, t) = b.k[m].q0;
+      T.q01(1, m, t) = b.k[m].q1;
+    } else {
+      b.k[m].q0 = T.q01(0, m, t);
+      b.k[m].q1 = T.q01(1, m, t);
+    }
+  }
 }
 
 // The barrier between passes: the block's, or warp 0's on a level of one warp.
@@ -115,7 +165,7 @@ __device__ __forceinline__ void tail2_sync(bool warp) {
 // npass colour passes (even) of a level; every thread of the block (or of
 // warp 0) calls it, act says whether it holds a block.
 __device__ __forceinline__ void tail2_passes(Tail2Block& b, const Tail2Level& T, int t, bool act, bool warp, int npass,
-                                             const Level<float>& L, const Coefs<float>& K) {
+                                             const Tail2Scalars& L, const Coefs<float>& K) {
   for (int k = 0; k < npass; k += 2) {
     if (act) {
       tile_update(b.c[0], b.c[1], b.c[2], tail2_get(b.w0), tail2_get(b.s0), b.a01, b.a02, b.aw0, b.as0, b.f1[0],
@@ -139,7 +189,7 @@ __device__ __forceinline__ void tail2_passes(Tail2Block& b, const Tail2Level& T,
 }
 
 // f += N(R u) of the block's cells (the state is still R u).
-__device__ __forceinline__ void tail2_rhs(Tail2Block& b, const Level<float>& L, const Coefs<float>& K) {
+__device__ __forceinline__ void tail2_rhs(Tail2Block& b, const Tail2Scalars& L, const Coefs<float>& K) {
   tile_add_N(b.f1[0], b.f2[0], b.f3[0], b.c[0], b.c[1], b.c[2], tail2_get(b.w0), tail2_get(b.s0), b.a01, b.a02, b.aw0,
              b.as0, b.k[0], L, K);
   tile_add_N(b.f1[1], b.f2[1], b.f3[1], b.c[1], b.c[0], b.c[3], tail2_get(b.e1), tail2_get(b.s1), b.a01, b.a13, b.ae1,
@@ -157,7 +207,7 @@ struct Tail2Coarse {
 };
 
 __device__ __forceinline__ Tail2Coarse tail2_restrict(const Tail2Block& b, const Tail2Level& T, int t,
-                                                      const Level<float>& L, const Coefs<float>& K) {
+                                                      const Tail2Scalars& L, const Coefs<float>& K) {
   const TileOuter o{tail2_get(b.w0), tail2_get(b.w2), tail2_get(b.e1), tail2_get(b.e3),
                     tail2_get(b.s0), tail2_get(b.s1), tail2_get(b.n2), tail2_get(b.n3)};
   Tail2Coarse q;
@@ -229,18 +279,38 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   const int n = tl.n, t = threadIdx.x, lane = t & 31;
   const Level<float>& Gc = tl.lev[n - 1];
   const bool lanes = Gc.ncell <= 32 && !tl.coarsest_f64;  // the coarsest grid on the lanes of warp 0
-  size_t coff = 0;  // the general code's coarsest level behind the others
-  for (int q = 0; q + 1 < n; ++q) coff += tail2_level_bytes(tl.lev[q].ncell >> 2);
-  // the coefficients' sources of every level: phi*, phi^m
-  for (int l = 1; l + 1 < n; ++l) {
-    const Tail2Level T = tail2_level(tl, l, smem);
-    const Level<float>& G = tl.lev[l];
-    for (int c = t; c < G.ncell; c += blockDim.x) {
-      const float ps = G.phis[c], pm = G.phim[c];
-      const int j = small_div(c, G.rnx), i = c - j * G.nx, m = (i & 1) + 2 * (j & 1), q = (i >> 1) + T.hx * (j >> 1);
-      T.s(m, q)->w = ps;
-      T.pm(m, q) = pm;
-    }
+  __shared__ Tail2Scalars sc[kTailMaxLevels];  // of the levels above the coarsest; [n - 1].off: their end
+  if (t < n) {
+    const Level<float>& G = tl.lev[t];
+    size_t off = 0;
+    for (int q = 0; q < t; ++q) off += tail2_level_bytes(tl.lev[q].ncell >> 2);
+    const int hx = G.nx >> 1;
+    sc[t] = Tail2Scalars{G.ih2, G.h2, G.sih2, G.e34ih2, __frcp_rn((float)max(hx, 1)), hx, G.ny >> 1, G.ncell >> 2, (int)off};
+  }
+  __syncthreads();
+  const int coff = sc[n - 1].off;  // the general code's coarsest level
+  // the top level's state, right-hand sides and phi_b (the loads come first;
+  // the constants of all levels are formed while they are on the way)
+  const Level<float>& G0 = tl.lev[0];
+  const Tail2Level T0 = tail2_level(sc[0], smem);
+  float u[4], v[4], w[4], g1[4], g2[4], g3[4], pb[4];
+  if (t < T0.nb) {
+    const int J = small_div(t, sc[0].rhx), I = t - J * T0.hx;
+    const int c0 = 2 * I + G0.nx * 2 * J, c1 = c0 + G0.nx;
+    auto ld = [&](const float* a, float (&x)[4]) {
+      const float2 lo = *reinterpret_cast<const float2*>(a + c0), hi = *reinterpret_cast<const float2*>(a + c1);
+      x[0] = lo.x;
+      x[1] = lo.y;
+      x[2] = hi.x;
+      x[3] = hi.y;
+    };
+    ld(G0.phi, u);
+    ld(G0.mu, v);
+    ld(G0.p, w);
+    ld(G0.fphi, g1);
+    ld(G0.fmu, g2);
+    ld(G0.fp, g3);
+    ld(G0.phib, pb);
   }
   float cps = 0.f, cpm = 0.f;
   if (lanes) {
@@ -256,38 +326,23 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
       S.cHn[c] = Gc.cHn[c]; S.cQ[c] = Gc.cQ[c]; S.cH[c] = Gc.cH[c];
     }
   }
-  const Level<float>& G0 = tl.lev[0];
-  {
-    const Tail2Level T = tail2_level(tl, 0, smem);
-    if (t < T.nb) {
-      const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
-      const int c0 = 2 * I + G0.nx * 2 * J, c1 = c0 + G0.nx;
-      auto ld = [&](const float* a, float (&v)[4]) {
-        const float2 lo = *reinterpret_cast<const float2*>(a + c0), hi = *reinterpret_cast<const float2*>(a + c1);
-        v[0] = lo.x;
-        v[1] = lo.y;
-        v[2] = hi.x;
-        v[3] = hi.y;
-      };
-      float u[4], v[4], w[4], ps[4], f1[4], f2[4], f3[4], pm[4], pb[4];
-      ld(G0.phi, u);
-      ld(G0.mu, v);
-      ld(G0.p, w);
-      ld(G0.phis, ps);
-      ld(G0.fphi, f1);
-      ld(G0.fmu, f2);
-      ld(G0.fp, f3);
-      ld(G0.phim, pm);
-      ld(G0.phib, pb);
+  // every level's blocks in one sequence over the threads, so that the small
+  // levels' are other warps' work
+  int total = 0;
+  for (int l = 0; l + 1 < n; ++l) total += sc[l].nb;
+  for (int e = t; e < total; e += blockDim.x) {
+    int l = 0, q = e;
+    while (q >= sc[l].nb) q -= sc[l++].nb;
+    tail2_constants(tail2_level(sc[l], smem), q, tl.lev[l], sc[l], K);
+  }
+  if (t < T0.nb) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        *T.s(m, t) = make_float4(u[m], v[m], w[m], ps[m]);
-        T.f(0, m, t) = f1[m];
-        T.f(1, m, t) = f2[m];
-        T.f(2, m, t) = f3[m];
-        T.pm(m, t) = pm[m];
-        T.pb(m, t) = pb[m];
-      }
+    for (int m = 0; m < 4; ++m) {
+      *T0.s(m, t) = make_float4(u[m], v[m], w[m], 0.f);
+      T0.f(0, m, t) = g1[m];
+      T0.f(1, m, t) = g2[m];
+      T0.f(2, m, t) = g3[m];
+      T0.pb(m, t) = pb[m];
     }
   }
   __syncthreads();
@@ -295,19 +350,12 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   Tail2Block b;
   TileCell corr{0.f, 0.f, 0.f};  // the next coarser level's correction at the block's coarse cell
   auto down = [&](int l, bool warp) {
-    const Tail2Level T = tail2_level(tl, l, smem);
-    const Level<float>& L = tl.lev[l];
+    const Tail2Scalars L = sc[l];
+    const Tail2Level T = tail2_level(L, smem);
     const bool act = t < T.nb;
     const bool rhs = l > 0 || tl.top_rhs;
     if (act) {
-      tail2_setup(b, T, t, L, K);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        b.c[m] = tail2_get(T.s(m, t));
-        b.f1[m] = T.f(0, m, t);
-        b.f2[m] = T.f(1, m, t);
-        b.f3[m] = T.f(2, m, t);
-      }
+      tail2_setup(b, T, t, L.rhx, true);
       if (rhs) {
         tail2_rhs(b, L, K);
 #pragma unroll
@@ -324,8 +372,8 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
     if (act) q = tail2_restrict(b, T, t, L, K);
     if (l + 2 < n) {
       if (act) {
-        const Tail2Level C = tail2_level(tl, l + 1, smem);
-        const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+        const Tail2Level C = tail2_level(sc[l + 1], smem);
+        const int J = small_div(t, L.rhx), I = t - J * T.hx;
         const int m = (I & 1) + 2 * (J & 1), x = (I >> 1) + C.hx * (J >> 1);
         tail2_put(C.s(m, x), q.u);
         C.u0(0, m, x) = q.u.phi;
@@ -350,29 +398,25 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
     }
   };
   auto up = [&](int l, bool warp) {
-    const Tail2Level T = tail2_level(tl, l, smem);
-    const Level<float>& L = tl.lev[l];
+    const Tail2Scalars L = sc[l];
+    const Tail2Level T = tail2_level(L, smem);
     const bool act = t < T.nb;
     if (act) {
       TileCell d = corr;
       if (l + 2 < n) {
-        const Tail2Level C = tail2_level(tl, l + 1, smem);
-        const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+        const Tail2Level C = tail2_level(sc[l + 1], smem);
+        const int J = small_div(t, L.rhx), I = t - J * T.hx;
         const int m = (I & 1) + 2 * (J & 1), x = (I >> 1) + C.hx * (J >> 1);
         const TileCell v = tail2_get(C.s(m, x));
         d = TileCell{v.phi - C.u0(0, m, x), v.mu - C.u0(1, m, x), v.p - C.u0(2, m, x)};
       }
-      tail2_setup(b, T, t, L, K);
+      tail2_setup(b, T, t, L.rhx, false);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        b.c[m] = tail2_get(T.s(m, t));
         b.c[m].phi += d.phi;
         b.c[m].mu += d.mu;
         b.c[m].p += d.p;
         tail2_put(T.s(m, t), b.c[m]);
-        b.f1[m] = T.f(0, m, t);
-        b.f2[m] = T.f(1, m, t);
-        b.f3[m] = T.f(2, m, t);
       }
     }
     tail2_sync(warp);
@@ -380,16 +424,13 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   };
   // the levels of more than 32 blocks on the whole block, the smaller ones on warp 0
   int small = 0;
-  while (small + 1 < n && (tl.lev[small].ncell >> 2) > 32) ++small;
-  for (int l = 0; l < small; ++l) {
-    down(l, false);
-    __syncthreads();
+  while (small + 1 < n && sc[small].nb > 32) ++small;
+  // (one call each way: a copy per barrier kind would double the code, and the
+  // instructions of a level's first visit come through cache misses)
+  for (int l = 0; l + 1 < n && (l < small || t < 32); ++l) {
+    down(l, l >= small);
+    tail2_sync(l >= small);
   }
-  if (t < 32)
-    for (int l = small; l + 1 < n; ++l) {
-      down(l, true);
-      __syncwarp();
-    }
   if (!lanes) {
     __syncthreads();
     const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
@@ -402,17 +443,19 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
     if (t < Gc.ncell) corr = TileCell{S.phi[t] - S.phi0[t], S.mu[t] - S.mu0[t], S.p[t] - S.p0[t]};
     __syncthreads();
   }
-  if (t < 32)
-    for (int l = n - 2; l >= small; --l) {
-      up(l, true);
-      __syncwarp();
+  for (int l = n - 2; l >= 0; --l) {
+    if (l >= small) {
+      if (t >= 32) continue;
+    } else if (l == small - 1) {
+      __syncthreads();  // warp 0's levels are done
     }
-  __syncthreads();
-  for (int l = small - 1; l >= 0; --l) up(l, false);
+    up(l, l >= small);
+    tail2_sync(l >= small);
+  }
   {
-    const Tail2Level T = tail2_level(tl, 0, smem);
+    const Tail2Level T = T0;
     if (t < T.nb) {
-      const int J = small_div(t, __frcp_rn((float)T.hx)), I = t - J * T.hx;
+      const int J = small_div(t, sc[0].rhx), I = t - J * T.hx;
       const int c0 = 2 * I + G0.nx * 2 * J, c1 = c0 + G0.nx;
       auto st = [&](float* a, float x0, float x1, float x2, float x3) {
         *reinterpret_cast<float2*>(a + c0) = make_float2(x0, x1);

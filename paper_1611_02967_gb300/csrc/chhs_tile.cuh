@@ -108,6 +108,8 @@ __device__ __forceinline__ void tile_face(const TileCell& c, const TileCell& n, 
   sw += w;
 }
 
+// (LV: a Level<float>, or another struct with its scalars ih2, h2, sih2, e34ih2.)
+//
 // A cell's constants: chi(phi_b + e, phi^m) - chi(phi_b, phi^m) = e (q0 + e (q1 + e/4));
 // x = sum a / n_c, hn = h^2 / n_c, em = (3/4) eps^2 n_c / h^2.
 struct TileConst {
@@ -120,9 +122,10 @@ __device__ __forceinline__ float tile_chi(float e, const TileConst& k) {
 
 // One Newton step of cell c (the update of cell_update: the pressure row
 // eliminated) with neighbours n0..n3 across faces a0..a3.
+template <class LV>
 __device__ __forceinline__ void tile_update(TileCell& c, const TileCell& n0, const TileCell& n1, const TileCell& n2,
                                             const TileCell& n3, float a0, float a1, float a2, float a3, float f1,
-                                            float f2, float f3, const TileConst& k, const Level<float>& L,
+                                            float f2, float f3, const TileConst& k, const LV& L,
                                             const Coefs<float>& K) {
   float sv = 0.f, sw = 0.f;
   tile_face(c, n0, a0, K.gamma, sv, sw);
@@ -142,9 +145,15 @@ __device__ __forceinline__ void tile_update(TileCell& c, const TileCell& n0, con
   c.p += fmaf(-__fmul_rn(K.gamma, k.x), dmu, __fmul_rn(k.hn, R3));
 }
 
+__device__ __forceinline__ void tile_quad(TileConst& k, float pm, float pb) {
+  k.q0 = __fmul_rn(0.25f, fmaf(pm, pm, __fmul_rn(pb, fmaf(3.f, pb, pm + pm))));
+  k.q1 = __fmul_rn(0.25f, fmaf(3.f, pb, pm));
+}
+
 // The constants of a cell from phi^m, phi_b, its face values and its number of
 // interior faces.
-__device__ __forceinline__ TileConst tile_constants(const Level<float>& L, const Coefs<float>& K, float pm, float pb,
+template <class LV>
+__device__ __forceinline__ TileConst tile_constants(const LV& L, const Coefs<float>& K, float pm, float pb,
                                                     float a0, float a1, float a2, float a3, int faces) {
   TileConst k;
   const float n = (float)faces, im = rcp_approx(n), sa = (a0 + a1) + (a2 + a3);
@@ -153,15 +162,15 @@ __device__ __forceinline__ TileConst tile_constants(const Level<float>& L, const
   k.Ae = __fmul_rn(L.sih2, fmaf(-__fmul_rn(K.gamma, sa), k.x, sM));
   k.hn = __fmul_rn(L.h2, im);
   k.em = __fmul_rn(L.e34ih2, n);
-  k.q0 = __fmul_rn(0.25f, fmaf(pm, pm, __fmul_rn(pb, fmaf(3.f, pb, pm + pm))));
-  k.q1 = __fmul_rn(0.25f, fmaf(3.f, pb, pm));
+  tile_quad(k, pm, pb);
   return k;
 }
 
 // f += N at cell c with neighbours n0..n3.
+template <class LV>
 __device__ __forceinline__ void tile_add_N(float& f1, float& f2, float& f3, const TileCell& c, const TileCell& n0,
                                            const TileCell& n1, const TileCell& n2, const TileCell& n3, float a0,
-                                           float a1, float a2, float a3, const TileConst& k, const Level<float>& L,
+                                           float a1, float a2, float a3, const TileConst& k, const LV& L,
                                            const Coefs<float>& K) {
   float sv = 0.f, sw = 0.f;
   tile_face(c, n0, a0, K.gamma, sv, sw);
@@ -180,12 +189,13 @@ struct TileOuter {
 };
 
 // The mean residual of the block: the fluxes of the faces inside it cancel.
+template <class LV>
 __device__ __forceinline__ void tile_block_residual(const TileCell& A, const TileCell& B, const TileCell& C,
                                                     const TileCell& D, const TileOuter& o, float aw0, float aw2,
                                                     float ae1, float ae3, float as0, float as1, float an2, float an3,
                                                     const float (&f1)[4], const float (&f2)[4], const float (&f3)[4],
                                                     const TileConst& kA, const TileConst& kB, const TileConst& kC,
-                                                    const TileConst& kD, const Level<float>& L,
+                                                    const TileConst& kD, const LV& L,
                                                     const Coefs<float>& K, float& r1, float& r2, float& r3) {
   float sv = 0.f, sw = 0.f;
   tile_face(A, o.w0, aw0, K.gamma, sv, sw);
