@@ -25,49 +25,13 @@
 
 namespace chhs_dev {
 
-// Face data of cell c recomputed from phi*: neighbour index per face (c
-// itself where the face is missing, so that every load is in bounds), a_f
-// and M_f (zero on missing faces), their sums and the interior-face count.
-template <int DIM>
-struct FacesC {
-  int e[2 * DIM];
-  float a[2 * DIM], M[2 * DIM];
-  float sM, sa;
-  int m;
-  unsigned in;  // bit q: face q is interior
-};
-
-template <int DIM>
-__device__ __forceinline__ void faces_c(const Level<float>& L, const Coefs<float>& K, int c, int i, int j, int k,
-                                        FacesC<DIM>& F) {
-  const int sy = L.nx, sz = L.nx * L.ny;
-  const bool in[6] = {i > 0, i + 1 < L.nx, j > 0, j + 1 < L.ny, k > 0, k + 1 < L.nz};
-  const int off[6] = {-1, 1, -sy, sy, -sz, sz};
-  const float pc = L.phis[c];
-  F.sM = -0.f;
-  F.sa = -0.f;
-  F.m = 0;
-  F.in = 0u;
-#pragma unroll
-  for (int q = 0; q < 2 * DIM; ++q) {
-    const int e = in[q] ? c + off[q] : c;
-    const float af = 0.5f * (pc + L.phis[e]);
-    F.e[q] = e;
-    F.a[q] = in[q] ? af : 0.f;
-    F.M[q] = in[q] ? 1.f + K.gamma * af * af : 0.f;
-    F.sM += F.M[q];
-    F.sa += F.a[q];
-    F.m += in[q] ? 1 : 0;
-    F.in |= in[q] ? (1u << q) : 0u;
-  }
-}
-
-// Values of the correction at cell x = (i, j, k), with the prolongation
-// P(e_c - e_c^0) of the next coarser level C added when `pro` is set.
+// Values of the correction at a cell.
 struct Val3 {
   float phi, mu, p;
 };
 
+// Values at cell x = (i, j, k), with the prolongation P(e_c - e_c^0) of the
+// next coarser level C added when `pro` is set.
 __device__ __forceinline__ Val3 read_val(const Level<float>& L, const Level<float>& C, int x, int i, int j, int k,
                                          bool pro) {
   Val3 v{L.phi[x], L.mu[x], L.p[x]};
@@ -80,56 +44,96 @@ __device__ __forceinline__ Val3 read_val(const Level<float>& L, const Level<floa
   return v;
 }
 
-// Coordinates of the neighbour across face q (the cell itself on a missing face).
+// The arithmetic of the 3D correction form, shared by every kernel that
+// smooths or restricts these levels (so that all of them give the same bits):
+// N from face differences d = neighbour - cell, with w = dp + gamma a dmu and
+// v = dmu + a w (= M dmu + a dp),
+//   N1 = phi - s/h^2 sum v,  N3 = -1/h^2 sum w,  N2 = mu - chi + (3/4) eps^2/h^2 sum dphi.
+// A missing face has the cell itself as its neighbour and a = 0.  Products
+// and sums are written as the instructions they are.
 template <int DIM>
-__device__ __forceinline__ void nb_coords(const FacesC<DIM>& F, int q, int i, int j, int k, int& a, int& b, int& d) {
-  const bool in = (F.in >> q) & 1u;
-  const int s = in ? ((q & 1) ? 1 : -1) : 0;
-  a = i + ((q >> 1) == 0 ? s : 0);
-  b = j + ((q >> 1) == 1 ? s : 0);
-  d = k + ((q >> 1) == 2 ? s : 0);
-}
+struct Sums3 {
+  float sv, sw, sd;
+};
 
-// N(e) at cell c in correction form on explicitly given values: own value u,
-// neighbour values nb[] (the cell itself on missing faces), base phi_b and
-// phi^m at c.
 template <int DIM>
-__device__ __forceinline__ void n_corr(const Level<float>& L, const Coefs<float>& K, const FacesC<DIM>& F,
-                                       const Val3& u, const Val3 (&nb)[2 * DIM], float phib, float pm, float& n1,
-                                       float& n2, float& n3) {
-  float Mp = -0.f, amu = -0.f, sphi = -0.f, sp = -0.f;
+__device__ __forceinline__ Sums3<DIM> sums3(const Val3& c, const Val3 (&nb)[2 * DIM], const float (&a)[2 * DIM],
+                                            float gamma) {
+  Sums3<DIM> S{0.f, 0.f, 0.f};
 #pragma unroll
   for (int q = 0; q < 2 * DIM; ++q) {
-    const bool in = (F.in >> q) & 1u;
-    Mp += F.M[q] * nb[q].mu;
-    Mp += F.a[q] * nb[q].p;
-    amu += F.a[q] * nb[q].mu;
-    sphi += in ? nb[q].phi : -0.f;
-    sp += in ? nb[q].p : -0.f;
+    const float dmu = nb[q].mu - c.mu, dp = nb[q].p - c.p;
+    const float w = fmaf(gamma, __fmul_rn(a[q], dmu), dp);
+    const float v = fmaf(a[q], w, dmu);
+    S.sv = q == 0 ? v : S.sv + v;
+    S.sw = q == 0 ? w : S.sw + w;
   }
-  const float mm = (float)F.m;
-  const float chi_d = 0.25f * u.phi * (3.f * phib * phib + 2.f * phib * pm + pm * pm + (3.f * phib + pm) * u.phi +
-                                       u.phi * u.phi);
-  n1 = u.phi - L.sih2 * ((Mp - F.sM * u.mu) - F.sa * u.p);
-  n2 = u.mu - chi_d + L.e34ih2 * (sphi - mm * u.phi);
-  n3 = -L.ih2 * ((sp - mm * u.p) + K.gamma * (amu - F.sa * u.mu));
+  float t = (nb[0].phi + nb[1].phi) + (nb[2].phi + nb[3].phi);
+  if (DIM == 3) t += nb[2 * DIM - 2].phi + nb[2 * DIM - 1].phi;
+  S.sd = fmaf(DIM == 3 ? -6.f : -4.f, c.phi, t);
+  return S;
 }
 
-// The cell's Newton step in correction form from its residual rows R1, R2,
-// R3 (the pressure row eliminated, as in cell_update): the updated values.
-template <int DIM>
-__device__ __forceinline__ Val3 corr_newton(const Level<float>& L, const Coefs<float>& K, const FacesC<DIM>& F,
-                                            const Val3& u, float phib, float pm, float R1, float R2, float R3) {
-  const float im = rcp_approx((float)F.m);
-  const float R3n = L.h2 * im * R3;
-  const float w = phib + u.phi;
-  const float B = (0.75f * w + 0.5f * pm) * w + 0.25f * pm * pm + L.e34ih2 * (float)F.m;
-  const float Ae = L.sih2 * (F.sM - K.gamma * F.sa * F.sa * im);
-  const float Cc = L.sih2 * F.sa, Gn = K.gamma * F.sa * im;
-  const float dphi = ((R1 - Ae * R2) - Cc * R3n) * rcp_approx(1.f + Ae * B);
-  const float dmu = R2 + B * dphi;
-  const float dp = R3n - Gn * dmu;
-  return Val3{u.phi + dphi, u.mu + dmu, u.p + dp};
+// chi(phi_b + e, phi^m) - chi(phi_b, phi^m) = e (q0 + e (q1 + e/4)).
+struct Chi3 {
+  float q0, q1;
+};
+
+__device__ __forceinline__ Chi3 chi3_of(float pm, float pb) {
+  return Chi3{__fmul_rn(0.25f, fmaf(pm, pm, __fmul_rn(pb, fmaf(3.f, pb, pm + pm)))),
+              __fmul_rn(0.25f, fmaf(3.f, pb, pm))};
+}
+
+__device__ __forceinline__ float chi3(float e, const Chi3& k) {
+  return __fmul_rn(e, fmaf(e, fmaf(0.25f, e, k.q1), k.q0));
+}
+
+// N of cell c from its sums.  (LV: a Level<float> or another struct with its
+// scalars ih2, h2, sih2, e34ih2.)
+template <int DIM, class LV>
+__device__ __forceinline__ Val3 n_corr(const LV& L, const Sums3<DIM>& S, const Val3& c, const Chi3& k) {
+  return Val3{fmaf(-L.sih2, S.sv, c.phi), fmaf(L.e34ih2, S.sd, c.mu - chi3(c.phi, k)), -__fmul_rn(L.ih2, S.sw)};
+}
+
+// The constants of a cell's Newton step from its face values (0 on missing
+// faces) and the number m of interior faces: Ae, x = sum a / m, hn = h^2 / m,
+// em = (3/4) eps^2 m / h^2.
+struct Newton3 {
+  float Ae, x, hn, em;
+};
+
+template <int DIM, class LV>
+__device__ __forceinline__ Newton3 newton3(const LV& L, float gamma, const float (&a)[2 * DIM], int m) {
+  const float n = (float)m, im = rcp_approx(n);
+  float sa = (a[0] + a[1]) + (a[2] + a[3]);
+  float s2 = fmaf(a[0], a[0], fmaf(a[1], a[1], fmaf(a[2], a[2], __fmul_rn(a[3], a[3]))));
+  if (DIM == 3) {
+    sa += a[2 * DIM - 2] + a[2 * DIM - 1];
+    s2 = fmaf(a[2 * DIM - 2], a[2 * DIM - 2], fmaf(a[2 * DIM - 1], a[2 * DIM - 1], s2));
+  }
+  Newton3 k;
+  k.x = __fmul_rn(sa, im);
+  k.Ae = __fmul_rn(L.sih2, fmaf(-__fmul_rn(gamma, sa), k.x, fmaf(gamma, s2, n)));
+  k.hn = __fmul_rn(L.h2, im);
+  k.em = __fmul_rn(L.e34ih2, n);
+  return k;
+}
+
+// The cell's Newton step in correction form (the pressure row eliminated, as
+// in cell_update): the updated values.
+template <int DIM, class LV>
+__device__ __forceinline__ Val3 update3(const LV& L, const Coefs<float>& K, const Val3& c, const Val3 (&nb)[2 * DIM],
+                                        const float (&a)[2 * DIM], float f1, float f2, float f3, const Chi3& k,
+                                        const Newton3& N) {
+  const Sums3<DIM> S = sums3<DIM>(c, nb, a, K.gamma);
+  const float R1 = fmaf(L.sih2, S.sv, f1 - c.phi);
+  const float R2 = fmaf(-L.e34ih2, S.sd, (f2 - c.mu) + chi3(c.phi, k));
+  const float R3 = fmaf(L.ih2, S.sw, f3);
+  const float B = fmaf(c.phi, fmaf(0.75f, c.phi, k.q1 + k.q1), k.q0 + N.em);
+  const float num = fmaf(-__fmul_rn(K.s, N.x), R3, fmaf(-N.Ae, R2, R1));
+  const float dphi = __fmul_rn(num, rcp_approx(fmaf(N.Ae, B, 1.f)));
+  const float dmu = fmaf(B, dphi, R2);
+  return Val3{c.phi + dphi, c.mu + dmu, c.p + fmaf(-__fmul_rn(K.gamma, N.x), dmu, __fmul_rn(N.hn, R3))};
 }
 
 // One colour pass of the correction-form smoother on a single-precision
@@ -162,20 +166,31 @@ __device__ __forceinline__ void smooth_c_body(int bx, const Level<float>& L, con
   const int i_other = 2 * ti + ((j + k + colour + 1) & 1);  // the other colour's cell of the x-pair
   if (i < L.nx) {
     const int c = i + L.nx * (j + L.ny * k);
-    FacesC<DIM> F;
-    faces_c<DIM>(L, K, c, i, j, k, F);
-    const float pm = L.phim[c], phib = L.phib[c];
+    const int sy = L.nx, sz = L.nx * L.ny;
+    const bool in[6] = {i > 0, i + 1 < L.nx, j > 0, j + 1 < L.ny, k > 0, k + 1 < L.nz};
+    const int off[6] = {-1, 1, -sy, sy, -sz, sz};
+    const float ps = L.phis[c];
+    int x[2 * DIM];  // the neighbours (the cell itself on a missing face, so that every load is in bounds)
+    float a[2 * DIM];
+    int m = 0;
+#pragma unroll
+    for (int q = 0; q < 2 * DIM; ++q) {
+      x[q] = in[q] ? c + off[q] : c;
+      const float af = 0.5f * (ps + L.phis[x[q]]);
+      a[q] = in[q] ? af : 0.f;
+      m += in[q] ? 1 : 0;
+    }
+    const Chi3 ch = chi3_of(L.phim[c], L.phib[c]);
     float f1 = L.fphi[c], f2 = L.fmu[c], f3 = L.fp[c];
     if (rhs) {  // f += N(R u), R u = (phi0, mu0, p0) of this coarse level
-      Val3 u0{L.phi0[c], L.mu0[c], L.p0[c]};
+      const Val3 u0{L.phi0[c], L.mu0[c], L.p0[c]};
       Val3 nb0[2 * DIM];
 #pragma unroll
-      for (int q = 0; q < 2 * DIM; ++q) nb0[q] = Val3{L.phi0[F.e[q]], L.mu0[F.e[q]], L.p0[F.e[q]]};
-      float n1, n2, n3;
-      n_corr<DIM>(L, K, F, u0, nb0, phib, pm, n1, n2, n3);
-      f1 += n1;
-      f2 += n2;
-      f3 += n3;
+      for (int q = 0; q < 2 * DIM; ++q) nb0[q] = Val3{L.phi0[x[q]], L.mu0[x[q]], L.p0[x[q]]};
+      const Val3 n = n_corr<DIM>(L, sums3<DIM>(u0, nb0, a, K.gamma), u0, ch);
+      f1 += n.phi;
+      f2 += n.mu;
+      f3 += n.p;
       L.fphi[c] = f1;
       L.fmu[c] = f2;
       L.fp[c] = f3;
@@ -184,13 +199,12 @@ __device__ __forceinline__ void smooth_c_body(int bx, const Level<float>& L, con
     Val3 nb[2 * DIM];
 #pragma unroll
     for (int q = 0; q < 2 * DIM; ++q) {
-      int a, b, d;
-      nb_coords<DIM>(F, q, i, j, k, a, b, d);
-      nb[q] = read_val(L, C, F.e[q], a, b, d, pro == 1);
+      const int d = in[q] ? ((q & 1) ? 1 : -1) : 0;
+      nb[q] = read_val(L, C, x[q], i + (q < 2 ? d : 0), j + (q >> 1 == 1 ? d : 0), k + (q >= 4 ? d : 0), pro == 1);
+      // a missing face's neighbour is the cell as it is read
+      if (!in[q]) nb[q] = u;
     }
-    float n1, n2, n3;
-    n_corr<DIM>(L, K, F, u, nb, phib, pm, n1, n2, n3);
-    const Val3 e = corr_newton<DIM>(L, K, F, u, phib, pm, f1 - n1, f2 - n2, f3 - n3);
+    const Val3 e = update3<DIM>(L, K, u, nb, a, f1, f2, f3, ch, newton3<DIM>(L, K.gamma, a, m));
     const float ephi = e.phi, emu = e.mu, ep = e.p;
     L.phi[c] = ephi;
     L.mu[c] = emu;
@@ -219,29 +233,6 @@ __global__ void __launch_bounds__(kSmoothBlock, 8) k_smooth_c(const __grid_const
                                                            const __grid_constant__ Level<double> U) {
   pdl_enter();
   smooth_c_body<DIM>(blockIdx.x, L, C, K, colour, rhs, pro, U);
-}
-
-// Face data of a cell from its phi* value pc and its neighbours' pe[] (the
-// cell's own value where in[q] is false), as faces_c forms it from indices
-// (the x-quad passes and the restriction).
-template <int DIM>
-__device__ __forceinline__ void faces_vals(const Coefs<float>& K, float pc, const float (&pe)[6], const bool (&in)[6],
-                                           FacesC<DIM>& F) {
-  F.sM = -0.f;
-  F.sa = -0.f;
-  F.m = 0;
-  F.in = 0u;
-#pragma unroll
-  for (int q = 0; q < 2 * DIM; ++q) {
-    const float af = 0.5f * (pc + pe[q]);
-    F.e[q] = 0;
-    F.a[q] = in[q] ? af : 0.f;
-    F.M[q] = in[q] ? 1.f + K.gamma * af * af : 0.f;
-    F.sM += F.M[q];
-    F.sa += F.a[q];
-    F.m += in[q] ? 1 : 0;
-    F.in |= in[q] ? (1u << q) : 0u;
-  }
 }
 
 // ------------------------------------------------------------ x-quad passes
@@ -401,34 +392,42 @@ __device__ __forceinline__ void smooth_c4_body(const Level<float>& L, const Leve
       nb[5] = Val3{at(A.zp), at(B.zp), at(D.zp)};
     };
     const bool in[6] = {h || Q.s || Q.xin, !h || !Q.s || Q.xin, Q.ym, Q.yp, Q.zm, Q.zp};
+    const float ps = at(S.o);
     const float pe[6] = {xm(S), xp(S), at(S.ym), at(S.yp), at(S.zm), at(S.zp)};
-    FacesC<3> F;
-    faces_vals<3>(K, at(S.o), pe, in, F);
-    const float pm = at(pm4), phib = at(pb4);
+    float a[6];
+    int m = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const float af = 0.5f * (ps + pe[q]);
+      a[q] = in[q] ? af : 0.f;
+      m += in[q] ? 1 : 0;
+    }
+    const Chi3 ch = chi3_of(at(pm4), at(pb4));
     float g1 = at(f1), g2 = at(f2), g3 = at(f3);
-    float n1, n2, n3;
     if (RHS) {  // f += N(R u), R u = (phi0, mu0, p0) of this coarse level
       const Val3 u0{at(P0.o), at(M0.o), at(R0.o)};
       Val3 nb0[6];
       nbs(P0, M0, R0, nb0);
-      n_corr<3>(L, K, F, u0, nb0, phib, pm, n1, n2, n3);
-      g1 += n1;
-      g2 += n2;
-      g3 += n3;
+      const Val3 n = n_corr<3>(L, sums3<3>(u0, nb0, a, K.gamma), u0, ch);
+      g1 += n.phi;
+      g2 += n.mu;
+      g3 += n.p;
       put(f1, g1);
       put(f2, g2);
       put(f3, g3);
     }
     Val3 u{at(P.o), at(M.o), at(R.o)};
+    Val3 nb[6];
+    nbs(P, M, R, nb);
     if (PRO == 2) {
       u.phi += h ? dP.y : dP.x;
       u.mu += h ? dM.y : dM.x;
       u.p += h ? dR.y : dR.x;
+#pragma unroll
+      for (int q = 0; q < 6; ++q)  // a missing face's neighbour is the cell as it is read
+        if (!in[q]) nb[q] = u;
     }
-    Val3 nb[6];
-    nbs(P, M, R, nb);
-    n_corr<3>(L, K, F, u, nb, phib, pm, n1, n2, n3);
-    const Val3 e = corr_newton<3>(L, K, F, u, phib, pm, g1 - n1, g2 - n2, g3 - n3);
+    const Val3 e = update3<3>(L, K, u, nb, a, g1, g2, g3, ch, newton3<3>(L, K.gamma, a, m));
     put(outP, e.phi);
     put(outM, e.mu);
     put(outR, e.p);
@@ -570,13 +569,15 @@ __device__ __forceinline__ void residual_restrict_c_body(int bx, const Level<flo
         pe[q] = cx(S[q - 1]);
         nb[q] = Val3{cx(Ph[q - 1]), cx(Mu[q - 1]), cx(Pr[q - 1])};
       }
-      if (DIM == 2) pe[4] = pe[5] = pc;
-      FacesC<DIM> Fc;
-      faces_vals<DIM>(K, pc, pe, in, Fc);
+      float a[2 * DIM];
+#pragma unroll
+      for (int q = 0; q < 2 * DIM; ++q) {
+        const float af = 0.5f * (pc + pe[q]);
+        a[q] = in[q] ? af : 0.f;
+      }
       const float phib = cx(pb);
-      float n1, n2, n3;
-      n_corr<DIM>(F, K, Fc, u, nb, phib, cx(pm), n1, n2, n3);
-      const float r[7] = {cx(f1) - n1, cx(f2) - n2, cx(f3) - n3, u.phi, u.mu, u.p, phib};
+      const Val3 n = n_corr<DIM>(F, sums3<DIM>(u, nb, a, K.gamma), u, chi3_of(cx(pm), phib));
+      const float r[7] = {cx(f1) - n.phi, cx(f2) - n.mu, cx(f3) - n.p, u.phi, u.mu, u.p, phib};
 #pragma unroll
       for (int q = 0; q < 7; ++q) v[q] = h ? v[q] + r[q] : r[q];
     }
