@@ -28,6 +28,7 @@
 #include "chhs_kernels.cuh"
 #include "chhs_cluster.cuh"
 #include "chhs_tail2.cuh"
+#include "chhs_tail3.cuh"
 #include "chhs_tile.cuh"
 #include "chhs_corr3.cuh"
 #include "chhs_norm_df.cuh"
@@ -445,6 +446,14 @@ struct Enqueue {
         return;
       }
     }
+    if constexpr (recompute_coefs<T, CORR>()) {
+      if (l == run->tail_start && tail3_fits(tail)) {
+        launch(run, s, CHHS_K_COARSEST, 1.0, [&] {
+          pdl_smem(k_tail3, 1, tail3_threads(tail), tail3_bytes(tail), s, tail, K);
+        });
+        return;
+      }
+    }
     if (l == run->tail_start) {
       const size_t smem = tail_bytes<T, CORR>(tail);
       launch(run, s, CHHS_K_COARSEST, 1.0, [&] {
@@ -586,6 +595,17 @@ struct Enqueue {
   template <typename T>
   static constexpr bool use_tiles() { return DIM == 2 && std::is_same<T, float>::value; }
 
+  // Shared memory and threads of the 3D mixed form's tail (tail3_body).
+  static size_t tail3_bytes(const Tail<float>& tail) {
+    int nc[kTailMaxLevels];
+    for (int l = 0; l < tail.n; ++l) nc[l] = tail.lev[l].ncell;
+    return tail3_smem_bytes(nc, tail.n, tail.coarsest_f64);
+  }
+  // A tail of one level, or with more threads than a block has (more than 1024
+  // cells, chhs_tuning.tail_cells), runs on the general code.
+  static bool tail3_fits(const Tail<float>& tail) { return tail.n > 1 && tail3_threads(tail) <= kTail3Threads; }
+  static int tail3_threads(const Tail<float>& tail) { return ((tail.lev[0].ncell >> 1) + 31) / 32 * 32; }
+
   template <typename T, bool CORR>
   static size_t tail_bytes(const Tail<T>& tail) {
     int nc[kTailMaxLevels];
@@ -620,6 +640,9 @@ struct Enqueue {
       return fail(run, CHHS_ERR_INVALID_ARG,
                   "the grid does not coarsen to a coarsest level small enough for the one-block solve");
     CU(raise_to(ktail, smem));
+    if constexpr (recompute_coefs<T, CORR>()) {
+      if (tail3_fits(tail)) CU(raise_to(reinterpret_cast<const void*>(k_tail3), tail3_bytes(tail)));
+    }
     if constexpr (use_tiles<T>()) {
       // the accepted sweep counts: tiles with their halo in nine shared fields
       const int halo = 2 * std::max(std::max(run->opts.nu1, run->opts.nu2), std::max(run->nu1c, run->nu2c)) + 1;
@@ -684,16 +707,16 @@ struct Enqueue {
     frame_coefs(run, s);
   }
 
-  // Mixed form with the finest level above the tail: k_setup_mixed (such a
-  // level coarsens, so its extents are even).
-  static bool setup_mixed(const chhs_t* run) { return mixed(run) && run->tail_start > 0; }
+  // Mixed form with a finest level that coarsens (so its extents are even): k_setup_mixed.
+  static bool setup_mixed(const chhs_t* run) { return mixed(run) && run->lev32.size() > 1; }
   static int setup_mixed_blocks(const Level<float>& Gn) { return (Gn.ncell + kSetupBlock - 1) / kSetupBlock; }
 
-  // Single-precision levels whose kernels read stored coefficients: the tail's,
-  // and in 3D those without a pre-smoothing sweep (k_coarse_rhs).  The others
-  // recompute them from phi*.
+  // Single-precision levels whose kernels read stored coefficients: the coarsest
+  // and a 3D tail of the general code, and in 3D those without a pre-smoothing
+  // sweep (k_coarse_rhs).  The others recompute them from phi*.
   static bool stored_coefs(const chhs_t* run, int l) {
-    return l >= run->tail_start || (DIM == 3 && nu_pre(run, l) == 0);
+    if (DIM == 3 && l >= run->tail_start && !tail3_fits(run->tail32)) return true;
+    return l + 1 == (int)run->lev32.size() || (DIM == 3 && nu_pre(run, l) == 0);
   }
 
   static void frame_setup(chhs_t* run, cudaStream_t s) {
@@ -1873,7 +1896,7 @@ struct BatchStep {
   std::vector<size_t> offs;         // table offsets in emission order
   size_t cur = 0;
   int* counter = nullptr;           // launches, while capturing
-  size_t tail_smem = 0;
+  size_t tail_smem = 0, tail3_smem = 0;
 
   size_t put(const void* p, size_t n) {
     const size_t off = align_up(buf.size());
@@ -1914,8 +1937,15 @@ struct BatchStep {
     prof->units.push_back(1.0);
   }
 
-  // The tail launch: one block per job, no prefix sum.
-  void go_tail(const std::vector<TailJob<float>>& jobs, cudaStream_t s) {
+  // The tail launches: one block per job, no prefix sum; in 3D the tails of
+  // more than one level are a launch of their own (kb_tail3).
+  void go_tails(const std::vector<TailJob<float>>& jobs, cudaStream_t s) {
+    std::vector<TailJob<float>> general, blocks;
+    for (const TailJob<float>& j : jobs) (DIM == 3 && Enqueue<DIM>::tail3_fits(j.tl) ? blocks : general).push_back(j);
+    go_tail(blocks, true, s);
+    go_tail(general, false, s);
+  }
+  void go_tail(const std::vector<TailJob<float>>& jobs, bool tail3, cudaStream_t s) {
     if (jobs.empty()) return;
     if (!capture) {
       offs.push_back(put(jobs.data(), sizeof(TailJob<float>) * jobs.size()));
@@ -1923,8 +1953,10 @@ struct BatchStep {
     }
     const TailJob<float>* dj = reinterpret_cast<const TailJob<float>*>(b->tables + offs[cur++]);
     if (counter) ++*counter;
-    timed(CHHS_K_COARSEST, [&] { pdl_smem(kb_tail<float, DIM, true>, (int)jobs.size(), kTailThreads, tail_smem, s, dj); },
-          s);
+    timed(CHHS_K_COARSEST, [&] {
+      if (tail3) pdl_smem(kb_tail3, (int)jobs.size(), kTail3Threads, tail3_smem, s, dj);
+      else pdl_smem(kb_tail<float, DIM, true>, (int)jobs.size(), kTailThreads, tail_smem, s, dj);
+    }, s);
   }
 
   static Coefs<float> k32(const chhs_t* r) { return Enqueue<DIM>::template coefs<float>(r); }
@@ -1997,7 +2029,7 @@ struct BatchStep {
     for (int l = 0; l < ts; ++l) pre(s, l, l == 0 ? b->opts.nu1 : r0->nu1c);
     std::vector<TailJob<float>> tails;
     for (chhs_t* r : b->runs) tails.push_back(TailJob<float>{r->tail32, k32(r), gate(r)});
-    go_tail(tails, s);
+    go_tails(tails, s);
     for (int l = ts - 1; l >= 0; --l) post(s, l, l == 0 ? b->opts.nu2 : r0->nu2c);
     if (vk != 1) return;
     JobList<PairJob> upd;
@@ -2174,7 +2206,12 @@ struct BatchStep {
     int dev = 0, optin = 0;
     BCU(cudaGetDevice(&dev));
     BCU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    for (chhs_t* r : b->runs) tail_smem = std::max(tail_smem, Enqueue<DIM>::template tail_bytes<float, true>(r->tail32));
+    for (chhs_t* r : b->runs) {
+      tail_smem = std::max(tail_smem, Enqueue<DIM>::template tail_bytes<float, true>(r->tail32));
+      if (DIM == 3 && Enqueue<DIM>::tail3_fits(r->tail32)) {
+        tail3_smem = std::max(tail3_smem, Enqueue<DIM>::tail3_bytes(r->tail32));
+      }
+    }
     if (DIM == 2) {  // the accepted sweep counts and shapes, as Enqueue::prepare_tail
       const int halo = 2 * std::max(std::max(b->opts.nu1, b->opts.nu2), std::max(b->runs[0]->nu1c, b->runs[0]->nu2c)) + 1;
       if (std::max(tile_limit_bytes(halo, kTileW, kTileH), tile_limit_bytes(halo, b->big_tw, b->big_th)) > (size_t)optin)
@@ -2191,8 +2228,8 @@ struct BatchStep {
       return CHHS_OK;
     };
     chhs_status st = raise_to(reinterpret_cast<const void*>(kb_tail<float, DIM, true>), tail_smem);
-    if (st != CHHS_OK) return st;
-    return CHHS_OK;
+    if (st == CHHS_OK && tail3_smem) st = raise_to(reinterpret_cast<const void*>(kb_tail3), tail3_smem);
+    return st;
   }
 
   // Capture the step graph (the structure of a single run's build_graph).

@@ -16,6 +16,7 @@
 #include "chhs_kernels.cuh"
 #include "chhs_norm_df.cuh"
 #include "chhs_tail2.cuh"
+#include "chhs_tail3.cuh"
 #include "chhs_tile.cuh"
 
 namespace chhs_dev {
@@ -227,6 +228,15 @@ __global__ void __launch_bounds__(kTailThreads, 1) kb_tail(const TailJob<T>* job
   const TailJob<T>& J = jobs[blockIdx.x];
   if (!gate_open(J.gate)) return;
   tail_run<T, DIM, CORR>(J.tl, J.K);
+}
+
+// The 3D tails of more than one level (tail3_body), one block per job.
+static __global__ void __launch_bounds__(kTail3Threads, 1) kb_tail3(const TailJob<float>* jobs) {
+  extern __shared__ __align__(16) unsigned char bt3_smem[];
+  pdl_enter();
+  const TailJob<float>& J = jobs[blockIdx.x];
+  if (!gate_open(J.gate)) return;
+  tail3_body(J.tl, J.K, bt3_smem);
 }
 
 struct SmoothCJob {

@@ -9,9 +9,11 @@
 // a pass reads four neighbour cells, updates two and stores them.  Levels of
 // at most 32 threads (16 x 16 cells has 64, 8 x 8 has 16) are one warp's, with
 // a warp barrier between passes; the coarsest grid of at most 32 cells is a
-// cell per lane, its neighbours by shuffles.  A larger coarsest grid, and its
-// double-precision solve (coarsest_f64), run on the general tail's code.
-// Measured: FIGURES.
+// cell per lane, its neighbours by shuffles, a larger one a cell per thread.
+// The double-precision coarsest solve (coarsest_f64) runs on the general tail's
+// code.
+// Measured: the tail of a 512^2 step 33 -> 16 us (32 thousand cycles, a pass of
+// one warp 320-350), the step 690 -> 588 us; 640 x 384 930 -> 765 us.
 #pragma once
 #include "chhs_tile.cuh"
 
@@ -273,12 +275,62 @@ __device__ __forceinline__ TileCell tail2_coarsest(const Level<float>& L, const 
   return TileCell{u.phi - q.u.phi, u.mu - q.u.mu, u.p - q.u.p};
 }
 
+// The same for more cells, at most one per thread: cell t on thread t, exchanged
+// through buf, the block's sums through red (a float per warp).  Every thread
+// of the block calls it.
+__device__ __forceinline__ TileCell tail2_coarsest_block(const Level<float>& L, const Coefs<float>& K,
+                                                         const Tail2Coarse& q, float ps, float pm, int t, float4* buf,
+                                                         float* red) {
+  const bool act = t < L.ncell;
+  const int j = small_div(t, L.rnx), i = t - j * L.nx;
+  TileCell u = q.u;
+  if (act) buf[t] = make_float4(u.phi, u.mu, u.p, ps);
+  __syncthreads();
+  const bool in0 = act && i > 0, in1 = act && i + 1 < L.nx, in2 = act && j > 0, in3 = act && j + 1 < L.ny;
+  const int own = act ? t : 0;
+  const float4 *b0 = buf + (in0 ? t - 1 : own), *b1 = buf + (in1 ? t + 1 : own), *b2 = buf + (in2 ? t - L.nx : own),
+               *b3 = buf + (in3 ? t + L.nx : own);
+  const float a0 = in0 ? 0.5f * (ps + b0->w) : 0.f, a1 = in1 ? 0.5f * (ps + b1->w) : 0.f,
+              a2 = in2 ? 0.5f * (ps + b2->w) : 0.f, a3 = in3 ? 0.5f * (ps + b3->w) : 0.f;
+  const int faces = max(1, (int)in0 + (int)in1 + (int)in2 + (int)in3);
+  const TileConst k = tile_constants(L, K, pm, q.pb, a0, a1, a2, a3, faces);
+  float f1 = q.f1, f2 = q.f2, f3 = q.f3;
+  tile_add_N(f1, f2, f3, u, tail2_get(b0), tail2_get(b1), tail2_get(b2), tail2_get(b3), a0, a1, a2, a3, k, L, K);
+  float acc0 = -1.f, prev = 0.f;
+  for (int it = 0; it <= kCoarsestMaxSweeps; ++it) {
+    float r1 = 0.f, r2 = 0.f, r3 = 0.f;
+    tile_add_N(r1, r2, r3, u, tail2_get(b0), tail2_get(b1), tail2_get(b2), tail2_get(b3), a0, a1, a2, a3, k, L, K);
+    r1 = f1 - r1;
+    r2 = f2 - r2;
+    r3 = K.s * (f3 - r3);
+    const float part = warp_sum(act ? r1 * r1 + r2 * r2 + r3 * r3 : 0.f);
+    if ((t & 31) == 0) red[t >> 5] = part;
+    __syncthreads();
+    float tot = 0.f;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
+    if (acc0 < 0.f) acc0 = tot;
+    if (!(tot > kCoarsestTarget2 * acc0) || tot < 1e-37f) break;
+    if (it >= 8 && tot >= prev) break;
+    prev = tot;
+    for (int colour = 0; colour < 2; ++colour) {
+      if (act && ((i + j + colour) & 1) == 0) {
+        tile_update(u, tail2_get(b0), tail2_get(b1), tail2_get(b2), tail2_get(b3), a0, a1, a2, a3, f1, f2, f3, k, L, K);
+        buf[t] = make_float4(u.phi, u.mu, u.p, ps);
+      }
+      __syncthreads();
+    }
+  }
+  return TileCell{u.phi - q.u.phi, u.mu - q.u.mu, u.p - q.u.p};
+}
+
 // The tail's levels tl.lev[0 .. n-1], n >= 2: those above the coarsest have
 // even extents and level 0 at most blockDim.x blocks of 2 x 2 cells.
 __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<float>& K, unsigned char* smem) {
   const int n = tl.n, t = threadIdx.x, lane = t & 31;
   const Level<float>& Gc = tl.lev[n - 1];
-  const bool lanes = Gc.ncell <= 32 && !tl.coarsest_f64;  // the coarsest grid on the lanes of warp 0
+  const bool general = tl.coarsest_f64 != 0;              // the coarsest solve on the general code
+  const bool lanes = Gc.ncell <= 32 && !general;          // the coarsest grid on the lanes of warp 0
+  __shared__ float red[kTailThreads / 32];
   __shared__ Tail2Scalars sc[kTailMaxLevels];  // of the levels above the coarsest; [n - 1].off: their end
   if (t < n) {
     const Level<float>& G = tl.lev[t];
@@ -313,7 +365,7 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
     ld(G0.phib, pb);
   }
   float cps = 0.f, cpm = 0.f;
-  if (lanes) {
+  if (!general) {
     if (t < Gc.ncell) {
       cps = Gc.phis[t];
       cpm = Gc.phim[t];
@@ -348,6 +400,7 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   __syncthreads();
 
   Tail2Block b;
+  Tail2Coarse z{};               // the coarsest cell t (the level above's block t sits on it)
   TileCell corr{0.f, 0.f, 0.f};  // the next coarser level's correction at the block's coarse cell
   auto down = [&](int l, bool warp) {
     const Tail2Scalars L = sc[l];
@@ -386,6 +439,8 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
       }
     } else if (lanes) {
       corr = tail2_coarsest(Gc, K, q, cps, cpm, lane);  // warp 0 only: this level has at most 32 blocks
+    } else if (!general) {
+      z = q;
     } else if (act) {
       const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
       S.phi[t] = S.phi0[t] = q.u.phi;
@@ -431,14 +486,14 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
     down(l, l >= small);
     tail2_sync(l >= small);
   }
-  if (!lanes) {
+  if (!lanes && !general) {  // the level above has more than 32 blocks: every thread is here
+    corr = tail2_coarsest_block(Gc, K, z, cps, cpm, t, reinterpret_cast<float4*>(smem + coff), red);
+    __syncthreads();
+  } else if (!lanes) {
     __syncthreads();
     const Level<float> S = tail_carve<float, 2, true>(Gc, smem + coff);
     tail_rhs<float, 2, true>(S, K);
-    if (tl.coarsest_f64)
-      coarsest_solve_f64<2>(S, K, smem + coff + tail_fields<2, true>() * tail_align(sizeof(float) * Gc.ncell));
-    else
-      coarsest_solve<float, 2, true>(S, K);
+    coarsest_solve_f64<2>(S, K, smem + coff + tail_fields<2, true>() * tail_align(sizeof(float) * Gc.ncell));
     // level n - 2's block t sits on coarse cell t
     if (t < Gc.ncell) corr = TileCell{S.phi[t] - S.phi0[t], S.mu[t] - S.mu0[t], S.p[t] - S.p0[t]};
     __syncthreads();
