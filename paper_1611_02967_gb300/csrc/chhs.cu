@@ -959,6 +959,7 @@ Level<T> make_level(const chhs_t* run, const Shape& sh, int l, char* base, bool 
   L.ax = f[11]; L.ay = f[12]; L.Mx = f[13]; L.My = f[14];
   L.sM = f[15]; L.sa = f[16];
   L.cAe = f[17]; L.cC = f[18]; L.cGn = f[19]; L.cHn = f[20]; L.cQ = f[21]; L.cH = f[22];
+  level_constants(L);
   int q = 23;
   L.az = run->dim == 3 ? f[q++] : nullptr;
   L.Mz = run->dim == 3 ? f[q++] : nullptr;

@@ -98,6 +98,7 @@ __device__ __forceinline__ Slab cluster_slab(const Tail<double>& tl, const Clust
   L.cAe = carve(); L.cC = carve(); L.cGn = carve(); L.cHn = carve(); L.cQ = carve(); L.cH = carve();
   if (DIM == 3) { L.az = carve(); L.Mz = carve(); }
   L.phis = nullptr;
+  level_constants(L);
   return B;
 }
 
@@ -307,12 +308,12 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_cluster(const __grid_consta
       const int c = base + t;
       double v[15];
       v[0] = G.phim[c]; v[1] = G.ax[c]; v[2] = G.ay[c]; v[3] = G.Mx[c]; v[4] = G.My[c];
-      v[5] = G.sM[c]; v[6] = G.sa[c]; v[7] = G.cAe[c]; v[8] = G.cC[c]; v[9] = G.cGn[c];
-      v[10] = G.cHn[c]; v[11] = G.cQ[c]; v[14] = G.cH[c];
+      v[5] = G.sM[c]; v[6] = G.sa[c]; v[11] = G.cQ[c]; v[14] = G.cH[c];
+      const float k0 = G.kAe[c], k1 = G.kC[c], k2 = G.kGn[c], k3 = G.kHn[c];
       if (DIM == 3) { v[12] = G.az[c]; v[13] = G.Mz[c]; }
       S.phim[t] = v[0]; S.ax[t] = v[1]; S.ay[t] = v[2]; S.Mx[t] = v[3]; S.My[t] = v[4];
-      S.sM[t] = v[5]; S.sa[t] = v[6]; S.cAe[t] = v[7]; S.cC[t] = v[8]; S.cGn[t] = v[9];
-      S.cHn[t] = v[10]; S.cQ[t] = v[11]; S.cH[t] = v[14];
+      S.sM[t] = v[5]; S.sa[t] = v[6]; S.cQ[t] = v[11]; S.cH[t] = v[14];
+      S.kAe[t] = k0; S.kC[t] = k1; S.kGn[t] = k2; S.kHn[t] = k3;
       if (DIM == 3) { S.az[t] = v[12]; S.Mz[t] = v[13]; }
       if (l == 0) {
         S.fphi[t] = G.fphi[c]; S.fmu[t] = G.fmu[c]; S.fp[t] = G.fp[c];
