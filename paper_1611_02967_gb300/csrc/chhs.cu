@@ -495,17 +495,16 @@ struct Enqueue {
       return;
     }
     smooth<T, CORR>(run, s, L, nu_pre(run, l), rhs && nu_pre(run, l) > 0);
-    constexpr int TX = DIM == 3 ? 8 : 16;
-    const long long tiles = (long long)((L.nx + TX - 1) / TX) * (L.ny / 2) * (DIM == 3 ? L.nz / 2 : 1);
-    const int rblocks = (int)((tiles * 32 + kBlock - 1) / kBlock);
     launch(run, s, CHHS_K_RESTRICT, L.ncell, [&] {
       if constexpr (std::is_same<T, double>::value && !CORR) {
         if (L.ncell <= 2 * run->split_threads && l > 0) {  // small level: the three rows on three warps
+          constexpr int TX = DIM == 3 ? 8 : 16;
+          const long long tiles = (long long)((L.nx + TX - 1) / TX) * (L.ny / 2) * (DIM == 3 ? L.nz / 2 : 1);
           pdl(k_residual_restrict_split<DIM>, (int)tiles, 96, s, L, C, K);
           return;
         }
+        pdl(k_residual_restrict64<DIM>, (C.ncell + kSetupBlock - 1) / kSetupBlock, kSetupBlock, s, L, C, K);
       }
-      pdl(k_residual_restrict<T, DIM, CORR>, rblocks, kBlock, s, L, C, K);
     });
     vcycle<T, CORR>(run, s, lev, tail, l + 1);
     launch(run, s, CHHS_K_PROLONG, L.ncell, [&] {

@@ -706,61 +706,108 @@ __global__ void __launch_bounds__(kBlock) k_coarse_rhs(Level<T> C, Coefs<T> K) {
 
 // ---------------------------------------------------------------- transfers
 
-// Residual and restriction, one thread per fine cell.  A warp covers a tile
-// of 16 x 2 (2D) or 8 x 2 x 2 (3D) fine cells, so the 2^d children of a
-// coarse cell sit in lanes l, l^1, l^16 (2D) or l, l^1, l^8, l^16 (3D) and are
-// summed by shuffles.  Writes u_c = R u (twice: the coarse iterate and u_c^0),
-// R phi_b in correction form, and f_c = R r (completed later by N_c(R u)).
-template <typename T, int DIM, bool CORR>
-__global__ void __launch_bounds__(kBlock) k_residual_restrict(Level<T> F, Level<T> C, Coefs<T> K) {
+// Residual and restriction of the plain double-precision form, one thread per
+// coarse cell (its 2^d children).  Writes u_c = R u (twice: the coarse iterate
+// and u_c^0) and f_c = R r (completed later by N_c(R u)).
+//
+// What bounds it: the FP64 pipe (~64 cycles per warp instruction and
+// sub-partition), so the work is the fewest FP64 instructions.  In the sum of
+// the children's residuals the fluxes of the faces between them cancel: only
+// the faces around the group are formed, from differences d = outside -
+// inside,
+//   sum N1 = sum phi - s/h^2 sum_f (M dmu + a dp),
+//   sum N3 = -1/h^2 sum_f (dp + gamma a dmu),
+//   sum N2 = sum mu + (3/4) eps^2/h^2 (sum_f phi_out + d sum phi) - sum cubic_P:
+// a cell's own face terms are in cubic_P's Q, as a neighbour across the inner
+// faces it counts d times.
+// One thread per fine cell formed every flux twice and added six values over
+// the children by shuffles, 12-18 FP64 additions per cell:
+// on 128^3 and its levels above 32^3 65 us a launch on average, here 38;
+// a 128^3 step 15.0 -> 13.6 ms, three of 512^2 7.32 -> 6.92 ms.
+template <int DIM>
+__global__ void __launch_bounds__(kSetupBlock) k_residual_restrict64(const __grid_constant__ Level<double> F,
+                                                                    const __grid_constant__ Level<double> C,
+                                                                    Coefs<double> K) {
   pdl_enter();
-  constexpr int TX = DIM == 3 ? 8 : 16;
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int tiles_x = (F.nx + TX - 1) / TX;
-  const int tiles_y = F.ny >> 1;
-  const int tiles_z = DIM == 3 ? (F.nz >> 1) : 1;
-  if (warp >= tiles_x * tiles_y * tiles_z) return;  // whole warp
-  const int tx = warp % tiles_x;
-  const int rest = warp / tiles_x;
-  const int ty = rest % tiles_y, tz = rest / tiles_y;
-  const int i = tx * TX + (lane % TX);
-  const int j = 2 * ty + ((lane / TX) & 1);
-  const int k = DIM == 3 ? 2 * tz + (lane >> 4) : 0;
-  const bool valid = i < F.nx;
-  constexpr int NV = CORR ? 7 : 6;
-  T v[NV];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= C.ncell) return;
+  int I, J, KK;
+  if (t < (1 << 21)) cell_ijk_small(t, C, I, J, KK);
+  else cell_ijk(t, C.nx, C.ny, I, J, KK);
+  constexpr int NZ = DIM == 3 ? 2 : 1;
+  const int sy = F.nx, sz = F.nx * F.ny;
+  const int c0 = 2 * I + sy * 2 * J + (DIM == 3 ? sz * 2 * KK : 0);
+  const bool xm = I > 0, xp = 2 * I + 2 < F.nx, ym = J > 0, yp = 2 * J + 2 < F.ny;
+  const bool zm = DIM == 3 && KK > 0, zp = DIM == 3 && 2 * KK + 2 < F.nz;
+  auto ld2 = [](const double* x, int c) { return *reinterpret_cast<const double2*>(x + c); };
+  double2 ph[NZ][2], mu[NZ][2], pr[NZ][2];
 #pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = T(0);
-  if (valid) {
-    int c = i + F.nx * (j + F.ny * k);
-    T n1, n2, n3;
-    eval_N<T, DIM, CORR>(F, K, F.phi, F.mu, F.p, c, i, j, k, n1, n2, n3);
-    v[0] = F.fphi[c] - n1;
-    v[1] = F.fmu[c] - n2;
-    v[2] = F.fp[c] - n3;
-    v[3] = F.phi[c];
-    v[4] = F.mu[c];
-    v[5] = F.p[c];
-    if (CORR) v[NV - 1] = F.phib[c];
-  }
+  for (int dk = 0; dk < NZ; ++dk)
 #pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    v[q] += __shfl_xor_sync(0xffffffffu, v[q], 1);
-    v[q] += __shfl_xor_sync(0xffffffffu, v[q], TX);
-    if (DIM == 3) v[q] += __shfl_xor_sync(0xffffffffu, v[q], 16);
-  }
-  const bool leader = valid && (lane & 1) == 0 && ((lane / TX) & 1) == 0 && (DIM == 2 || lane < 16);
-  if (!leader) return;
-  const T w = DIM == 3 ? T(0.125) : T(0.25);
-  int q = (i >> 1) + C.nx * ((j >> 1) + C.ny * (k >> 1));
-  C.fphi[q] = w * v[0];
-  C.fmu[q] = w * v[1];
-  C.fp[q] = w * v[2];
-  C.phi[q] = C.phi0[q] = w * v[3];
-  C.mu[q] = C.mu0[q] = w * v[4];
-  C.p[q] = C.p0[q] = w * v[5];
-  if (CORR) C.phib[q] = w * v[NV - 1];
+    for (int dj = 0; dj < 2; ++dj) {
+      const int c = c0 + dj * sy + dk * sz;
+      ph[dk][dj] = ld2(F.phi, c);
+      mu[dk][dj] = ld2(F.mu, c);
+      pr[dk][dj] = ld2(F.p, c);
+    }
+  // sums over the outer faces: v = M dmu + a dp, aw = a dmu, w = dp, sd = outside phi
+  double v = 0.0, aw = 0.0, w = 0.0, sd = 0.0;
+  auto face = [&](double phe, double mue, double pe, double muc, double pc, double a, double M) {
+    const double dmu = mue - muc, dp = pe - pc;
+    v = ::fma(M, dmu, v);
+    v = ::fma(a, dp, v);
+    aw = ::fma(a, dmu, aw);
+    w += dp;
+    sd += phe;
+  };
+  auto pair = [&](int e, int fc, const double* af, const double* Mf, const double2& muc, const double2& pc) {
+    const double2 phe = ld2(F.phi, e), mue = ld2(F.mu, e), pe = ld2(F.p, e), a = ld2(af, fc), M = ld2(Mf, fc);
+    face(phe.x, mue.x, pe.x, muc.x, pc.x, a.x, M.x);
+    face(phe.y, mue.y, pe.y, muc.y, pc.y, a.y, M.y);
+  };
+#pragma unroll
+  for (int dk = 0; dk < NZ; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) {
+      const int c = c0 + dj * sy + dk * sz;
+      if (xm) face(F.phi[c - 1], F.mu[c - 1], F.p[c - 1], mu[dk][dj].x, pr[dk][dj].x, F.ax[c - 1], F.Mx[c - 1]);
+      if (xp) face(F.phi[c + 2], F.mu[c + 2], F.p[c + 2], mu[dk][dj].y, pr[dk][dj].y, F.ax[c + 1], F.Mx[c + 1]);
+      if (dj == 0 && ym) pair(c - sy, c - sy, F.ay, F.My, mu[dk][dj], pr[dk][dj]);
+      if (dj == 1 && yp) pair(c + sy, c, F.ay, F.My, mu[dk][dj], pr[dk][dj]);
+      if (DIM == 3) {
+        if (dk == 0 && zm) pair(c - sz, c - sz, F.az, F.Mz, mu[dk][dj], pr[dk][dj]);
+        if (dk == NZ - 1 && zp) pair(c + sz, c, F.az, F.Mz, mu[dk][dj], pr[dk][dj]);
+      }
+    }
+  // the cells' own terms and the restricted state
+  double sph = 0.0, smu = 0.0, sp = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll
+  for (int dk = 0; dk < NZ; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) {
+      const int c = c0 + dj * sy + dk * sz;
+      const double2 f1 = ld2(F.fphi, c), f2 = ld2(F.fmu, c), f3 = ld2(F.fp, c), H = ld2(F.cH, c), Q = ld2(F.cQ, c);
+      const double2 u = ph[dk][dj];
+      sph += u.x + u.y;
+      smu += mu[dk][dj].x + mu[dk][dj].y;
+      sp += pr[dk][dj].x + pr[dk][dj].y;
+      s1 += f1.x + f1.y;
+      s3 += f3.x + f3.y;
+      s2 += f2.x + f2.y;
+      s2 = ::fma(::fma(::fma(0.25, u.x, H.x), u.x, Q.x), u.x, s2);
+      s2 = ::fma(::fma(::fma(0.25, u.y, H.y), u.y, Q.y), u.y, s2);
+    }
+  const double r1 = ::fma(F.sih2, v, s1 - sph);
+  // over the inner faces every cell is a neighbour DIM times
+  const double r2 = ::fma(-F.e34ih2, ::fma((double)DIM, sph, sd), s2 - smu);
+  const double r3 = ::fma(F.ih2, ::fma(K.gamma, aw, w), s3);
+  const double q = DIM == 3 ? 0.125 : 0.25;
+  C.fphi[t] = q * r1;
+  C.fmu[t] = q * r2;
+  C.fp[t] = q * r3;
+  C.phi[t] = C.phi0[t] = q * sph;
+  C.mu[t] = C.mu0[t] = q * smu;
+  C.p[t] = C.p0[t] = q * sp;
 }
 
 // One row of the plain form's N at cell c, on the fields (phi, mu, p):
@@ -810,7 +857,7 @@ __device__ __forceinline__ double* f_row(const Level<double>& F, int role) {
   return role == 0 ? F.fphi : role == 1 ? F.fp : F.fmu;
 }
 
-// k_residual_restrict for small double-precision levels (plain form): the
+// The same for small double-precision levels, one thread per fine cell: the
 // three warps of a block take the phi, pressure and mu rows of the same
 // 16 x 2 (8 x 2 x 2) tile, so each warp's FP64 chain is a third as long.
 // Each row's coarse values depend on that row only, so the warps need no
