@@ -437,10 +437,10 @@ struct Enqueue {
                      int l) {
     const Coefs<T> K = coefs<T>(run);
     const Level<T>& L = lev[l];
-    if constexpr (std::is_same<T, double>::value && !CORR) {
+    if constexpr (std::is_same<T, double>::value && !CORR && DIM == 2) {
       if (l == run->cluster_start) {
         launch(run, s, CHHS_K_COARSEST, 1.0, [&] {
-          pdl_cluster(k_cluster<DIM>, run->cplan.blocks, kTailThreads, cluster_smem_bytes<DIM>(run->cluster, run->cplan),
+          pdl_cluster(k_cluster, run->cplan.blocks, kTailThreads, cluster_smem_bytes(run->cluster, run->cplan),
                       s, run->cluster, run->cplan, K, nu_pre(run, l), nu_post(run, l));
         });
         return;
@@ -997,14 +997,13 @@ void fill_tail(Tail<T>& tail, const std::vector<Level<T>>& lev, int start, const
 // precision).  In 3D a 16^3 level would leave a block 512 cells and 24 arrays
 // of them (196 KB), for passes that the FP64 pipes of 16 SMs bound anyway.
 // With split_threads 0 the handle asks for the grid-wide passes.
-template <int DIM>
 void place_cluster(chhs_t* run) {
   if (run->opts.precision != 0 || run->split_threads <= 0) return;
   const Layout& Lo = run->layout;
   const int nl = (int)Lo.shapes.size();
   int dev = 0, optin = 0;
   cudaFuncAttributes fa;
-  const void* fn = reinterpret_cast<const void*>(k_cluster<DIM>);
+  const void* fn = reinterpret_cast<const void*>(k_cluster);
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
       cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
@@ -1019,12 +1018,12 @@ void place_cluster(chhs_t* run) {
     tl.nu1 = run->nu1c;
     tl.nu2 = run->nu2c;
     ClusterPlan P{};
-    auto nrows = [&](int l) { return DIM == 3 ? tl.lev[l].nz : tl.lev[l].ny; };
+    auto nrows = [&](int l) { return tl.lev[l].ny; };
     P.blocks = 2;
     while (P.blocks < kClusterMax && 2 * P.blocks < nrows(0)) P.blocks *= 2;
     P.tail = run->tail_start - start;
     for (int l = 0; l < tl.n; ++l) P.rows[l] = l < P.tail ? cluster_rows(nrows(l), P.blocks) : nrows(l);
-    const size_t smem = cluster_smem_bytes<DIM>(tl, P);
+    const size_t smem = cluster_smem_bytes(tl, P);
     if (smem + fa.sharedSizeBytes > (size_t)optin) continue;
     if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -1043,7 +1042,7 @@ void place_cluster(chhs_t* run) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int fit = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit, k_cluster<DIM>, &cfg) != cudaSuccess || fit < 1) {
+    if (cudaOccupancyMaxActiveClusters(&fit, k_cluster, &cfg) != cudaSuccess || fit < 1) {
       cudaGetLastError();
       continue;
     }
@@ -1067,7 +1066,7 @@ void place_tail(chhs_t* run) {
   fill_tail(run->tail, run->lev, run->tail_start, run->opts, run->nu1c, run->nu2c);
   fill_tail(run->tail32, run->lev32, run->tail_start, run->opts, run->nu1c, run->nu2c);
   run->cluster_start = -1;
-  if (run->dim == 2) place_cluster<2>(run);
+  if (run->dim == 2) place_cluster(run);
 }
 
 chhs_status setup_handle(chhs_t* run) {
