@@ -895,9 +895,9 @@ struct Enqueue {
   }
 
   static chhs_status dissipation(chhs_t* run) {
-    const int nb = nblocks(run->ncell());
+    const int nb = run->norm_blocks;
     k_dissip_partial<DIM><<<nb, kBlock, 0, run->stream>>>(run->lev[0], run->gamma, 1.0 / run->h, run->partials);
-    k_dissip_finish<<<1, 32, 0, run->stream>>>(run->partials, nb, run->st);
+    k_dissip_finish<<<1, kBlock, 0, run->stream>>>(run->partials, nb, run->st);
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(run->host_st, run->st, sizeof(DevState), cudaMemcpyDeviceToHost, run->stream));
     CU(cudaStreamSynchronize(run->stream));
@@ -914,10 +914,10 @@ struct Enqueue {
 
   static chhs_status energy(chhs_t* run) {
     const int nx = run->n[0], ny = run->n[1], nz = run->n[2];
-    const int nb = nblocks(run->ncell());
+    const int nb = run->norm_blocks;
     k_energy_partial<DIM><<<nb, kBlock, 0, run->stream>>>(run->lev[0].phim, run->phimm1, nx, ny, nz,
                                                           1.0 / run->h, run->partials);
-    k_energy_finish<<<1, 1024, 0, run->stream>>>(run->partials, nb, run->st);
+    k_energy_finish<<<1, kBlock, 0, run->stream>>>(run->partials, nb, run->st);
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(run->host_st, run->st, sizeof(DevState), cudaMemcpyDeviceToHost, run->stream));
     CU(cudaStreamSynchronize(run->stream));
@@ -1713,8 +1713,11 @@ chhs_status chhs_autotune(chhs_t* run, int trial_steps, chhs_tuning* out) {
 chhs_status chhs_mass(chhs_t* run, double* mass_out) {
   if (!run || !mass_out) return fail(run, CHHS_ERR_INVALID_ARG, "NULL argument");
   run->err.clear();
-  chhs_status s = run->dim == 2 ? Enqueue<2>::energy(run) : Enqueue<3>::energy(run);
-  if (s != CHHS_OK) return s;
+  k_mass_partial<<<run->norm_blocks, kBlock, 0, run->stream>>>(run->lev[0].phim, run->ncell(), run->partials);
+  k_mass_finish<<<1, kBlock, 0, run->stream>>>(run->partials, run->norm_blocks, run->st);
+  CU(cudaGetLastError());
+  CU(cudaMemcpyAsync(run->host_st, run->st, sizeof(DevState), cudaMemcpyDeviceToHost, run->stream));
+  CU(cudaStreamSynchronize(run->stream));
   double hd = run->dim == 2 ? run->h * run->h : run->h * run->h * run->h;
   *mass_out = hd * run->host_st->diag[0];
   return CHHS_OK;
