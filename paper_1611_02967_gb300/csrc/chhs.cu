@@ -508,7 +508,7 @@ struct Enqueue {
     });
     vcycle<T, CORR>(run, s, lev, tail, l + 1);
     launch(run, s, CHHS_K_PROLONG, L.ncell, [&] {
-      pdl(k_prolong<T, DIM>, nblocks(L.ncell), kBlock, s, L, C);
+      pdl(k_prolong<T, DIM>, nblocks(C.ncell), kBlock, s, L, C);
     });
     smooth<T, CORR>(run, s, L, nu_post(run, l), false);
   }
@@ -562,7 +562,7 @@ struct Enqueue {
     vcycle<float, true>(run, s, lev, tail, l + 1);
     if (nu2 == 0) {
       launch(run, s, CHHS_K_PROLONG, L.ncell, [&] {
-        pdl(k_prolong<float, DIM>, nblocks(L.ncell), kBlock, s, L, C);
+        pdl(k_prolong<float, DIM>, nblocks(C.ncell), kBlock, s, L, C);
       });
       return;
     }
@@ -2162,7 +2162,7 @@ struct BatchStep {
     if (nu2 == 0) {
       JobList<PairJob> jl;
       runs_at([&](chhs_t* r, const Level<float>& L, const Level<float>& C) {
-        jl.add(PairJob{L, C, k32(r), Level<double>{}, gate(r)}, nblocks(L.ncell));
+        jl.add(PairJob{L, C, k32(r), Level<double>{}, gate(r)}, nblocks(C.ncell));
       });
       go(CHHS_K_PROLONG, jl, kb_prolong<DIM>, kBlock, 0, s);
       return;

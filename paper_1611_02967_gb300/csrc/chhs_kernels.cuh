@@ -909,17 +909,50 @@ __global__ void __launch_bounds__(96) k_residual_restrict_split(Level<double> F,
   }
 }
 
-// u += P(u_c - u_c^0), P piecewise constant.
+template <typename T>
+struct Pair;
+template <>
+struct Pair<float> {
+  using type = float2;
+};
+template <>
+struct Pair<double> {
+  using type = double2;
+};
+
+// u += P(u_c - u_c^0), P piecewise constant: a thread per coarse cell forms
+// its three differences once and adds them to its 2 x 2 (x 2) fine cells, a
+// pair of cells per access (a level that has a coarser one has even sides).
+// In double precision the FP64 instructions bound a thread per fine cell; this
+// has 27 for eight cells against 48 (128^3 step 13.65 -> 13.56 ms, 512^2 2.307 -> 2.298).
 template <typename T, int DIM>
 __device__ __forceinline__ void prolong_body(int bx, Level<T> F, Level<T> C) {
-  int c = bx * blockDim.x + threadIdx.x;
-  if (c >= F.ncell) return;
+  using T2 = typename Pair<T>::type;
+  const int q = bx * blockDim.x + threadIdx.x;
+  if (q >= C.ncell) return;
   int i, j, k;
-  cell_ijk(c, F.nx, F.ny, i, j, k);
-  int q = (i >> 1) + C.nx * ((j >> 1) + C.ny * (DIM == 3 ? (k >> 1) : 0));
-  F.phi[c] += C.phi[q] - C.phi0[q];
-  F.mu[c] += C.mu[q] - C.mu0[q];
-  F.p[c] += C.p[q] - C.p0[q];
+  cell_ijk(q, C.nx, C.ny, i, j, k);
+  const int c = 2 * i + F.nx * (2 * j + F.ny * (DIM == 3 ? 2 * k : 0));
+  constexpr int NR = DIM == 3 ? 4 : 2;  // rows of the fine cells
+  T2* row[3][NR];
+  T2 v[3][NR];
+  T* const u[3] = {F.phi, F.mu, F.p};
+  const T d[3] = {C.phi[q] - C.phi0[q], C.mu[q] - C.mu0[q], C.p[q] - C.p0[q]};
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      row[m][r] = reinterpret_cast<T2*>(u[m] + c + F.nx * ((r & 1) + F.ny * (r >> 1)));
+      v[m][r] = *row[m][r];
+    }
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      v[m][r].x += d[m];
+      v[m][r].y += d[m];
+      *row[m][r] = v[m][r];
+    }
 }
 
 template <typename T, int DIM>
