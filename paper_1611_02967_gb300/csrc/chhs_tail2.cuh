@@ -25,7 +25,7 @@ namespace chhs_dev {
 // do not depend on the V-cycle (the 12 face values, Ae, x, hn, em per cell).
 constexpr int kTail2Consts = 28;
 struct Tail2Level {
-  float4* s0;  // (phi, mu, p): position m (of 4) of block q at m nb + q
+  float4* s0;  // (mu, p, phi): position m (of 4) of block q at m nb + q
   float *u, *fs, *pms, *pbs, *qs, *cs;  // field k, position m of block q at (4 k + m) nb + q
   int hx, hy, nb;                       // blocks per row, rows, blocks
   __device__ __forceinline__ float4* s(int m, int q) const { return s0 + m * nb + q; }
@@ -78,9 +78,9 @@ struct Tail2Block {
 
 __device__ __forceinline__ TileCell tail2_get(const float4* p) {
   const float4 v = *p;
-  return TileCell{v.x, v.y, v.z};
+  return TileCell{v.z, v.x, v.y};
 }
-__device__ __forceinline__ void tail2_put(float4* p, const TileCell& c) { *p = make_float4(c.phi, c.mu, c.p, 0.f); }
+__device__ __forceinline__ void tail2_put(float4* p, const TileCell& c) { *p = make_float4(c.mu, c.p, c.phi, 0.f); }
 
 // The constants of block q of level L (global phi*, phi^m) into shared memory.
 __device__ __forceinline__ void tail2_constants(const Tail2Level& T, int q, const Level<float>& L,
@@ -284,7 +284,7 @@ __device__ __forceinline__ TileCell tail2_coarsest_block(const Level<float>& L, 
   const bool act = t < L.ncell;
   const int j = small_div(t, L.rnx), i = t - j * L.nx;
   TileCell u = q.u;
-  if (act) buf[t] = make_float4(u.phi, u.mu, u.p, ps);
+  if (act) buf[t] = make_float4(u.mu, u.p, u.phi, ps);
   __syncthreads();
   const bool in0 = act && i > 0, in1 = act && i + 1 < L.nx, in2 = act && j > 0, in3 = act && j + 1 < L.ny;
   const int own = act ? t : 0;
@@ -315,7 +315,7 @@ __device__ __forceinline__ TileCell tail2_coarsest_block(const Level<float>& L, 
     for (int colour = 0; colour < 2; ++colour) {
       if (act && ((i + j + colour) & 1) == 0) {
         tile_update(u, tail2_get(b0), tail2_get(b1), tail2_get(b2), tail2_get(b3), a0, a1, a2, a3, f1, f2, f3, k, L, K);
-        buf[t] = make_float4(u.phi, u.mu, u.p, ps);
+        buf[t] = make_float4(u.mu, u.p, u.phi, ps);
       }
       __syncthreads();
     }
@@ -390,7 +390,7 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   if (t < T0.nb) {
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      *T0.s(m, t) = make_float4(u[m], v[m], w[m], 0.f);
+      *T0.s(m, t) = make_float4(v[m], w[m], u[m], 0.f);
       T0.f(0, m, t) = g1[m];
       T0.f(1, m, t) = g2[m];
       T0.f(2, m, t) = g3[m];
