@@ -234,16 +234,20 @@ typedef struct {
   int split_threads;  /* double-precision levels with at most this many cells per colour
                          use the three-warp split update (0: never); unless 0, 2D levels of at
                          most 4096 cells run in one launch of a block cluster */
-  int tile_threads;   /* threads per tile on the 2D mixed form's levels of at least 512 x 256 cells */
+  int tile_threads;   /* accepted for the tiles of the 2D mixed form's levels of at least 512 x 256
+                         cells and not used: a tile has a thread per 2 x 2 cells, halo included.
+                         More than 512: CHHS_ERR_CUDA */
   int coarse_nu1;     /* pre- and post-smoothing sweeps on the levels below the finest (the finest */
   int coarse_nu2;     /* keeps opts->nu1, nu2) */
-  int tile_w, tile_h; /* interior of a tile on those levels (even; default 32 x 32 on 512 threads) */
+  int tile_w, tile_h; /* interior of a tile on those levels (even; default 32 x 32; at least 16 x 16
+                         is taken, and a side is halved where the halo would need more than 512
+                         threads; no shape changes a result) */
   int norm_f64_per8;  /* mixed form, double-single residual: the share of the residual kernel's
                          blocks that use double-precision instructions, so that the FP64 pipe works
                          beside the single-precision ones: n/128 for n in 0..7 (default 3), all of
                          them for 8 */
-  int small_tile_w, small_tile_h; /* 2D mixed form: tile interior on the smaller levels */
-  int small_tile_threads;         /* (default 16 x 8 cells on 256 threads) and its block size */
+  int small_tile_w, small_tile_h; /* the same on the smaller levels (default 16 x 8: taken as 16 x 16) */
+  int small_tile_threads;         /* as tile_threads (default 256) */
   int quad_passes;    /* 3D mixed form: 1 (default) runs the colour passes of levels whose x extent
                          is a multiple of 4 with one thread per four cells of a row (16-byte loads),
                          0 with one thread per cell; the results are the same bit for bit.  Not 0
@@ -472,9 +476,8 @@ chhs_status chhs_batch_step(chhs_batch_t* batch, int nsteps, int* status_out, in
  * graph; the runs' states are kept.  Of chhs_tuning the batch takes
  * tail_cells, coarse_nu1, coarse_nu2 and norm_f64_per8 (the same for all its
  * runs) and, in 2D, tile_w, tile_h and tile_threads for the per-run tile
- * launches of its large levels (default 32 x 32 cells on 512 threads; the
- * batched launch of the small levels keeps 32 x 16 on 512); the other fields
- * are ignored.  Errors:
+ * launches of its large levels (default 32 x 32 cells; the batched launch of
+ * the small levels keeps 32 x 16); the other fields are ignored.  Errors:
  * CHHS_ERR_INVALID_ARG (NULL, tail_cells < 1, coarse sweep counts < 0 or both
  * 0, norm_f64_per8 outside 0..8, a tile as chhs_set_tuning refuses, or a
  * setting some run cannot take -- the previous setting is then kept),

@@ -78,12 +78,11 @@ int level_fields(int dim, bool single) {
 constexpr int kNormF64Per8 = 3;
 
 // Tiles of the 2D single-precision levels: a level of at least
-// kLargeTileCells cells takes chhs_tuning's tile_* (default 32 x 32 cells on
-// 512 threads), a smaller one small_tile_* (default 16 x 8 on 256: four times
-// the blocks on the small, latency-bound levels).  On the 512^2 mixed step
-// 16 x 8 below the finest level measured 4% faster than 32 x 16 there, and
-// 32 x 32 on levels of 256 x 512 cells and more took the batched
-// configuration's large runs from 6.3e8 to 7.2e8 cell-steps/s.
+// kLargeTileCells cells takes chhs_tuning's tile_* (default 32 x 32 cells), a
+// smaller one small_tile_* (default 16 x 8, which tile_shape raises to 16 x
+// 16: four times the blocks of 32 x 32 on the small, latency-bound levels).
+// The thread counts are kept for the settings' sake; a tile's block has a
+// thread per 2 x 2 cells (chhs_tile.cuh, with the measurements).
 constexpr int kLargeTileW = 32, kLargeTileH = 32, kLargeTileThreads = 512;
 constexpr int kSmallTileW = 16, kSmallTileH = 8, kSmallTileThreads = 256;
 constexpr int kLargeTileCells = 512 * 256;

@@ -31,9 +31,13 @@
 // What bounds it: latency -- on small levels the load, the passes' block
 // barriers and the update's dependent chain, on large ones too: 127 registers
 // leave one block of 16 warps per SM, which issues 44 % of the time (ncu,
-// 2048^2: 67 M warp instructions, global loads the largest stall).  Two blocks
+// 2048^2, with seven instructions per face: 67 M warp instructions, global loads
+// the largest stall; five per face since, tile_face).  Two blocks
 // at 64 or three at 85 registers spill or cut smaller tiles and are slower
-// (2048^2 step 4.77 ms, 5.88 and 5.58).
+// (2048^2 step 4.77 ms, 5.88 and 5.58).  Blocks that stay and copy the next
+// tile's fields asynchronously during the passes sit at the register limit and
+// gave 0.86 to 1.03 times that speed as the compiler scheduled them (512^2
+// 0.99); L2 prefetches of a tile a wave ahead 0.95.
 // One cell per thread with all fields in shared memory and the coefficients
 // recomputed in every pass took twice the instructions; its 512^2 step 835 us
 // against 683, 640 x 384 1.12 -> 0.94 ms, batch of 24 15.4 -> 14.2 ms.
