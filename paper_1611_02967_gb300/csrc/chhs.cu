@@ -710,12 +710,15 @@ struct Enqueue {
   static int setup_mixed_blocks(const Level<float>& Gn) { return (Gn.ncell + kSetupBlock - 1) / kSetupBlock; }
 
   // Single-precision levels whose kernels read stored coefficients: the coarsest
-  // and a 3D tail of the general code, and in 3D those without a pre-smoothing
-  // sweep (k_coarse_rhs).  The others recompute them from phi*.
+  // and a 3D tail of the general code (the finest level too when it is in that
+  // tail), and in 3D the coarser ones without a pre-smoothing sweep
+  // (k_coarse_rhs).  The others recompute them from phi*.
   static bool stored_coefs(const chhs_t* run, int l) {
     if (DIM == 3 && l >= run->tail_start && !tail3_fits(run->tail32)) return true;
-    return l + 1 == (int)run->lev32.size() || (DIM == 3 && nu_pre(run, l) == 0);
+    return l + 1 == (int)run->lev32.size() || (DIM == 3 && l > 0 && nu_pre(run, l) == 0);
   }
+  // ... of which k_setup_mixed leaves the finest level's to k_coef_restrict.
+  static bool stored_finest(const chhs_t* run) { return setup_mixed(run) && stored_coefs(run, 0); }
 
   static void frame_setup(chhs_t* run, cudaStream_t s) {
     const Level<double>& F = run->lev[0];
@@ -754,6 +757,10 @@ struct Enqueue {
       launch(run, s, CHHS_K_FRAME, 1.0, [&] {
         pdl(k_coef_restrict_f32<DIM>, nblocks(F.ncell), kBlock, s, F, G[0], K32, ng > 1 ? G[1] : G[0],
             ng > 1 ? 1 : 0);
+      });
+    if (stored_finest(run))
+      launch(run, s, CHHS_K_FRAME, 1.0, [&] {
+        pdl(k_coef_restrict<float, DIM>, nblocks(G[0].ncell), kBlock, s, G[0], K32, G[0], 0, 1);
       });
     for (int l = 1; l < ng; ++l)
       launch(run, s, CHHS_K_FRAME, 1.0, [&] {
@@ -1996,6 +2003,11 @@ struct BatchStep {
              nblocks(r->lev[0].ncell));
     }
     go(CHHS_K_FRAME, jf, kb_coef_restrict_f32<DIM>, kBlock, 0, s);
+    JobList<CoefJob> j0;
+    for (chhs_t* r : b->runs)
+      if (Enqueue<DIM>::stored_finest(r))
+        j0.add(CoefJob{r->lev32[0], r->lev32[0], k32(r), 0, 1}, nblocks(r->lev32[0].ncell));
+    go(CHHS_K_FRAME, j0, kb_coef_restrict<DIM>, kBlock, 0, s);
     for (int l = 1; l < maxng; ++l) {
       JobList<CoefJob> jl;
       for (chhs_t* r : b->runs) {

@@ -1265,11 +1265,12 @@ __global__ void __launch_bounds__(kBlock) k_setup_coef(Level<double> L, const do
   setup_coef_body<DIM>(blockIdx.x, L, phimm1, eps2, st, K, Cn, has_next);
 }
 
-// The set-up of a mixed-precision step whose finest level is above the tail:
-// phi*, f_mu and the initial guess in double precision (the residual kernel
-// forms the coefficients from phi*, takes f_phi = phi^m and f_p = 0), phi^m
-// and phi* rounded for the finest single-precision level, and their
-// restriction to the next.
+// The set-up of a mixed-precision step whose finest level coarsens: phi*, f_mu
+// and the initial guess in double precision (the residual kernel forms the
+// coefficients from phi*, takes f_phi = phi^m and f_p = 0), phi^m and phi*
+// rounded for the finest single-precision level, and their restriction to the
+// next.  (A finest level inside a 3D tail of the general code gets its stored
+// coefficients from k_coef_restrict.)
 //
 // What bounds it: the FP64 pipe.  k_setup_coef with k_coef_restrict_f32 also
 // wrote 16 double- and 15 single-precision coefficient arrays that no kernel
