@@ -608,7 +608,8 @@ struct Enqueue {
   static size_t tail_bytes(const Tail<T>& tail) {
     int nc[kTailMaxLevels];
     for (int l = 0; l < tail.n; ++l) nc[l] = tail.lev[l].ncell;
-    return tail_smem_bytes<T, DIM, CORR>(nc, tail.n, tail.coarsest_f64);
+    const size_t general = tail_smem_bytes<T, DIM, CORR>(nc, tail.n, tail.coarsest_f64);
+    return use_tiles<T>() && tail.n >= 2 ? std::max(general, tail2_smem_bytes(nc, tail.n, tail.coarsest_f64)) : general;
   }
 
   // Opt the tail kernel in to the shared memory its levels need.

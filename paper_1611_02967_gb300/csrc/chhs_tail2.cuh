@@ -49,6 +49,29 @@ struct Tail2Scalars {
   int hx, hy, nb, off;
 };
 
+// What the block shares beside the levels, at the start of the dynamic shared
+// memory: as static memory it would also be taken from the largest one-level
+// grids of k_tail, which need all of a block's.
+struct Tail2Shared {
+  Tail2Scalars sc[kTailMaxLevels];  // of the levels above the coarsest; [n - 1].off: their end
+  float red[kTailThreads / 32];
+};
+constexpr size_t kTail2Head = (sizeof(Tail2Shared) + 15) / 16 * 16;
+
+// Shared memory of tail2_body: its levels take 84 bytes a cell where the general
+// code's take 92, so that only tails of less than 64 cells above the coarsest
+// need more than tail_smem_bytes.
+__host__ __device__ inline size_t tail2_smem_bytes(const int* ncell, int n, int coarsest_f64) {
+  size_t b = kTail2Head;
+  for (int l = 0; l + 1 < n; ++l) b += tail2_level_bytes(ncell[l] >> 2);
+  if (!coarsest_f64) return b + (ncell[n - 1] > 32 ? sizeof(float4) * ncell[n - 1] : 0);
+  return b + tail_smem_bytes<float, 2, true>(ncell + n - 1, 1, 1);
+}
+// A level of more than 2 x 2 cells per thread would not fit beside the coarsest
+// in a block's 227 KB: no check of its own is needed.
+static_assert((size_t)(227 * 1024) / (5 * tail_fields<2, true>()) <= 4 * kTailThreads,
+              "a two-level tail that fits in shared memory has a thread per 2 x 2 cells");
+
 __device__ __forceinline__ Tail2Level tail2_level(const Tail2Scalars& L, unsigned char* smem) {
   Tail2Level T;
   T.hx = L.hx;
@@ -330,11 +353,12 @@ __device__ __forceinline__ void tail2_body(const Tail<float>& tl, const Coefs<fl
   const Level<float>& Gc = tl.lev[n - 1];
   const bool general = tl.coarsest_f64 != 0;              // the coarsest solve on the general code
   const bool lanes = Gc.ncell <= 32 && !general;          // the coarsest grid on the lanes of warp 0
-  __shared__ float red[kTailThreads / 32];
-  __shared__ Tail2Scalars sc[kTailMaxLevels];  // of the levels above the coarsest; [n - 1].off: their end
+  Tail2Shared& shared = *reinterpret_cast<Tail2Shared*>(smem);
+  float* const red = shared.red;
+  Tail2Scalars* const sc = shared.sc;
   if (t < n) {
     const Level<float>& G = tl.lev[t];
-    size_t off = 0;
+    size_t off = kTail2Head;
     for (int q = 0; q < t; ++q) off += tail2_level_bytes(tl.lev[q].ncell >> 2);
     const int hx = G.nx >> 1;
     sc[t] = Tail2Scalars{G.ih2, G.h2, G.sih2, G.e34ih2, __frcp_rn((float)max(hx, 1)), hx, G.ny >> 1, G.ncell >> 2, (int)off};
