@@ -236,7 +236,7 @@ typedef struct {
                          most 4096 cells run in one launch of a block cluster */
   int tile_threads;   /* accepted for the tiles of the 2D mixed form's levels of at least 512 x 256
                          cells and not used: a tile has a thread per 2 x 2 cells, halo included.
-                         More than 512: CHHS_ERR_CUDA */
+                         More than 512 where the grid has such a level: CHHS_ERR_INVALID_ARG */
   int coarse_nu1;     /* pre- and post-smoothing sweeps on the levels below the finest (the finest */
   int coarse_nu2;     /* keeps opts->nu1, nu2) */
   int tile_w, tile_h; /* interior of a tile on those levels (even; default 32 x 32; at least 16 x 16
@@ -247,7 +247,7 @@ typedef struct {
                          beside the single-precision ones: n/128 for n in 0..7 (default 3), all of
                          them for 8 */
   int small_tile_w, small_tile_h; /* the same on the smaller levels (default 16 x 8: taken as 16 x 16) */
-  int small_tile_threads;         /* as tile_threads (default 256) */
+  int small_tile_threads;         /* as tile_threads, for the smaller levels (default 256) */
   int quad_passes;    /* 3D mixed form: 1 (default) runs the colour passes of levels whose x extent
                          is a multiple of 4 with one thread per four cells of a row (16-byte loads),
                          0 with one thread per cell; the results are the same bit for bit.  Not 0

@@ -648,8 +648,10 @@ struct Enqueue {
       if (std::max(tile_limit_bytes(halo, run->tile_w, run->tile_h),
                    tile_limit_bytes(halo, run->stile_w, run->stile_h)) > (size_t)optin)
         return fail(run, CHHS_ERR_INVALID_ARG, "nu1/nu2 too large for the single-precision tiles");
-      if (std::max(run->tile_threads, run->stile_threads) > kTileThreads)
-        return fail(run, CHHS_ERR_CUDA, "more threads than a tile's block has");
+      // a block size that no block may have is refused where a level asks for it
+      for (int l = 0; l < run->tail_start; ++l)
+        if ((run->lev32[l].ncell >= kLargeTileCells ? run->tile_threads : run->stile_threads) > kTileThreads)
+          return fail(run, CHHS_ERR_INVALID_ARG, "more threads than a tile's block has");
     }
     return CHHS_OK;
   }
@@ -2230,7 +2232,9 @@ struct BatchStep {
       const int halo = 2 * std::max(std::max(b->opts.nu1, b->opts.nu2), std::max(b->runs[0]->nu1c, b->runs[0]->nu2c)) + 1;
       if (std::max(tile_limit_bytes(halo, kTileW, kTileH), tile_limit_bytes(halo, b->big_tw, b->big_th)) > (size_t)optin)
         return bfail(b, CHHS_ERR_INVALID_ARG, "a run's coarse tail or tiles need more shared memory than a block has");
-      if (b->big_tt > kTileThreads) return bfail(b, CHHS_ERR_CUDA, "more threads than a tile's block has");
+      for (const chhs_t* r : b->runs)
+        if (r->tail_start > 0 && r->lev32[0].ncell >= kSoloTileCells && b->big_tt > kTileThreads)
+          return bfail(b, CHHS_ERR_INVALID_ARG, "more threads than a tile's block has");
     }
     auto raise_to = [&](const void* fn, size_t dyn) -> chhs_status {
       cudaFuncAttributes fa;

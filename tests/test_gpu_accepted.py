@@ -1,6 +1,7 @@
 """Grids and settings at the limits of what the mixed form accepts: the largest
 2D grids that a block's shared memory holds as one level (2 524 cells) or two
-(42 x 48, chhs_tuning.tail_cells 2048), alone and in a batch."""
+(42 x 48, chhs_tuning.tail_cells 2048), alone and in a batch, and block sizes
+of tiles, which matter only where a level of the grid asks for them."""
 import numpy as np
 import pytest
 
@@ -59,3 +60,19 @@ def test_one_more_cell_is_refused():
         with pytest.raises(chhs.ChhsError) as e:
             _steps(shape, tuning=((4096, 8192, 512, 2, 2), {}))
         assert e.value.status == chhs.CHHS_ERR_INVALID_ARG
+
+
+def test_tile_threads_matter_only_to_levels_that_ask_for_them():
+    shape = (128, 128)  # every level above the tail is a small one
+    ref = _steps(shape)
+    assert _same(ref, _steps(shape, tuning=((1024, 8192, 1024, 2, 2), {})))
+    assert _same(ref, _steps(shape, refused=((1024, 8192, 512, 2, 2), dict(small_tile=(16, 8, 1024)))))
+    shape = (512, 512)  # the finest level is a large one
+    assert _same(_steps(shape), _steps(shape, refused=((1024, 8192, 1024, 2, 2), {})))
+    opts = chhs.default_opts(precision=1)
+    with chhs.Batch([((64, 64), H, EPS, GAMMA, DT)], opts=opts) as b:
+        b.set_tuning(1024, 2, 2, tile=(32, 32, 1024))
+    with chhs.Batch([(shape, H, EPS, GAMMA, DT)], opts=opts) as b:
+        with pytest.raises(chhs.ChhsError):
+            b.set_tuning(1024, 2, 2, tile=(32, 32, 1024))
+        b.step(1)
