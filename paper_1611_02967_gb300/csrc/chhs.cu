@@ -1568,7 +1568,6 @@ chhs_status chhs_set_tuning(chhs_t* run, const chhs_tuning* t) {
       !tile_ok(t->small_tile_w, t->small_tile_h, t->small_tile_threads) || t->norm_f64_per8 < 0 ||
       t->norm_f64_per8 > 8 || (t->quad_passes != 0 && t->quad_passes != 1))
     return fail(run, CHHS_ERR_INVALID_ARG, "invalid tuning");
-  run->norm_f64_per8 = t->norm_f64_per8;
   run->err.clear();
   CU(cudaStreamSynchronize(run->stream));
   const chhs_tuning keep = current_tuning(run);

@@ -1,7 +1,8 @@
 """Grids and settings at the limits of what the mixed form accepts: the largest
 2D grids that a block's shared memory holds as one level (2 524 cells) or two
 (42 x 48, chhs_tuning.tail_cells 2048), alone and in a batch, and block sizes
-of tiles, which matter only where a level of the grid asks for them."""
+of tiles, which matter only where a level of the grid asks for them.  A refused
+setting leaves the one before in force, bit for bit."""
 import numpy as np
 import pytest
 
@@ -76,3 +77,12 @@ def test_tile_threads_matter_only_to_levels_that_ask_for_them():
         with pytest.raises(chhs.ChhsError):
             b.set_tuning(1024, 2, 2, tile=(32, 32, 1024))
         b.step(1)
+
+
+def test_refused_tuning_changes_nothing():
+    shape = (64, 64)
+    ref = _steps(shape, 2)
+    # the whole grid in the tail: no room in shared memory
+    assert _same(ref, _steps(shape, 2, refused=((4096, 8192, 512, 1, 1), dict(norm_f64_per8=8))))
+    # what a setting left behind would have shown
+    assert not _same(ref, _steps(shape, 2, tuning=((1024, 8192, 512, 2, 2), dict(norm_f64_per8=8))))
