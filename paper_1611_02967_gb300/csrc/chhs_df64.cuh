@@ -84,13 +84,22 @@ DF_HD float df_from_bits(uint32_t b) {
 #endif
 }
 
+DF_HD float df_from_uint(uint32_t m) {  // rounded to nearest
+#if defined(__CUDA_ARCH__)
+  return __uint2float_rn(m);
+#else
+  return (float)m;
+#endif
+}
+
 // x split into hi + lo with integer and single-precision operations only (a
-// conversion instruction runs at the double-precision rate on this GPU): hi
-// is x with its significand cut to 24 bits, lo the next 23 bits (the last 6
-// of the 53 are dropped), so |x - (hi + lo)| < 2^-46 |x|.  Magnitudes below 2^-126 give 0
-// (an absolute error far below anything the residual resolves), magnitudes
-// beyond the float range and non-finite values give +-infinity in hi, so a
-// non-finite state still yields a non-finite residual.
+// conversion from double runs at the double-precision rate on this GPU): hi is
+// x with its significand cut to 24 bits, lo the other 29 rounded to 24, so
+// |x - (hi + lo)| <= 2^-48 |x|.  (The residual's error is mostly that of its
+// inputs: with lo cut to 23 bits, 2^-46, it was twice as large.)  Magnitudes
+// below 2^-126 give 0 (an absolute error far below anything the residual
+// resolves), magnitudes beyond the float range and non-finite values give
+// +-infinity in hi, so a non-finite state still yields a non-finite residual.
 DF_HD df64 df_split(double x) {
   const uint64_t b = df_bits(x);
   const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
@@ -99,10 +108,8 @@ DF_HD df64 df_split(double x) {
   if (e < 897) return df64{df_from_bits(sign), 0.f};
   if (e > 1150) return df64{df_from_bits(sign | 0x7F800000u), 0.f};
   const float hi = df_from_bits(sign | ((uint32_t)(e - 896) << 23) | ((hw & 0xFFFFFu) << 3) | (lw >> 29));
-  // the next 23 significand bits as an exact float integer m (the bits of
-  // 2^23 + m, minus 2^23), scaled by 2^(e - 1069): their place value
-  const uint32_t m = (lw & 0x1FFFFFFFu) >> 6;
-  const float mf = df_fsub(df_from_bits(0x4B000000u | m), 8388608.0f);
+  // the place value of the last bit is 2^(e - 1075), here as 2^-6 2^(e - 1069)
+  const float mf = df_fmul(df_from_uint(lw & 0x1FFFFFFFu), 0.015625f);
   const int se = e - 942;
   const float scale = se > 0 ? df_from_bits((uint32_t)se << 23) : 0.f;
   const float lo_mag = df_fmul(mf, scale);
@@ -143,11 +150,13 @@ DF_HD df64 df_mul(df64 x, df64 y) {
   return df_quick_sum(p, e);
 }
 
-// Sum and product without the renormalisation, for sums of differences: the
-// high parts' sum with its error, the low parts added to it.  Exact to 2^-46
-// of the larger operand like df_add and df_mul, but after a cancellation the
-// result's low part may be as large as its high part (every operation here
-// takes such pairs); 8 and 4 instructions instead of 11 and 7.
+// Sum and product without the renormalisation (8 and 4 instructions instead of
+// 11 and 7): the high parts' sum with its error, the low parts added to it.
+// The sum is exact to 2^-44 of the larger operand, the product of freshly split
+// numbers to 2^-43 of itself.  After a cancellation the result's low part may
+// be as large as its high part, and a product with it, which drops the low
+// parts' product, is exact to 2^-44 of the product of the magnitudes before the
+// cancellation; df_mul_wide keeps that product for such a factor.
 DF_HD df64 df_add_raw(df64 x, df64 y) {
   const df64 s = df_two_sum(x.hi, y.hi);
   return df64{s.hi, df_fadd(s.lo, df_fadd(x.lo, y.lo))};
@@ -158,6 +167,14 @@ DF_HD df64 df_sub_raw(df64 x, df64 y) { return df_add_raw(x, df_neg(y)); }
 DF_HD df64 df_mul_raw(df64 x, df64 y) {
   const float p = df_fmul(x.hi, y.hi);
   float e = df_ffma(x.hi, y.hi, -p);
+  e = df_ffma(x.hi, y.lo, e);
+  return df64{p, df_ffma(x.lo, y.hi, e)};
+}
+
+DF_HD df64 df_mul_wide(df64 x, df64 y) {
+  const float p = df_fmul(x.hi, y.hi);
+  float e = df_ffma(x.hi, y.hi, -p);
+  e = df_ffma(x.lo, y.lo, e);
   e = df_ffma(x.hi, y.lo, e);
   return df64{p, df_ffma(x.lo, y.hi, e)};
 }

@@ -13,8 +13,9 @@
 // (N2 and f_mu carry the same constant shift (phi^m)^3/4 as the
 // double-precision kernels, see cubic_P; f_phi = phi^m and f_p = 0 on the
 // finest level), with every double input split into hi + lo and every
-// operation a double-single one: the residual is exact to ~1e-14 relative to
-// the terms, far below the 1e-10 stopping tolerance.
+// operation a double-single one (chhs_ndf.cuh, with the error measured against
+// 64 bits): exact to ~2^-44 of the largest term, far below the 1e-10 stopping
+// tolerance.
 //
 // What bounds it: issue slots (a double-single addition is 8 instructions),
 // so the work per cell is kept small.  In 3D a block takes a column of 32 x 8
@@ -33,7 +34,7 @@
 #pragma once
 #include <type_traits>
 
-#include "chhs_df64.cuh"
+#include "chhs_ndf.cuh"
 #include "chhs_kernels.cuh"
 
 namespace chhs_dev {
@@ -81,51 +82,21 @@ struct DfCoefs {
 // small, n/128 of the blocks, and they are the launch's first (256^3: 497 us
 // without, 499 us with 3/128, 581 with 3/32, 919 with 3/8; a share of 3/8 had
 // paid while the double-single blocks spent twice the instructions).
-struct NdfSingle {
-  using V = df64;
-  static __device__ __forceinline__ V from(double x) { return df_split(x); }
-  static __device__ __forceinline__ V add(V a, V b) { return df_add_raw(a, b); }
-  static __device__ __forceinline__ V sub(V a, V b) { return df_sub_raw(a, b); }
-  static __device__ __forceinline__ V mul(V a, V b) { return df_mul_raw(a, b); }
-  static __device__ __forceinline__ V fma(V a, V b, V c) { return df_add_raw(df_mul_raw(a, b), c); }
-  static __device__ __forceinline__ V half(V a) { return df64{0.5f * a.hi, 0.5f * a.lo}; }
-  static __device__ __forceinline__ V zero() { return df64{0.f, 0.f}; }
-  static __device__ __forceinline__ float cut(V a) { return df_to_float(a); }
-  static __device__ __forceinline__ float base(V a) { return a.hi; }
-};
 struct NdfDouble {
   using V = double;
   static __device__ __forceinline__ V from(double x) { return x; }
   static __device__ __forceinline__ V add(V a, V b) { return a + b; }
   static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
+  static __device__ __forceinline__ V diff(V a, V b) { return a - b; }
   static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ V mul_wide(V a, V b) { return a * b; }
   static __device__ __forceinline__ V fma(V a, V b, V c) { return ::fma(a, b, c); }
+  static __device__ __forceinline__ V fma_wide(V a, V b, V c) { return ::fma(a, b, c); }
   static __device__ __forceinline__ V half(V a) { return 0.5 * a; }
   static __device__ __forceinline__ V zero() { return 0.0; }
   static __device__ __forceinline__ float cut(V a) { return f64_to_f32_rz(a); }
   static __device__ __forceinline__ float base(V a) { return f64_to_f32_rz(a); }
 };
-
-// A face's fluxes from the cell below it to the one above, and the four
-// fields of a cell (phi, mu, p, phi*).
-template <class A>
-struct NdfFlux {
-  typename A::V v, w, d;
-};
-template <class A>
-struct NdfCell {
-  typename A::V phi, mu, p, ps;
-};
-
-template <class A>
-__device__ __forceinline__ NdfFlux<A> ndf_face(const NdfCell<A>& lo, const NdfCell<A>& hi, typename A::V gamma) {
-  NdfFlux<A> F;
-  const typename A::V a = A::half(A::add(lo.ps, hi.ps)), dmu = A::sub(hi.mu, lo.mu);
-  F.d = A::sub(hi.phi, lo.phi);
-  F.w = A::fma(gamma, A::mul(a, dmu), A::sub(hi.p, lo.p));
-  F.v = A::fma(a, F.w, dmu);
-  return F;
-}
 
 // Block sums: thread 0 returns the sum of squares, the double-single sum of
 // p and the maximum.
@@ -204,12 +175,8 @@ struct NdfOut {
   double s64;
   SUMS& sums;
   __device__ __forceinline__ void cell(int c, const NdfCell<A>& u, V sv, V sw, V sd, double pm64, double fmu64) {
-    const V pm = A::from(pm64);
-    const V r1 = A::fma(sih2, sv, A::sub(pm, u.phi));
-    const V quad = A::fma(u.phi, A::add(u.phi, pm), A::mul(pm, pm));
-    const V cub = A::half(A::half(A::mul(u.phi, quad)));
-    const V r2 = A::sub(A::add(A::sub(A::from(fmu64), u.mu), cub), A::mul(e34ih2, sd));
-    const V r3 = A::mul(ih2, sw);
+    V r1, r2, r3;
+    ndf_residual<A>(u, sv, sw, sd, A::from(pm64), A::from(fmu64), sih2, ih2, e34ih2, r1, r2, r3);
     const float r1f = A::cut(r1), r2f = A::cut(r2), r3f = A::cut(r3);
     if constexpr (std::is_same<SUMS, NdfSums64>::value) {
       sums.add(r1, r2, s64 * r3);
