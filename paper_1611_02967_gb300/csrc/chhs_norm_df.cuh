@@ -98,18 +98,24 @@ struct NdfDouble {
   static __device__ __forceinline__ float base(V a) { return f64_to_f32_rz(a); }
 };
 
-// Block sums: thread 0 returns the sum of squares, the double-single sum of
-// p and the maximum.
-__device__ __forceinline__ void ndf_block_reduce(float& sq, df64& ps, float& mx) {
-  __shared__ float s_sq[kNdfTX * kNdfTY / 32], s_mx[kNdfTX * kNdfTY / 32];
-  __shared__ df64 s_ps[kNdfTX * kNdfTY / 32];
+// Block sums: thread 0 returns the double-single sums of squares and of p and
+// the maximum.  (An overflow stays an infinity: the error term of an infinite
+// sum is not a number, so the plain sum is kept beside it.)
+__device__ __forceinline__ void ndf_block_reduce(df64& sq, df64& ps, float& mx) {
+  __shared__ float s_mx[kNdfTX * kNdfTY / 32];
+  __shared__ df64 s_sq[kNdfTX * kNdfTY / 32], s_ps[kNdfTX * kNdfTY / 32];
+  auto below = [](df64 a, int o) {
+    return df64{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};
+  };
+  float plain = sq.hi;
   for (int o = 16; o > 0; o >>= 1) {
-    sq += __shfl_down_sync(0xffffffffu, sq, o);
+    plain += __shfl_down_sync(0xffffffffu, plain, o);
+    sq = df_add(sq, below(sq, o));
     mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    const df64 other{__shfl_down_sync(0xffffffffu, ps.hi, o), __shfl_down_sync(0xffffffffu, ps.lo, o)};
-    ps = df_add(ps, other);
+    ps = df_add(ps, below(ps, o));
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (!isfinite(plain)) sq = df64{plain, 0.f};
   if (lane == 0) {
     s_sq[wid] = sq;
     s_mx[wid] = mx;
@@ -118,26 +124,30 @@ __device__ __forceinline__ void ndf_block_reduce(float& sq, df64& ps, float& mx)
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      sq += s_sq[w];
+      plain += s_sq[w].hi;
+      sq = df_add(sq, s_sq[w]);
       mx = fmaxf(mx, s_mx[w]);
       ps = df_add(ps, s_ps[w]);
     }
+    if (!isfinite(plain)) sq = df64{plain, 0.f};
   }
   __syncthreads();
 }
 
-// Sums of a block's cells: in single precision (p double-single) beside the
-// double-single residual, in double precision with f64_residual.
+// Sums of a block's cells: double-single beside the double-single residual (a
+// block's 4096 cells in single precision would lose several of its bits), in
+// double precision with f64_residual.
 struct NdfSums32 {
-  float sq = 0.f, mx = 0.f;
-  df64 ps{0.f, 0.f};
+  float mx = 0.f;
+  df64 sq{0.f, 0.f}, ps{0.f, 0.f};
   __device__ __forceinline__ void add(float r1, float r2, float r3s) {
-    sq += r1 * r1 + r2 * r2 + r3s * r3s;
+    const df64 s = df_two_sum(sq.hi, r1 * r1 + r2 * r2 + r3s * r3s);
+    sq = df64{s.hi, sq.lo + s.lo};
     mx = fmaxf(mx, fmaxf(fmaxf(fabsf(r1), fabsf(r2)), fabsf(r3s)));
   }
   __device__ __forceinline__ void finish(double (&out)[3]) {
     ndf_block_reduce(sq, ps, mx);
-    out[0] = (double)sq;
+    out[0] = df_to_double(sq);
     out[1] = df_to_double(ps);
     out[2] = (double)mx;
   }
