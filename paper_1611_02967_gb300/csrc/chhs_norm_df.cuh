@@ -98,34 +98,31 @@ struct NdfDouble {
   static __device__ __forceinline__ float base(V a) { return f64_to_f32_rz(a); }
 };
 
-// Block sums: thread 0 returns the double-single sums of squares and of p and
-// the maximum.  (An overflow stays an infinity: the error term of an infinite
-// sum is not a number, so the plain sum is kept beside it.)
+// Block sums: thread 0 returns the sum of squares (single precision within a
+// warp), the double-single sum of p and the maximum.  (An overflow stays an
+// infinity: the error term of an infinite sum is not a number.)
 __device__ __forceinline__ void ndf_block_reduce(df64& sq, df64& ps, float& mx) {
-  __shared__ float s_mx[kNdfTX * kNdfTY / 32];
-  __shared__ df64 s_sq[kNdfTX * kNdfTY / 32], s_ps[kNdfTX * kNdfTY / 32];
-  auto below = [](df64 a, int o) {
-    return df64{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};
-  };
-  float plain = sq.hi;
+  __shared__ float s_sq[kNdfTX * kNdfTY / 32], s_mx[kNdfTX * kNdfTY / 32];
+  __shared__ df64 s_ps[kNdfTX * kNdfTY / 32];
+  float plain = isfinite(sq.hi) ? sq.hi + sq.lo : sq.hi;
   for (int o = 16; o > 0; o >>= 1) {
     plain += __shfl_down_sync(0xffffffffu, plain, o);
-    sq = df_add(sq, below(sq, o));
     mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    ps = df_add(ps, below(ps, o));
+    const df64 other{__shfl_down_sync(0xffffffffu, ps.hi, o), __shfl_down_sync(0xffffffffu, ps.lo, o)};
+    ps = df_add(ps, other);
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (!isfinite(plain)) sq = df64{plain, 0.f};
   if (lane == 0) {
-    s_sq[wid] = sq;
+    s_sq[wid] = plain;
     s_mx[wid] = mx;
     s_ps[wid] = ps;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    sq = df64{plain, 0.f};
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      plain += s_sq[w].hi;
-      sq = df_add(sq, s_sq[w]);
+      plain += s_sq[w];
+      sq = df_add(sq, df64{s_sq[w], 0.f});
       mx = fmaxf(mx, s_mx[w]);
       ps = df_add(ps, s_ps[w]);
     }
@@ -134,9 +131,10 @@ __device__ __forceinline__ void ndf_block_reduce(df64& sq, df64& ps, float& mx) 
   __syncthreads();
 }
 
-// Sums of a block's cells: double-single beside the double-single residual (a
-// block's 4096 cells in single precision would lose several of its bits), in
-// double precision with f64_residual.
+// Sums of a block's cells: double-single over a thread's beside the
+// double-single residual (up to 16 cells; in single precision the squares lost
+// more than in the 256-cell blocks before), in double precision with
+// f64_residual.
 struct NdfSums32 {
   float mx = 0.f;
   df64 sq{0.f, 0.f}, ps{0.f, 0.f};
