@@ -242,10 +242,9 @@ typedef struct {
   int tile_w, tile_h; /* interior of a tile on those levels (even; default 32 x 32; at least 16 x 16
                          is taken, and a side is halved where the halo would need more than 512
                          threads; no shape changes a result) */
-  int norm_f64_per8;  /* mixed form, double-single residual: the share of the residual kernel's
-                         blocks that use double-precision instructions, so that the FP64 pipe works
-                         beside the single-precision ones: n/128 for n in 0..7 (default 3), all of
-                         them for 8 */
+  int norm_f64_per8;  /* mixed form: of every 8 blocks of the residual kernel, how many use
+                         double-precision instructions instead of double-single ones (0..8; default
+                         3).  Fewer than 4 are none: so few were a matter of speed, and do not pay */
   int small_tile_w, small_tile_h; /* the same on the smaller levels (default 16 x 8: taken as 16 x 16) */
   int small_tile_threads;         /* as tile_threads, for the smaller levels (default 256) */
   int quad_passes;    /* 3D mixed form: 1 (default) runs the colour passes of levels whose x extent

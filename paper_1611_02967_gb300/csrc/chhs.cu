@@ -73,8 +73,8 @@ int level_fields(int dim, bool single) {
   return kBaseFields + (dim == 3 ? 14 : 12) + (single ? 1 + (dim == 2 ? 6 : 0) : 0);
 }
 
-// The mixed form's residual kernel: the share of its blocks evaluated with
-// double-precision instructions, in 128ths (chhs_norm_df.cuh).
+// The mixed form's residual kernel: of every 8 of its blocks, how many use
+// double-precision instructions; fewer than 4 are none (chhs_norm_df.cuh).
 constexpr int kNormF64Per8 = 3;
 
 // Tiles of the 2D single-precision levels: a level of at least
@@ -214,7 +214,7 @@ struct chhs {
   // block size; chhs_autotune)
   int tile_w = kLargeTileW, tile_h = kLargeTileH;
   int stile_w = kSmallTileW, stile_h = kSmallTileH, stile_threads = kSmallTileThreads;
-  int norm_f64_per8 = kNormF64Per8;      // share of the residual's blocks on the FP64 pipe (mixed form)
+  int norm_f64_per8 = kNormF64Per8;      // of 8 blocks of the residual, how many on the FP64 pipe (mixed form)
   int quad_passes = 1;              // 3D mixed form: x-quad colour passes where nx % 4 == 0 (k_smooth_c4)
   Tail<double> tail{};              // its levels (double-precision V-cycles)
   Tail<float> tail32{};             // (single-precision inner V-cycles)
@@ -666,11 +666,14 @@ struct Enqueue {
   // The stopping norm (and, when mixed, the next inner solve's right-hand side).
   static void norm(chhs_t* run, cudaStream_t s, cudaGraphConditionalHandle cond, int mode, int use_cond) {
     const Coefs<double> K = coefs<double>(run);
+    const NdfMode arith = ndf_mode(run->norm_f64_per8, run->opts.f64_residual);
     const Level<double>& L = run->lev[0];
     const int nb = run->norm_blocks;
     launch(run, s, CHHS_K_NORM, L.ncell, [&] {
       if (mixed(run))
-        pdl(run->opts.f64_residual ? k_norm_mixed_df<DIM, true> : k_norm_mixed_df<DIM, false>,
+        pdl(arith == kNdfF64     ? k_norm_mixed_df<DIM, kNdfF64>
+            : arith == kNdfShare ? k_norm_mixed_df<DIM, kNdfShare>
+                                 : k_norm_mixed_df<DIM, kNdfSingle>,
             (int)ndf_blocks<DIM>(L.nx, L.ny, L.nz), kNdfTX * kNdfTY, s, L, df_coefs(run), K, run->norm_f64_per8,
             run->lev32[0], run->partials, run->st, cond, mode, use_cond);
       else
@@ -2032,7 +2035,11 @@ struct BatchStep {
       jl.add(NormJob{L, r->lev32[0], k64(r), Enqueue<DIM>::df_coefs(r), r->partials, r->st, r->norm_f64_per8},
              (int)ndf_blocks<DIM>(L.nx, L.ny, L.nz));
     }
-    go(CHHS_K_NORM, jl, b->opts.f64_residual ? kb_norm_mixed_df<DIM, true> : kb_norm_mixed_df<DIM, false>,
+    const NdfMode arith = ndf_mode(b->runs[0]->norm_f64_per8, b->opts.f64_residual);  // the same for all runs
+    go(CHHS_K_NORM, jl,
+       arith == kNdfF64     ? kb_norm_mixed_df<DIM, kNdfF64>
+       : arith == kNdfShare ? kb_norm_mixed_df<DIM, kNdfShare>
+                            : kb_norm_mixed_df<DIM, kNdfSingle>,
        kNdfTX * kNdfTY, 0, s, b->d_ticket, cc, mode, b->d_ticket + 1);
   }
 

@@ -179,7 +179,7 @@ __device__ __forceinline__ void batch_norm_epilogue(const NormJob* jobs, int njo
 // The stopping norms of all runs (mode 0: start of a step, every run; mode 1:
 // after a V-cycle, the runs still iterating).  Each run's last block takes
 // that run's decision.
-template <int DIM, bool F64>
+template <int DIM, int MODE>
 __global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) kb_norm_mixed_df(const NormJob* jobs, const int* start, int njobs,
                                                                   unsigned int* ticket, const BatchConds* cc,
                                                                   int mode, unsigned int* any_out) {
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) kb_norm_mix
   const int lb = blockIdx.x - start[j];
   bool reports = lb == 0;
   if (mode == 0 || gate_open(&J.st->go))
-    reports = norm_mixed_df_body<DIM, F64>(lb, start[j + 1] - start[j], J.L, J.Kdf, J.K, J.f64_per8, J.G, J.partials,
+    reports = norm_mixed_df_body<DIM, MODE>(lb, start[j + 1] - start[j], J.L, J.Kdf, J.K, J.f64_per8, J.G, J.partials,
                                       J.st, 0, mode, 0);
   batch_norm_epilogue(jobs, njobs, reports, ticket, cc, any_out);
 }

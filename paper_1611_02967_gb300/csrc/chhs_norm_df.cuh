@@ -29,8 +29,8 @@
 // Measured per launch (GB300, kernel by kernel with events), against a kernel
 // of one plane per block that read the stored a and M, formed each flux on
 // both sides and ran three of eight tiles on the FP64 pipe (~1 460
-// instructions per cell): 256^3 1056 -> 491 us, 128^3 159 -> 93 us,
-// 2048^2 231 -> 136 us.
+// instructions per cell): 256^3 1056 -> 510 us, 128^3 159 -> 85 us,
+// 2048^2 231 -> 133 us.
 #pragma once
 #include <type_traits>
 
@@ -75,13 +75,22 @@ struct DfCoefs {
   float s;
 };
 
-// The residual's arithmetic: double-single, or double precision for the share
-// of the blocks that runs on the FP64 pipe (chhs_tuning.norm_f64_per8, or all
-// with chhs_opts.f64_residual).  Both are 8 bytes a value.  A block on the
-// FP64 pipe takes ~5 times as long as one beside it, so the share's unit is
-// small, n/128 of the blocks, and they are the launch's first (256^3: 497 us
-// without, 499 us with 3/128, 581 with 3/32, 919 with 3/8; a share of 3/8 had
-// paid while the double-single blocks spent twice the instructions).
+// The residual's arithmetic (A): double-single (NdfSingle), or double precision
+// for blocks that run on the FP64 pipe.  Both are 8 bytes a value.
+//
+// Which blocks (chhs_tuning.norm_f64_per8, chhs_opts.f64_residual): from 4 on, so
+// many of every 8, as asked; below 4 none.  So few of them were a matter of
+// speed, the FP64 pipe working beside the others: 3 of 8 had paid while the
+// double-single blocks spent twice the instructions; now the FP64 pipe takes
+// longer over them than all blocks take without it (4 of 8 against none: 256^3
+// 991 us and 510, 128^3 179 and 85, 2048^2 289 and 133, 512^2 41 and 23), and the
+// double-single error is below that of such a mix (chhs_ndf.cuh).  With
+// f64_residual the sums are in double precision too.
+enum NdfMode { kNdfSingle = 0, kNdfShare = 1, kNdfF64 = 2 };
+__host__ __device__ inline NdfMode ndf_mode(int f64_per8, int f64_residual) {
+  return f64_residual ? kNdfF64 : f64_per8 >= 4 ? kNdfShare : kNdfSingle;
+}
+
 struct NdfDouble {
   using V = double;
   static __device__ __forceinline__ V from(double x) { return x; }
@@ -384,10 +393,9 @@ __device__ __forceinline__ void ndf_column(NdfShared& sh, int x0, int y0, int k0
 }
 
 // bx: the block's index among the run's nbx blocks (x-tiles fastest, then
-// y-tiles, then the chunks of planes; in 2D strips, then runs of rows).  F64: every block and the sums in
-// double precision (f64_residual).  Returns true in the run's last block
-// (which took the loop decision).
-template <int DIM, bool F64>
+// y-tiles, then the chunks of planes; in 2D strips, then runs of rows).  Returns
+// true in the run's last block (which took the loop decision).
+template <int DIM, int MODE>
 __device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<double>& L, const DfCoefs& K,
                                                    const Coefs<double>& K64, int f64_per8, const Level<float>& G,
                                                    double* partials, DevState* st, cudaGraphConditionalHandle cond,
@@ -409,14 +417,16 @@ __device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<
     }
   };
   double out[3];
-  if constexpr (F64) {
+  if constexpr (MODE == kNdfF64) {
     NdfSums64 sums;
     residual(NdfDouble{}, sums, L.sih2, L.ih2, L.e34ih2, K64.gamma);
     sums.finish(out);
   } else {
     NdfSums32 sums;
-    if (f64_per8 == 8 || bx < (int)((long long)nbx * f64_per8 / 128)) residual(NdfDouble{}, sums, L.sih2, L.ih2, L.e34ih2, K64.gamma);
-    else residual(NdfSingle{}, sums, K.sih2, K.ih2, K.e34ih2, K.gamma);
+    if (MODE == kNdfShare && (bx & 7) < f64_per8)
+      residual(NdfDouble{}, sums, L.sih2, L.ih2, L.e34ih2, K64.gamma);
+    else
+      residual(NdfSingle{}, sums, K.sih2, K.ih2, K.e34ih2, K.gamma);
     sums.finish(out);
   }
   if (threadIdx.x == 0) {
@@ -433,7 +443,7 @@ __device__ __forceinline__ bool norm_mixed_df_body(int bx, int nbx, const Level<
   return true;
 }
 
-template <int DIM, bool F64>
+template <int DIM, int MODE>
 __global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) k_norm_mixed_df(const __grid_constant__ Level<double> L,
                                                                  DfCoefs K, Coefs<double> K64, int f64_per8,
                                                                  const __grid_constant__ Level<float> G,
@@ -441,7 +451,7 @@ __global__ void __launch_bounds__(kNdfTX * kNdfTY, DIM == 3 ? 3 : 4) k_norm_mixe
                                                                  cudaGraphConditionalHandle cond, int mode,
                                                                  int use_cond) {
   pdl_enter();
-  norm_mixed_df_body<DIM, F64>(blockIdx.x, gridDim.x, L, K, K64, f64_per8, G, partials, st, cond, mode, use_cond);
+  norm_mixed_df_body<DIM, MODE>(blockIdx.x, gridDim.x, L, K, K64, f64_per8, G, partials, st, cond, mode, use_cond);
 }
 
 }  // namespace chhs_dev
