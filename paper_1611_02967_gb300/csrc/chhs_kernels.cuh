@@ -24,6 +24,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chhs_predict.cuh"
+
 namespace chhs_dev {
 
 constexpr int kBlock = 256;        // block size of the plain per-cell kernels
@@ -83,15 +85,16 @@ struct DevState {
   unsigned int ticket;  // blocks of the norm kernel that have finished
   unsigned int pad_;
   // V-cycles between two stopping norms (loop_decision): the iteration about
-  // to run does `inner` of them (1 .. max_inner); rho is the measured
-  // contraction per V-cycle, rprev the previous norm.
+  // to run does `inner` of them (1 .. max_inner); the last measured contraction
+  // is rnum / rden over `ran` V-cycles (0: none yet), rprev the previous norm.
   int inner;
   int go_more[3];  // go and inner >= 2 + q: the batched step's gates of the extra V-cycles
   int max_inner;   // 0 or 1: a norm after every V-cycle
   int checks;      // stopping norms after V-cycles in the current call
   int use_if;      // IF nodes of cond_if in the step graph (0 .. 3)
-  double rho;
+  double rnum, rden;
   double rprev;
+  int ran;
   cudaGraphConditionalHandle cond_if[3];  // IF node q: a (2 + q)-th V-cycle in the iteration
 };
 
@@ -1005,31 +1008,16 @@ __device__ __forceinline__ void sum_partials(const double* partials, int nparts,
 // step is converged when r <= tol and rmax <= tol_max.  Returns 1 while
 // another cycle is due.
 // V-cycles for the next iteration of the step's loop: the number the
-// measured contraction rho predicts the norms (r against tol, the pointwise
-// rmax against tol_max) still need, rounded to the nearest (a V-cycle past
-// the stopping point needs a contraction twice as strong, in log terms, as
-// the one measured over the iteration before; rounding down instead cost
-// ~0.8 more norms per step and no fewer V-cycles on the benchmark
-// workloads); at least 1, at most max_inner and the V-cycles left under
-// max_v.  Every stop is still decided by a norm of the iterate.
-//
-// The prediction runs in single precision, with log2 of a double taken from
-// its exponent and its leading significand bits: on one thread at the end of
-// a norm, FP64 log, pow and division (each a chain of FP64 instructions of
-// ~64 cycles) took ~8 us per norm, on the critical path of every iteration.
-__device__ __forceinline__ float log2_f64(double x) {  // x > 0, normal
-  const int hi = __double2hiint(x);
-  const float m = __uint_as_float(0x3F800000u | (((unsigned)hi & 0xFFFFFu) << 3) | ((unsigned)__double2loint(x) >> 29));
-  return (float)((hi >> 20) - 1023) + log2f(m);
-}
-
+// contraction measured over the last one predicts (chhs_predict.cuh), rounded
+// to the nearest (a V-cycle past the stopping point needs a contraction twice
+// as strong, in log terms, as the one measured over the iteration before;
+// rounding down instead cost ~0.8 more norms per step and no fewer V-cycles on
+// the benchmark workloads); at least 1, at most max_inner and the V-cycles left
+// under max_v.  Every stop is still decided by a norm of the iterate.
 __device__ __forceinline__ int next_inner(const DevState* st, double r, double rmax) {
   const int cap = min(st->max_inner, st->max_v - st->vcycles);
-  if (cap <= 1 || !(st->rho > 0.0 && st->rho < 1.0)) return 1;
-  const float lr = log2_f64(st->rho), lt = log2_f64(st->tol);
-  float need = r > st->tol ? (lt - log2_f64(r)) / lr : 0.f;
-  if (rmax > st->tol_max) need = fmaxf(need, (log2_f64(st->tol_max) - log2_f64(rmax)) / lr);
-  return max(1, min(cap, (int)floorf(need + 0.5f)));
+  if (st->ran == 0) return 1;
+  return predict_inner(r, rmax, st->tol, st->tol_max, st->rnum, st->rden, st->ran, cap);
 }
 
 __device__ __forceinline__ unsigned int loop_decision(DevState* st, double r, double rmax, int mode) {
@@ -1052,8 +1040,11 @@ __device__ __forceinline__ unsigned int loop_decision(DevState* st, double r, do
       // contraction per V-cycle over the iteration just finished (kept across
       // steps: the next step's first iteration starts from it)
       const bool finite = isfinite(r);
-      if (st->rprev > 0.0 && r > 0.0 && finite)
-        st->rho = (double)fminf(fmaxf(exp2f((log2_f64(r) - log2_f64(st->rprev)) / (float)ran), 1e-3f), 0.9f);
+      if (st->rprev > 0.0 && r > 0.0 && finite) {
+        st->rnum = r;
+        st->rden = st->rprev;
+        st->ran = ran;
+      }
       if (!finite || r > 1e8 * (st->r0 + 1.0)) {
         st->failed = 5;  // CHHS_ERR_DIVERGED
       } else if (above) {
