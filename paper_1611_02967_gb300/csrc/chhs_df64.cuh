@@ -117,6 +117,19 @@ DF_HD df64 df_split(double x) {
   return df64{hi, lo};
 }
 
+// The conversion (float)x with integer instructions wherever the result is a
+// normal single: rounded to nearest, ties to even, a carry out of the
+// significand raising the exponent (beyond the largest, to infinity).  Zeros,
+// subnormal results, infinities and NaNs take the conversion itself.
+DF_HD float f64_to_f32_rn(double x) {
+  const uint64_t b = df_bits(x);
+  const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
+  const int e = (int)((hw >> 20) & 0x7FFu) - 896;
+  if ((unsigned)(e - 1) >= 254u) return (float)x;
+  const uint32_t mag = (uint32_t)e << 23 | (hw & 0xFFFFFu) << 3 | lw >> 29;
+  return df_from_bits((hw & 0x80000000u) | (mag + (((lw & 0x1FFFFFFFu) + 0x0FFFFFFFu + (mag & 1u)) >> 29)));
+}
+
 // Knuth's two-sum: s + err = a + b exactly.
 DF_HD df64 df_two_sum(float a, float b) {
   const float s = df_fadd(a, b);

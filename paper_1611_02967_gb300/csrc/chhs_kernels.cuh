@@ -1272,18 +1272,6 @@ __global__ void __launch_bounds__(kBlock) k_setup_coef(Level<double> L, const do
 // restriction on the integer and single-precision pipes: ~18.
 // Measured, with the rest of the step unchanged: a 256^3 step 25.8 -> 22.9 ms,
 // three of 128^3 10.8 -> 10.0 ms, two of 2048^2 11.4 -> 10.4 ms.
-//
-// Double to single precision rounded to nearest with integer instructions
-// (ties away from zero), a conversion costing as much as an FP64 FMA;
-// magnitudes below the smallest normal single give 0, beyond its range
-// infinity.
-__device__ __forceinline__ float f64_to_f32_rn(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7FFu) - 896;
-  const unsigned mag = ((unsigned)e << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29) + ((lo >> 28) & 1u);
-  return __uint_as_float((hi & 0x80000000u) | (e <= 0 ? 0u : e >= 255 ? 0x7F800000u : mag));
-}
-
 template <int DIM>
 __device__ __forceinline__ void setup_mixed_body(int bx, const Level<double>& L, const double* phimm1, double eps2,
                                                  const DevState* st, const Level<float>& G, const Level<float>& Gn) {
