@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <type_traits>
 #include <utility>
@@ -249,6 +250,19 @@ chhs_status fail(chhs_t* r, chhs_status s, const std::string& msg) {
     if (e_ != cudaSuccess)                                                                \
       return fail(run, CHHS_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
+
+// Opts a kernel in to dyn bytes of dynamic shared memory.  The opt-in is per
+// kernel and process-wide: it is only ever raised, so that no handle lowers it
+// below what another handle's graph launches need, and under a lock, so that no
+// thread sets a smaller size than another has just set.
+cudaError_t raise_smem(const void* fn, size_t dyn) {
+  static std::mutex lock;
+  std::lock_guard<std::mutex> hold(lock);
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= dyn) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+}
 
 // Every kernel of the solver goes through here: counted while the graph is
 // captured, bracketed by events while profiling.
@@ -625,22 +639,14 @@ struct Enqueue {
       cudaFuncAttributes fa;
       return cudaFuncGetAttributes(&fa, fn) == cudaSuccess && dyn + fa.sharedSizeBytes <= (size_t)optin;
     };
-    // the opt-in is per kernel and process-wide: only ever raise it, so that no
-    // handle lowers it below what another handle's graph launches need
-    auto raise_to = [&](const void* fn, size_t dyn) -> cudaError_t {
-      cudaFuncAttributes fa;
-      cudaError_t e = cudaFuncGetAttributes(&fa, fn);
-      if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= dyn) return e;
-      return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    };
     const size_t smem = tail_bytes<T, CORR>(tail);
     const void* ktail = reinterpret_cast<const void*>(k_tail<T, DIM, CORR>);
     if (!fits(ktail, smem))
       return fail(run, CHHS_ERR_INVALID_ARG,
                   "the grid does not coarsen to a coarsest level small enough for the one-block solve");
-    CU(raise_to(ktail, smem));
+    CU(raise_smem(ktail, smem));
     if constexpr (recompute_coefs<T, CORR>()) {
-      if (tail3_fits(tail)) CU(raise_to(reinterpret_cast<const void*>(k_tail3), tail3_bytes(tail)));
+      if (tail3_fits(tail)) CU(raise_smem(reinterpret_cast<const void*>(k_tail3), tail3_bytes(tail)));
     }
     if constexpr (use_tiles<T>()) {
       // the accepted sweep counts: tiles with their halo in nine shared fields
@@ -1037,8 +1043,7 @@ void place_cluster(chhs_t* run) {
     for (int l = 0; l < tl.n; ++l) P.rows[l] = l < P.tail ? cluster_rows(nrows(l), P.blocks) : nrows(l);
     const size_t smem = cluster_smem_bytes(tl, P);
     if (smem + fa.sharedSizeBytes > (size_t)optin) continue;
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (raise_smem(fn, smem) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
@@ -2247,8 +2252,7 @@ struct BatchStep {
       BCU(cudaFuncGetAttributes(&fa, fn));
       if (dyn + fa.sharedSizeBytes > (size_t)optin)
         return bfail(b, CHHS_ERR_INVALID_ARG, "a run's coarse tail or tiles need more shared memory than a block has");
-      if ((size_t)fa.maxDynamicSharedSizeBytes < dyn)
-        BCU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+      BCU(raise_smem(fn, dyn));
       return CHHS_OK;
     };
     chhs_status st = raise_to(reinterpret_cast<const void*>(kb_tail<float, DIM, true>), tail_smem);
