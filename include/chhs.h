@@ -260,13 +260,12 @@ typedef struct {
 /* Autotuner of the handle's launch shapes and coarse sweep counts: tries
  * candidate settings (where the one-block tail starts; in double precision,
  * up to which level size the split update is used; in the 2D mixed form, the
- * tile block size and tile shape on levels of at least 512 x 256 cells, 32 x
- * 16, 32 x 32 or 64 x 16 cells, and on the smaller levels the same shape or
- * 16 x 8 cells on 256 threads; the
+ * tile shape on levels of at least 512 x 256 cells, 32 x 16, 32 x 32 or 64 x
+ * 16 cells, and on the smaller levels the same shape or 16 x 8 cells; the
  * sweeps on the levels below the finest: the options' nu1, nu2 or, when both
- * exceed 1, one each), times
- * trial_steps steps of the handle's own problem from its current state with
- * each, keeps the fastest and rebuilds the step graph with it.  The state is
+ * exceed 1, one each), times trial_steps steps of the handle's own problem from
+ * its current state with each (settings that give the same launches once),
+ * keeps the fastest and rebuilds the step graph with it.  The state is
  * restored after every trial and at the end, so the run continues exactly
  * where it was.  Candidates that fail (shared memory too small, a trial that
  * does not converge) are skipped.  Allocates a temporary copy of the state
@@ -488,12 +487,12 @@ chhs_status chhs_batch_set_tuning(chhs_batch_t* batch, const chhs_tuning* tuning
  * tail starts: levels of at most 256 / 1024 / 4096 cells in 2D, 64 / 512 /
  * 4096 in 3D; the sweeps below the finest level: the options' nu1, nu2 or,
  * when both exceed 1, one each; in 2D the large levels' tile shape, 32 x 16,
- * 32 x 32 or 64 x 16 cells), keeps the fastest and rebuilds the batch's
- * graph with it.  Every run's state is restored after each trial and at the
- * end.  Candidates that fail are skipped.  Allocates a temporary copy of
- * all states (4 doubles per cell).  out (nullable) receives the setting
- * (ms_per_step -1 if the fastest could not be rebuilt and the original was
- * kept).  Errors: CHHS_ERR_INVALID_ARG (NULL batch, trial_steps < 1),
+ * 32 x 32 or 64 x 16 cells; settings that give the same launches once), keeps
+ * the fastest and rebuilds the batch's graph with it.  Every run's state is
+ * restored after each trial and at the end.  Candidates that fail are skipped.
+ * Allocates a temporary copy of all states (4 doubles per cell).  out
+ * (nullable) receives the setting (ms_per_step -1 if the fastest could not be
+ * rebuilt and the original was kept).  Errors: CHHS_ERR_INVALID_ARG (NULL batch, trial_steps < 1),
  * CHHS_ERR_OOM, CHHS_ERR_CUDA.  The paper has no counterpart. */
 chhs_status chhs_batch_autotune(chhs_batch_t* batch, int trial_steps, chhs_tuning* out);
 

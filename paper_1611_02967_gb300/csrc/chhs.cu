@@ -20,6 +20,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <set>
 #include <string>
 #include <type_traits>
 #include <utility>
@@ -1072,14 +1073,46 @@ void place_cluster(chhs_t* run) {
 
 // The first level of the one-block tail: the coarsest, and every level above
 // it with at most tail_cells cells (up to kTailMaxLevels levels).
-void place_tail(chhs_t* run) {
+int first_tail_level(const chhs_t* run, int tail_cells) {
   const Layout& Lo = run->layout;
   const int nl = (int)Lo.shapes.size();
   auto cells = [&](int l) { return Lo.shapes[l].n[0] * Lo.shapes[l].n[1] * Lo.shapes[l].n[2]; };
-  run->tail_start = nl - 1;
-  while (run->tail_start > 0 && cells(run->tail_start - 1) <= run->tail_cells &&
-         nl - (run->tail_start - 1) <= kTailMaxLevels)
-    --run->tail_start;
+  int start = nl - 1;
+  while (start > 0 && cells(start - 1) <= tail_cells && nl - (start - 1) <= kTailMaxLevels) --start;
+  return start;
+}
+
+// What distinguishes the launches of the handle's step under one setting from
+// those under another (the autotuners time equal ones once): tile shapes of a
+// level of the 2D mixed form ...
+void tile_key(std::vector<int>& key, const Level<float>& L, int np1, int np2, int tw, int th) {
+  for (const auto& steps : {Enqueue<2>::tile_pre(L, np1, false), Enqueue<2>::tile_post(L, np1, np2, false, nullptr)})
+    for (const Enqueue<2>::TileStep& q : steps) {
+      const TileShape T = tile_shape(tw, th, q.npass, q.restrict_out);
+      key.insert(key.end(), {T.tw, T.th});
+    }
+}
+// ... and the whole of a handle's.
+std::vector<int> launch_key(const chhs_t* run) {
+  std::vector<int> key = {run->tail_start, run->cluster_start, run->cplan.blocks, run->nu1c, run->nu2c};
+  const bool mixed = run->opts.precision == 1;
+  for (int l = 0; l < (run->cluster_start >= 0 ? run->cluster_start : run->tail_start); ++l) {
+    if (mixed && run->dim == 2) {
+      const Level<float>& L = run->lev32[l];
+      const bool large = L.ncell >= kLargeTileCells;
+      tile_key(key, L, 2 * Enqueue<2>::nu_pre(run, l), 2 * Enqueue<2>::nu_post(run, l), large ? run->tile_w : run->stile_w,
+               large ? run->tile_h : run->stile_h);
+    } else if (!mixed && l > 0) {
+      const Level<double>& L = run->lev[l];
+      key.push_back(((L.nx + 1) / 2) * L.ny * L.nz <= run->split_threads);
+      key.push_back(L.ncell <= 2 * run->split_threads);
+    }
+  }
+  return key;
+}
+
+void place_tail(chhs_t* run) {
+  run->tail_start = first_tail_level(run, run->tail_cells);
   fill_tail(run->tail, run->lev, run->tail_start, run->opts, run->nu1c, run->nu2c);
   fill_tail(run->tail32, run->lev32, run->tail_start, run->opts, run->nu1c, run->nu2c);
   run->cluster_start = -1;
@@ -1626,7 +1659,8 @@ chhs_status chhs_autotune(chhs_t* run, int trial_steps, chhs_tuning* out) {
   std::vector<std::pair<int, int>> coarse = {{run->opts.nu1, run->opts.nu2}};
   if (run->opts.nu1 > 1 && run->opts.nu2 > 1) coarse.push_back({1, 1});
   // 2D mixed form: tile shapes (interior cells; wider tiles recompute a
-  // smaller share of halo cells but make fewer blocks) and block sizes
+  // smaller share of halo cells but make fewer blocks) and the block sizes that
+  // go with them, which change no launch
   struct Shape2 {
     int tt, tw, th;
   };
@@ -1694,7 +1728,11 @@ chhs_status chhs_autotune(chhs_t* run, int trial_steps, chhs_tuning* out) {
   Cand best = orig;
   float best_ms = -1.f;
   chhs_status s;
+  std::set<std::vector<int>> seen;
   for (const Cand& c : cands) {
+    take_tuning(run, c);
+    place_tail(run);
+    if (!seen.insert(launch_key(run)).second) continue;  // the launches of a candidate before
     if (apply(c) != CHHS_OK) continue;  // e.g. a tail too large for shared memory
     if ((s = restore()) != CHHS_OK) return s;
     if (chhs_step(run, 1, nullptr, nullptr) != CHHS_OK) continue;  // warm-up
@@ -2691,8 +2729,20 @@ chhs_status chhs_batch_autotune(chhs_batch_t* b, int trial_steps, chhs_tuning* o
   Cand best = orig;
   if (!copy_states(true) || cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     s = CHHS_ERR_CUDA;
+  std::set<std::vector<int>> seen;
+  auto key_of = [&](const Cand& c) {
+    std::vector<int> key = {c.n1, c.n2};
+    for (const chhs_t* r : b->runs) {
+      const int start = first_tail_level(r, c.tc);
+      key.push_back(start);
+      for (int l = 0; b->dim == 2 && l < start && r->lev32[l].ncell >= BatchStep<2>::kSoloTileCells; ++l)
+        tile_key(key, r->lev32[l], 2 * (l == 0 ? b->opts.nu1 : c.n1), 2 * (l == 0 ? b->opts.nu2 : c.n2), c.tw, c.th);
+    }
+    return key;
+  };
   for (size_t q = 0; s == CHHS_OK && q < cands.size(); ++q) {
     const Cand& c = cands[q];
+    if (!seen.insert(key_of(c)).second) continue;  // the launches of a candidate before
     if (batch_apply(b, c.tc, c.n1, c.n2, r0->norm_f64_per8, c.tw, c.th, c.tt) != CHHS_OK) continue;  // e.g. a tail too big
     // one untimed step (the new graph's first launch), then the timed ones,
     // each from the saved state
