@@ -361,28 +361,23 @@ struct Enqueue {
   static int nu_pre(const chhs_t* run, int l) { return l == 0 ? run->opts.nu1 : run->nu1c; }
   static int nu_post(const chhs_t* run, int l) { return l == 0 ? run->opts.nu2 : run->nu2c; }
 
-  // sweeps red-black sweeps; with rhs the first one also completes the FAS
-  // right-hand side of this (coarse) level.
-  template <typename T, bool CORR>
-  static void smooth(chhs_t* run, cudaStream_t s, const Level<T>& L, int sweeps, bool rhs) {
-    const Coefs<T> K = coefs<T>(run);
+  // sweeps red-black sweeps in double precision; with rhs the first one also
+  // completes the FAS right-hand side of this (coarse) level.
+  static void smooth(chhs_t* run, cudaStream_t s, const Level<double>& L, int sweeps, bool rhs) {
+    const Coefs<double> K = coefs<double>(run);
     const int threads = ((L.nx + 1) / 2) * L.ny * L.nz;
     const int blocks = (threads + kSmoothBlock - 1) / kSmoothBlock;
-    // small double-precision levels: each cell's update split over three warps
-    const bool split = std::is_same<T, double>::value && !CORR && threads <= run->split_threads &&
-                       L.ncell != run->ncell();
+    // small levels: each cell's update split over three warps
+    const bool split = threads <= run->split_threads && L.ncell != run->ncell();
     for (int it = 0; it < sweeps; ++it)
       for (int colour = 0; colour < 2; ++colour) {
         const int with_rhs = (rhs && it == 0) ? 1 : 0;
         const int kind = L.ncell == run->ncell() ? CHHS_K_SMOOTH_FINEST : CHHS_K_SMOOTH;
         launch(run, s, kind, colour_cells(L, colour), [&] {
-          if constexpr (std::is_same<T, double>::value && !CORR) {
-            if (split) {
-              pdl(k_smooth_split<DIM>, (threads + 31) / 32, 96, s, L, K, colour, with_rhs);
-              return;
-            }
-          }
-          pdl(k_smooth<T, DIM, CORR>, blocks, kSmoothBlock, s, L, K, colour, with_rhs);
+          if (split)
+            pdl(k_smooth_split<DIM>, (threads + 31) / 32, 96, s, L, K, colour, with_rhs);
+          else
+            pdl(k_smooth<double, DIM, false>, blocks, kSmoothBlock, s, L, K, colour, with_rhs);
         });
       }
   }
@@ -499,32 +494,31 @@ struct Enqueue {
       // the finished correction of the finest level goes straight into u
       tiles(tile_post(L, np1, np2, rhs, l == 0 && fused_update(run) && run->vc_update ? &run->lev[0] : nullptr));
       return;
-    }
-    if (rhs && nu_pre(run, l) == 0)
-      launch(run, s, CHHS_K_COARSE_RHS, L.ncell, [&] {
-        pdl(k_coarse_rhs<T, DIM, CORR>, nblocks(L.ncell), kBlock, s, L, K);
-      });
-    if constexpr (recompute_coefs<T, CORR>()) {
-      corr_vcycle_level(run, s, lev, tail, l);
-      return;
-    }
-    smooth<T, CORR>(run, s, L, nu_pre(run, l), rhs && nu_pre(run, l) > 0);
-    launch(run, s, CHHS_K_RESTRICT, L.ncell, [&] {
-      if constexpr (std::is_same<T, double>::value && !CORR) {
-        if (L.ncell <= 2 * run->split_threads && l > 0) {  // small level: the three rows on three warps
-          constexpr int TX = DIM == 3 ? 8 : 16;
-          const long long tiles = (long long)((L.nx + TX - 1) / TX) * (L.ny / 2) * (DIM == 3 ? L.nz / 2 : 1);
-          pdl(k_residual_restrict_split<DIM>, (int)tiles, 96, s, L, C, K);
-          return;
-        }
-        pdl(k_residual_restrict64<DIM>, (C.ncell + kSetupBlock - 1) / kSetupBlock, kSetupBlock, s, L, C, K);
+    } else {
+      if (rhs && nu_pre(run, l) == 0)
+        launch(run, s, CHHS_K_COARSE_RHS, L.ncell, [&] {
+          pdl(k_coarse_rhs<T, DIM, CORR>, nblocks(L.ncell), kBlock, s, L, K);
+        });
+      if constexpr (recompute_coefs<T, CORR>()) {
+        corr_vcycle_level(run, s, lev, tail, l);
+      } else {  // double precision
+        smooth(run, s, L, nu_pre(run, l), rhs && nu_pre(run, l) > 0);
+        launch(run, s, CHHS_K_RESTRICT, L.ncell, [&] {
+          if (L.ncell <= 2 * run->split_threads && l > 0) {  // small level: the three rows on three warps
+            constexpr int TX = DIM == 3 ? 8 : 16;
+            const long long tiles = (long long)((L.nx + TX - 1) / TX) * (L.ny / 2) * (DIM == 3 ? L.nz / 2 : 1);
+            pdl(k_residual_restrict_split<DIM>, (int)tiles, 96, s, L, C, K);
+            return;
+          }
+          pdl(k_residual_restrict64<DIM>, (C.ncell + kSetupBlock - 1) / kSetupBlock, kSetupBlock, s, L, C, K);
+        });
+        vcycle<T, CORR>(run, s, lev, tail, l + 1);
+        launch(run, s, CHHS_K_PROLONG, L.ncell, [&] {
+          pdl(k_prolong<T, DIM>, nblocks(C.ncell), kBlock, s, L, C);
+        });
+        smooth(run, s, L, nu_post(run, l), false);
       }
-    });
-    vcycle<T, CORR>(run, s, lev, tail, l + 1);
-    launch(run, s, CHHS_K_PROLONG, L.ncell, [&] {
-      pdl(k_prolong<T, DIM>, nblocks(C.ncell), kBlock, s, L, C);
-    });
-    smooth<T, CORR>(run, s, L, nu_post(run, l), false);
+    }
   }
 
   // 3D single-precision (correction-form) levels above the tail: colour

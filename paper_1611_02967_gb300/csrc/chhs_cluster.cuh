@@ -10,7 +10,7 @@
 // (~570 cycles measured at 512 threads) takes the launch's place.
 //
 // Slabs: level l gives every block R_l = 2 ceil(rows / (2 blocks)) rows, an
-// even number starting at an even row, so that the 2^d children of a coarse
+// even number starting at an even row, so that the four children of a coarse
 // cell lie in one block; small levels leave blocks idle.  A block keeps one
 // halo row below and above its slab; a pass stores the updated cells of its
 // first and last row into the neighbours' halos as well, so all stencil reads
