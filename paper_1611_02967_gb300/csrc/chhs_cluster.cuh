@@ -21,10 +21,12 @@
 // held by block 0 whole and run there as in k_tail, the others waiting at the
 // barrier.
 //
-// Measured (GB300, default tuning): a 64 x 64 step of 6.6 V-cycles, all of it
-// in the cluster, 847 us with a launch per pass -> 646 us; 512 x 512, where the
-// levels 64 x 64 ... 16 x 16 move here, 2.31 -> 2.22 ms with the cells of a level
-// in registers (cluster_passes) against one update per launch-like pass.
+// Measured (GB300, default tuning, both sides in turn): with a launch per pass
+// against the cluster with one update per launch-like pass, a 64 x 64 step of
+// 6.6 V-cycles, all of it in the cluster, 840 -> 734 us, and a 512 x 512 step,
+// where the levels 64 x 64 ... 16 x 16 move here, 2.53 -> 2.48 ms; that against
+// the cells of a level in registers (cluster_passes), the outer-flux restriction
+// and the asynchronous copies 700 -> 655 us and 2.34 -> 2.29 ms.
 #pragma once
 #include <cooperative_groups.h>
 
